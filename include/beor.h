@@ -74,9 +74,10 @@ enum { BEOR_PREC_FP64 = 0, BEOR_PREC_MIXED = 1 };
  * precision = BEOR_PREC_MIXED: trailing and panel updates of the blocked
  *   Cholesky run as exact bf16 slice products on the tensor cores with fp32
  *   accumulation, the working matrix is kept as a pair of fp32 words per
- *   real number, the diagonal-block Cholesky factorisations and the
- *   log-determinants are float64 (the blocks' inverses are formed on the
- *   fp32 pipe to ~2^-48), and a float64-accurate residual against the
+ *   real number, the diagonal-block Cholesky factorisations are float64
+ *   (posterior mean) or 64-bit fixed point with at least its accuracy (lnL),
+ *   the log-determinants float64 (the blocks' inverses are formed to ~2^-48),
+ *   and a float64-accurate residual against the
  *   float64 precompute corrects the quadratic form (lnL) or refines the
  *   solution (posterior mean). */
 int beor_create(beor_ctx **out, int device, int precision);
@@ -275,9 +276,9 @@ int beor_set_lookahead(int on);
  *               so that all end on the last block step (their light final
  *               steps overlap); 0 = all start on step 0.
  *   reserve_diag: 1 = each launch for columns j >= k + 2 also leaves free as
- *               many SMs as step k + 1 has diagonal blocks (one CTA per
- *               problem, running beside it at high priority), so that they
- *               start at once; 0 = no such reserve. */
+ *               many SMs as step k + 1's diagonal blocks take (one, two or
+ *               four CTAs per problem, running beside it at high priority), so
+ *               that they start at once; 0 = no such reserve. */
 typedef struct {
   int lookahead;
   int rest_ctas;

@@ -218,6 +218,12 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
   L += 2;
   RUN(KC_INIT, launch_copy_dbar(v, s));
   L += 1;
+  // problems that take block step k
+  auto active = [&](int k) {
+    int n = 0;
+    for (const Prob& pr : pl.h_prob) n += k >= pr.k_off && k - pr.k_off < pr.nt;
+    return n;
+  };
   const bool la = pl.mixed && pl.lookahead;
   if (la) {
     // Look-ahead schedule of the mixed factorisation (three streams):
@@ -236,7 +242,7 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
       if (x == cudaSuccess) x = cudaStreamWaitEvent(pl.side2, pl.ev_diag, 0);
       return x;
     };
-    RUN(KC_DIAG, launch_diag(v, 0, true, s, hi));
+    RUN(KC_DIAG, launch_diag(v, 0, true, active(0), s, hi));
     L += 1;
     if ((e = fwd_after_diag()) != cudaSuccess) return e;
     RUN_ON(KC_SOLVE, pl.side2, launch_fwd_step(v, true, v.vec_b, -1, pl.side2));
@@ -252,7 +258,7 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
       L += trail_launch_count(pl.maps, k, TRAIL_NEXT_COL);
       if ((e = cudaEventRecord(pl.ev_col, s)) != cudaSuccess) return e;
       if ((e = cudaStreamWaitEvent(pl.side, pl.ev_col, 0)) != cudaSuccess) return e;
-      RUN(KC_DIAG, launch_diag(v, k + 1, true, s, hi));
+      RUN(KC_DIAG, launch_diag(v, k + 1, true, active(k + 1), s, hi));
       L += 1;
       if ((e = fwd_after_diag()) != cudaSuccess) return e;
       RUN_ON(KC_SOLVE, pl.side2, launch_fwd_step(v, true, v.vec_b, k, pl.side2));
@@ -261,14 +267,7 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
         // reserve_diag: leave free the SMs that step k + 1's diagonal blocks
         // (one CTA each, running beside this launch) need
         int cap = 0;
-        if (pl.sch.reserve_diag) {
-          int active = 0;
-          for (const Prob& pr : pl.h_prob) {
-            const int kp = k + 1 - pr.k_off;
-            active += kp >= 0 && kp < pr.nt && pr.n > 0;
-          }
-          cap = std::max(8, device_sms() - active);
-        }
+        if (pl.sch.reserve_diag) cap = std::max(8, device_sms() - diag_tc_ctas(active(k + 1)));
         RUN_ON(KC_TRAIL, pl.side, launch_trail_mixed(v, pl.maps, k, TRAIL_REST, pl.side, 0, cap));
         L += trail_launch_count(pl.maps, k, TRAIL_REST);
       }
@@ -285,7 +284,7 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
     if ((e = cudaStreamWaitEvent(s, pl.ev_fwd, 0)) != cudaSuccess) return e;
   } else {
     for (int k = 0; k < pl.max_nt; ++k) {
-      RUN(KC_DIAG, launch_diag(v, k, pl.mixed, s));
+      RUN(KC_DIAG, launch_diag(v, k, pl.mixed, active(k), s));
       L += 1;
       if (k + 1 < pl.max_nt) {
         if (pl.mixed) {
@@ -490,6 +489,7 @@ int build_plan(beor_ctx* const* ctxs, int nsets, const int* Bs, bool need_x, int
   v.dinv_elems = dinv_elems;
   v.grid_rest = pl->sch.rest_ctas;
   v.grid_col = pl->sch.col_ctas;
+  v.mean = need_x ? 1 : 0;
   if (pl->mixed) {
     chk(mixed_maps_create(v, &pl->maps));
     int lo = 0, hi = 0;

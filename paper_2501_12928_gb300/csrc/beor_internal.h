@@ -34,7 +34,8 @@ struct BatchView {
   int max_nt;
   // workspaces
   void* ws;                  // packed tiles of every problem (double2 or float4)
-  double2* dinv;             // inverse diagonal blocks, packed lower 128x128 per block
+  double2* dinv;             // inverse diagonal blocks, packed lower 128x128 per block (lnL on the mixed
+                             // path: float4 double-float elements in the same place)
   double* phi_inv;           // [rows] prior inverse per problem row (padded rows = 1)
   double2* vec_b;            // [rows] right-hand side / residual
   double2* vec_y;            // [rows] forward-solve result
@@ -70,29 +71,48 @@ struct BatchView {
   // schedule: CTAs of the trailing launches for columns j >= k + 2 and of the
   // next-column / panel launches (0: one per SM)
   int grid_rest, grid_col;
+  int mean;                  // posterior mean: the solution itself is refined
 };
 
-// Launch with an explicit scheduling priority (0: the stream's own); the
-// attribute is kept by stream capture, so graph nodes carry it too.
+// Launch with an explicit scheduling priority (0: the stream's own) and
+// cluster size; the attributes are kept by stream capture, so graph nodes carry
+// them too.
 template <typename... Exp, typename... Act>
-static cudaError_t launch_prio(void (*kern)(Exp...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int prio,
-                               Act&&... args) {
+static cudaError_t launch_cluster(void (*kern)(Exp...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int prio,
+                                  int cluster, Act&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributePriority;
-  at[0].val.priority = prio;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (prio != 0) {
+    at[n].id = cudaLaunchAttributePriority;
+    at[n++].val.priority = prio;
+  }
+  if (cluster > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = cluster;
+    at[n].val.clusterDim.y = 1;
+    at[n++].val.clusterDim.z = 1;
+  }
   cfg.attrs = at;
-  cfg.numAttrs = prio != 0 ? 1 : 0;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Act>(args)...);
+}
+template <typename... Exp, typename... Act>
+static cudaError_t launch_prio(void (*kern)(Exp...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int prio,
+                               Act&&... args) {
+  return launch_cluster(kern, grid, block, smem, s, prio, 1, std::forward<Act>(args)...);
 }
 
 // chol.cu (both precisions)
 cudaError_t launch_prior_init(const BatchView& v, bool mixed, cudaStream_t s);
-cudaError_t launch_diag(const BatchView& v, int k, bool mixed, cudaStream_t s, int prio = 0);
+cudaError_t launch_diag(const BatchView& v, int k, bool mixed, int active, cudaStream_t s, int prio = 0);
+// diag_tc.cu: the mixed path's diagonal blocks of step k, of `active` problems
+cudaError_t launch_diag_tc(const BatchView& v, int k, int active, cudaStream_t s, int prio);
+int diag_tc_ctas(int active);   // CTAs of its launch
 cudaError_t launch_panel_f64(const BatchView& v, int k, cudaStream_t s);
 cudaError_t launch_trail_f64(const BatchView& v, int k, cudaStream_t s);
 cudaError_t launch_solve(const BatchView& v, bool mixed, const double2* rhs, double2* out, cudaStream_t s);

@@ -13,6 +13,7 @@
 //  * lnl:           q = Re(dbar^H abar), or its residual-corrected form, and lnL.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "beor_common.cuh"
 #include "beor_internal.h"
@@ -494,7 +495,13 @@ __global__ void __launch_bounds__(512) diag_kernel(BatchView v, int kg, int mixe
   }
 }
 
-cudaError_t launch_diag(const BatchView& v, int k, bool mixed, cudaStream_t s, int prio) {
+// Mixed plans of lnL factor their diagonal blocks in diag_tc.cu.  The
+// posterior mean keeps this kernel: its amplitudes are Sigma^-1 times the
+// float64-accurate residual's rounding (relative 5e-8 at kappa ~ 1e8, 3280
+// modes), so that any other rounding of the factor moves them by as much,
+// while the quadratic form of lnL does not see it (1e-10).
+cudaError_t launch_diag(const BatchView& v, int k, bool mixed, int active, cudaStream_t s, int prio) {
+  if (mixed && !v.mean) return launch_diag_tc(v, k, active, s, prio);
   // packed block, one column, and (mixed) the third float terms of L
   const size_t smem = sizeof(double2) * (DG_PACK + BEOR_TB) + sizeof(float2) * DG_PACK;
   static bool init = false;
@@ -718,36 +725,89 @@ __device__ __forceinline__ void cacc_reduce8(CAcc& a, const float4*) {
   }
 }
 
-// y_blk = Linv (or Linv^H when herm) * r_blk, float64; 128 threads of the CTA
-__device__ __forceinline__ void diag_apply(const double2* __restrict__ li, const double2* rk, double2* out,
-                                           bool herm) {
+// The inverse diagonal block times a block of the right-hand side, y = Linv rk
+// or (herm) Linv^H rk, into out; 256 threads.  Float64 blocks (the float64 path
+// and the posterior mean): one thread per row, the loads unrolled ahead of the
+// chain of float64 products.
+__device__ __forceinline__ void diag_apply(const double2* __restrict__ li, const double2* rk, const dfl*, const dfl*,
+                                           CAcc*, double2* out, bool herm) {
   const int t = threadIdx.x;
   if (t >= BEOR_TB) return;
   double sr = 0.0, si = 0.0;
-  if (!herm) {
-    for (int m = 0; m <= t; ++m) {
-      const double2 a = li[pk(t, m)], q = rk[m];
-      sr = fma(a.x, q.x, fma(-a.y, q.y, sr));
-      si = fma(a.x, q.y, fma(a.y, q.x, si));
+  const int m0 = herm ? t : 0, m1 = herm ? BEOR_TB - 1 : t;
+  constexpr int U = 8;
+  double2 a[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) a[u] = li[herm ? pk(min(m0 + u, m1), t) : pk(t, min(m0 + u, m1))];
+  for (int m = m0; m <= m1; m += U) {
+    double2 n[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) n[u] = li[herm ? pk(min(m + U + u, m1), t) : pk(t, min(m + U + u, m1))];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (m + u > m1) break;
+      const double2 q = rk[m + u];
+      const double ai = herm ? -a[u].y : a[u].y;
+      sr = fma(a[u].x, q.x, fma(-ai, q.y, sr));
+      si = fma(a[u].x, q.y, fma(ai, q.x, si));
     }
-  } else {
-    for (int m = t; m < BEOR_TB; ++m) {
-      const double2 a = li[pk(m, t)], q = rk[m];
-      sr = fma(a.x, q.x, fma(a.y, q.y, sr));
-      si = fma(a.x, q.y, fma(-a.y, q.x, si));
-    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) a[u] = n[u];
   }
   out[t] = make_double2(sr, si);
+}
+// Double-float blocks (lnL on the mixed path): compensated products on the fp32
+// pipe, as for the off-diagonal tiles.  33,000 float64 products of one block
+// take 10 us on one SM, and as a chain per row with uncoalesced loads they took
+// 40 us of a step; eight lanes per row (forward) or two threads per column
+// (backward) read the block coalesced.
+__device__ __forceinline__ void diag_apply(const float4* __restrict__ li, const double2*, const dfl* rkr,
+                                           const dfl* rki, CAcc* part, double2* out, bool herm) {
+  const int tid = threadIdx.x;
+  if (!herm) {
+    const int lane8 = tid & 7;
+    for (int t = tid >> 3; t < BEOR_TB; t += 32) {
+      CAcc a;
+      cacc_zero(a);
+#pragma unroll 4
+      for (int m = lane8; m <= t; m += 8)
+        cacc_mac(a, li + pk(t, m), make_double2(0.0, 0.0), rkr[m], rki[m], false);
+      cacc_reduce8(a, li);
+      if (lane8 == 0) out[t] = cacc_get(a, li);
+    }
+  } else {
+    const int t = tid & 127, half = tid >> 7;
+    CAcc a;
+    cacc_zero(a);
+#pragma unroll 4
+    for (int m = t + half; m < BEOR_TB; m += 2)
+      cacc_mac(a, li + pk(m, t), make_double2(0.0, 0.0), rkr[m], rki[m], true);
+    if (half) part[t] = a;
+    __syncthreads();
+    if (!half) {
+      cacc_add(a, part[t]);
+      out[t] = cacc_get(a, li);
+    }
+  }
 }
 
 // Forward step k (k = -1: only y_0).  CTA (i, p), i = k+1 .. nt-1:
 // r_i -= L_ik y_k; the CTA with i == k+1 then sets y_{k+1} = Linv r_{k+1}.
-template <typename WS>
+// DV: element type of the inverse diagonal blocks.
+template <typename WS, typename DV>
 __global__ void __launch_bounds__(256) fwd_step_kernel(BatchView v, int kg, const double2* __restrict__ rhs) {
   __shared__ double2 yk[BEOR_TB];
   __shared__ dfl ykr[BEOR_TB], yki[BEOR_TB];
   __shared__ CAcc part[BEOR_TB];
   __shared__ double2 rk[BEOR_TB];
+  __shared__ dfl rkr[BEOR_TB], rki[BEOR_TB];
+  auto set_rk = [&](int t, double2 q) {
+    rk[t] = q;
+    if (std::is_same<DV, float4>::value) {
+      rkr[t] = df_from_double(q.x);
+      rki[t] = df_from_double(q.y);
+    }
+  };
   const int p = blockIdx.y;
   const Prob pr = v.prob[p];
   const int k = kg - pr.k_off;   // this problem's step (-1: start)
@@ -765,9 +825,9 @@ __global__ void __launch_bounds__(256) fwd_step_kernel(BatchView v, int kg, cons
     if (tid < BEOR_TB) r[i * BEOR_TB + tid] = rhs[pr.row_off + i * BEOR_TB + tid];
     if (i != 0) return;
     __syncthreads();
-    if (tid < BEOR_TB) rk[tid] = r[tid];
+    if (tid < BEOR_TB) set_rk(tid, r[tid]);
     __syncthreads();
-    diag_apply(v.dinv + pr.dinv_off, rk, yk, false);
+    diag_apply(reinterpret_cast<const DV*>(v.dinv) + pr.dinv_off, rk, rkr, rki, part, yk, false);
     __syncthreads();
     if (tid < BEOR_TB) y[tid] = yk[tid];
     return;
@@ -795,11 +855,11 @@ __global__ void __launch_bounds__(256) fwd_step_kernel(BatchView v, int kg, cons
     cur.x -= s.x;
     cur.y -= s.y;
     r[i * BEOR_TB + row] = cur;
-    rk[row] = cur;
+    if (i == k + 1) set_rk(row, cur);
   }
   if (i != k + 1) return;
   __syncthreads();
-  diag_apply(v.dinv + pr.dinv_off + (int64_t)i * DG_PACK, rk, yk, false);
+  diag_apply(reinterpret_cast<const DV*>(v.dinv) + pr.dinv_off + (int64_t)i * DG_PACK, rk, rkr, rki, part, yk, false);
   __syncthreads();
   if (tid < BEOR_TB) y[i * BEOR_TB + tid] = yk[tid];
 }
@@ -808,11 +868,20 @@ __global__ void __launch_bounds__(256) fwd_step_kernel(BatchView v, int kg, cons
 // i = 0 .. k-1: r_i -= L_ki^H x_k; the CTA with i == k-1 then sets
 // x_{k-1} = Linv^H r_{k-1}.  Steps run from the largest nt down; problems
 // with fewer tiles join when k < their nt.
-template <typename WS>
+template <typename WS, typename DV>
 __global__ void __launch_bounds__(256) bwd_step_kernel(BatchView v, int k, double2* __restrict__ out) {
   __shared__ double2 xk[BEOR_TB];
   __shared__ dfl xkr[BEOR_TB], xki[BEOR_TB];
   __shared__ double2 rk[BEOR_TB];
+  __shared__ dfl rkr[BEOR_TB], rki[BEOR_TB];
+  __shared__ CAcc part[BEOR_TB];
+  auto set_rk = [&](int t, double2 q) {
+    rk[t] = q;
+    if (std::is_same<DV, float4>::value) {
+      rkr[t] = df_from_double(q.x);
+      rki[t] = df_from_double(q.y);
+    }
+  };
   const int p = blockIdx.y;
   const Prob pr = v.prob[p];
   if (prob_skipped(v.status[p])) return;
@@ -828,9 +897,9 @@ __global__ void __launch_bounds__(256) bwd_step_kernel(BatchView v, int k, doubl
     if (tid < BEOR_TB) r[i * BEOR_TB + tid] = y[i * BEOR_TB + tid];
     if (k != pr.nt || i != pr.nt - 1) return;
     __syncthreads();
-    if (tid < BEOR_TB) rk[tid] = r[i * BEOR_TB + tid];
+    if (tid < BEOR_TB) set_rk(tid, r[i * BEOR_TB + tid]);
     __syncthreads();
-    diag_apply(v.dinv + pr.dinv_off + (int64_t)i * DG_PACK, rk, xk, true);
+    diag_apply(reinterpret_cast<const DV*>(v.dinv) + pr.dinv_off + (int64_t)i * DG_PACK, rk, rkr, rki, part, xk, true);
     __syncthreads();
     if (tid < BEOR_TB) x[i * BEOR_TB + tid] = xk[tid];
     return;
@@ -867,12 +936,12 @@ __global__ void __launch_bounds__(256) bwd_step_kernel(BatchView v, int k, doubl
       cur.x -= sv.x;
       cur.y -= sv.y;
       r[i * BEOR_TB + c] = cur;
-      rk[c] = cur;
+      if (i == k - 1) set_rk(c, cur);
     }
   }
   if (i != k - 1) return;
   __syncthreads();
-  diag_apply(v.dinv + pr.dinv_off + (int64_t)i * DG_PACK, rk, xk, true);
+  diag_apply(reinterpret_cast<const DV*>(v.dinv) + pr.dinv_off + (int64_t)i * DG_PACK, rk, rkr, rki, part, xk, true);
   __syncthreads();
   if (tid < BEOR_TB) x[i * BEOR_TB + tid] = xk[tid];
 }
@@ -882,24 +951,26 @@ __global__ void __launch_bounds__(256) bwd_step_kernel(BatchView v, int k, doubl
 cudaError_t launch_fwd_step(const BatchView& v, bool mixed, const double2* rhs, int k, cudaStream_t s, int prio) {
   const int nb = k < 0 ? v.max_nt : v.max_nt - k - 1;
   if (nb <= 0) return cudaSuccess;
-  if (mixed) return launch_prio(fwd_step_kernel<float4>, dim3(nb, v.P), dim3(256), 0, s, prio, v, k, rhs);
-  return launch_prio(fwd_step_kernel<double2>, dim3(nb, v.P), dim3(256), 0, s, prio, v, k, rhs);
+  auto kern = !mixed ? fwd_step_kernel<double2, double2>
+                     : v.mean ? fwd_step_kernel<float4, double2> : fwd_step_kernel<float4, float4>;
+  return launch_prio(kern, dim3(nb, v.P), dim3(256), 0, s, prio, v, k, rhs);
 }
 
 // out = L^-H y (y in vec_y), every problem.
-template <typename WS>
+template <typename WS, typename DV>
 static cudaError_t bwd_impl(const BatchView& v, double2* out, cudaStream_t s) {
   const int nt = v.max_nt;
-  bwd_step_kernel<WS><<<dim3(nt, v.P), 256, 0, s>>>(v, nt, out);
+  bwd_step_kernel<WS, DV><<<dim3(nt, v.P), 256, 0, s>>>(v, nt, out);
   for (int k = nt - 1; k >= 1; --k) {
     // problems whose last block is k-1 (nt_p == k) start here
-    bwd_step_kernel<WS><<<dim3(k, v.P), 256, 0, s>>>(v, k, out);
+    bwd_step_kernel<WS, DV><<<dim3(k, v.P), 256, 0, s>>>(v, k, out);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_bwd(const BatchView& v, bool mixed, double2* out, cudaStream_t s) {
-  return mixed ? bwd_impl<float4>(v, out, s) : bwd_impl<double2>(v, out, s);
+  if (!mixed) return bwd_impl<double2, double2>(v, out, s);
+  return v.mean ? bwd_impl<float4, double2>(v, out, s) : bwd_impl<float4, float4>(v, out, s);
 }
 
 cudaError_t launch_solve_fwd(const BatchView& v, bool mixed, const double2* rhs, cudaStream_t s) {
