@@ -116,8 +116,8 @@ struct Plan {
   std::vector<SetDesc> h_sets;
   std::vector<int> first;   // first problem index of each set
   DevBuf d_prob, d_sets, ws, dinv, phi_inv, vecs, scal, flags, phis, panel_sl, panel_exp, linv_sl, linv_exp;
-  DevBuf xtr, rwork;                // float32-pipe residual: x triples, work items
-  int n_rwork = 0;
+  DevBuf xtr, rwork, rpart;         // float32-pipe residual: x triples, work items, partial sums
+  int n_rwork = 0, rcols = 0, rgroup = 0;
   std::vector<int64_t> phi_off;
   BatchView view{};
   MixedMaps* maps = nullptr;
@@ -315,14 +315,14 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
       RUN(KC_REFINE, launch_residual(v, s));
       RUN(KC_SOLVE, launch_solve(v, true, v.vec_r, v.vec_d, s));
       RUN(KC_REFINE, launch_refine_update(v, s));
-      L += 5 + solve_launch_count(pl.max_nt);
+      L += 4 + solve_launch_count(pl.max_nt);
     }
   } else if (corr) {
     // lnL only: one float64 residual r = dbar - Sigma x~ and y = L~^-1 r
     // correct the quadratic form (see lnl_kernel)
     RUN(KC_REFINE, launch_residual(v, s));
     RUN(KC_SOLVE, launch_solve_fwd(v, true, v.vec_r, s));
-    L += 4 + pl.max_nt;
+    L += 3 + pl.max_nt;
   }
   RUN(KC_LNL, launch_lnl(v, s, corr ? 1 : 0));
   L += 1;
@@ -432,15 +432,34 @@ int build_plan(beor_ctx* const* ctxs, int nsets, const int* Bs, bool need_x, int
     chk(pl->linv_sl.alloc(sizeof(__nv_bfloat16) * (size_t)BEOR_NPLANE * pl->P * BEOR_TB * BEOR_TB));
     chk(pl->linv_exp.alloc(sizeof(int32_t) * (size_t)pl->P * BEOR_TB));
     chk(pl->xtr.alloc(sizeof(float) * 6 * (size_t)rows));
-    // residual work items: row block x 16 block columns x 16 problems
+    // residual work items: row block x T block columns x up to 16 problems, T =
+    // 16 if that gives every SM several CTAs, else 4 or 1 (one problem alone:
+    // two tiles per item, one per half CTA)
     std::vector<RWork> wk;
+    const int64_t want = 6 * (int64_t)device_sms();
+    auto items = [&](int T) {
+      int64_t n = 0;
+      for (int s = 0; s < nsets; ++s) n += (int64_t)ctxs[s]->nt * ((ctxs[s]->nt + T - 1) / T) * ((Bs[s] + 15) / 16);
+      return n;
+    };
+    const int T = items(16) >= want && !need_x ? 16 : items(4) >= want && !need_x ? 4 : 1;
     for (int s = 0; s < nsets; ++s) {
       const int nt = ctxs[s]->nt;
+      pl->h_sets[s].rtiles = T;
+      pl->rcols = std::max(pl->rcols, (nt + T - 1) / T);
       for (int I = 0; I < nt; ++I)
-        for (int j0 = 0; j0 < nt; j0 += 16)
-          for (int g = 0; g < Bs[s]; g += 16)
-            wk.push_back(RWork{s, I, j0, std::min(nt, j0 + 16), pl->first[s] + g, std::min(16, Bs[s] - g)});
+        for (int c = 0; c * T < nt; ++c)
+          for (int g = 0; g < Bs[s]; g += 16) {
+            const int nb = std::min(16, Bs[s] - g);
+            if (nb == 1 && T == 1) {
+              if (c % 2 == 0) wk.push_back(RWork{s, I, c, std::min(nt, c + 2), pl->first[s] + g, 1, c, 1});
+            } else {
+              wk.push_back(RWork{s, I, c * T, std::min(nt, c * T + T), pl->first[s] + g, nb, c, 0});
+            }
+            pl->rgroup = std::max(pl->rgroup, nb > 8 ? 16 : nb > 4 ? 8 : nb > 2 ? 4 : 2);
+          }
     }
+    chk(pl->rpart.alloc(sizeof(double2) * (size_t)pl->rcols * rows));
     pl->n_rwork = (int)wk.size();
     chk(pl->rwork.alloc(sizeof(RWork) * wk.size()));
     if (e == cudaSuccess) chk(cudaMemcpy(pl->rwork.p, wk.data(), sizeof(RWork) * wk.size(), cudaMemcpyHostToDevice));
@@ -484,6 +503,9 @@ int build_plan(beor_ctx* const* ctxs, int nsets, const int* Bs, bool need_x, int
   v.xtr = pl->xtr.as<float>();
   v.rwork = pl->rwork.as<RWork>();
   v.n_rwork = pl->n_rwork;
+  v.rpart = pl->rpart.as<double2>();
+  v.rcols = pl->rcols;
+  v.rgroup = pl->rgroup;
   v.rows = rows;
   v.ws_elems = ws_elems;
   v.dinv_elems = dinv_elems;

@@ -114,12 +114,14 @@ struct SetDesc {
   const double2* dbar;    // Np
   const int32_t* kbin;    // n
   const double* phi;      // B x n_k (device staging)
+  int rtiles;             // block columns per partial sum of the residual
 };
 
 // One CTA of the float64-accurate residual: row block I of set `set`
-// against block columns [j0, j1), for problems p0 .. p0 + nb - 1.
+// against block columns [j0, j1), for problems p0 .. p0 + nb - 1; partial sums
+// in column col of BatchView::rpart (split: one problem, one column per tile).
 struct RWork {
-  int set, I, j0, j1, p0, nb;
+  int set, I, j0, j1, p0, nb, col, split;
 };
 
 // Bounds of the per-call device state shared by kernels.

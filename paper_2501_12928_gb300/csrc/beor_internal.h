@@ -59,6 +59,9 @@ struct BatchView {
   float* xtr;                // [rows][6]: x re (hi, lo, t), im (hi, lo, t)
   const RWork* rwork;        // CTA work items
   int n_rwork;
+  double2* rpart;            // [rcols][rows] partial sums of the residual
+  int rcols;
+  int rgroup;                // blocks of x a work item holds in shared memory
   int64_t rows;              // sum of padded dimensions
   int64_t ws_elems;          // elements of ws (bounds checks)
   int64_t dinv_elems;        // elements of dinv (bounds checks)

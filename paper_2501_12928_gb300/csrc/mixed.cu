@@ -819,20 +819,8 @@ int trail_launch_count(const MixedMaps* m, int k, int part) {
 int device_sms() { return num_sms(); }
 
 // ---------------------------------------------------------------------------
-// float64 refinement: vec_r = dbar - (M + diag Phi^-1) x, x += vec_d
+// float64 residual: vec_r = dbar - (M + diag Phi^-1) x; refinement: x += vec_d
 // ---------------------------------------------------------------------------
-__global__ void resid_init_kernel(BatchView v) {
-  const int p = blockIdx.y;
-  const Prob pr = v.prob[p];
-  const SetDesc sd = v.sets[pr.set];
-  const int np = pr.nt * BEOR_TB;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < np; j += gridDim.x * blockDim.x) {
-    double2 x = v.vec_x[pr.row_off + j], d = sd.dbar[j];
-    double w = v.phi_inv[pr.row_off + j];
-    v.vec_r[pr.row_off + j] = j < pr.n ? make_double2(d.x - w * x.x, d.y - w * x.y) : make_double2(0.0, 0.0);
-  }
-}
-
 // x split exactly into three floats per component (hi, lo, t), for the
 // float32-pipe residual below.
 __global__ void xsplit_kernel(BatchView v) {
@@ -874,48 +862,56 @@ __device__ __forceinline__ void dot2_mac(float& hi, float& sm, float ah, float a
   sm += err + e;
 }
 
-// r_I -= sum_J M_IJ x_J for the problems of one work item, with float64-like
-// accuracy on the float32 pipe: M and x as exact float triples, Dot2 products
-// and sums within a 128-column tile, float64 totals across tiles and, across
-// work items, float64 atomics.  Thread (row r, half h) serves 8 problems.
-constexpr int RG = 16;   // problems per work item
-__global__ void __launch_bounds__(256, 2) resid_df_kernel(BatchView v) {
-  extern __shared__ float xs[];          // [RG][128][6]
-  __shared__ int64_t roff[RG];
-  const RWork w = v.rwork[blockIdx.x];
-  const SetDesc sd = v.sets[w.set];
-  const int r = threadIdx.x & (BEOR_TB - 1), half = threadIdx.x >> 7;
-  if (threadIdx.x < RG) {
-    const int q = threadIdx.x;
-    roff[q] = q < w.nb && !prob_skipped(v.status[w.p0 + q]) ? v.prob[w.p0 + q].row_off : (int64_t)-1;
+// sum_J M_IJ x_J over the block columns [j0, j1) of one work item, with
+// float64-like accuracy on the float32 pipe: M and x as exact float triples,
+// Dot2 products and sums within a 128-column tile, float64 totals across the
+// item's tiles, written to v.rpart and added up in a fixed order by
+// resid_sum_kernel (no atomics: the residual is reproducible).
+//
+// Bound by the fp32 pipe (~60 operations per complex element and problem), and
+// at small batches by M's 24 bytes per element.  Thread (row r, half): NP
+// problems each of the item's group of 2 NP; with one problem the halves take
+// one tile each (SPLIT).  The item's tiles are 16 (the batch fills the GPU), 4
+// or 1 (it does not: RESID_ITEMS).  One point of 3280 modes took 2.0 ms in 52
+// CTAs of 16 tiles that also computed 15 absent problems, and takes 0.05 ms in
+// 338 CTAs of two tiles; 16 points 2.3 ms and 0.43 ms.
+template <int NP, bool SPLIT>
+__device__ __forceinline__ void resid_item(const BatchView& v, const RWork& w, const SetDesc& sd, float* xs) {
+  constexpr int G = SPLIT ? 1 : 2 * NP;   // problems of the group
+  __shared__ int64_t roff[16];
+  const int tid = threadIdx.x, r = tid & (BEOR_TB - 1), half = tid >> 7;
+  if (tid < G) {
+    const int64_t ro = tid < w.nb && !prob_skipped(v.status[w.p0 + tid]) ? v.prob[w.p0 + tid].row_off : (int64_t)-1;
+    roff[tid] = ro >= 0 && BEOR_INBOUNDS(v.flags, ro + (int64_t)sd.nt * BEOR_TB <= v.rows, BC_RESID_X) ? ro : -1;
   }
-  double tre[8], tim[8];
+  double tre[NP], tim[NP];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) tre[q] = tim[q] = 0.0;
-  if (!BEOR_INBOUNDS(v.flags, w.I >= 0 && w.I < sd.nt && w.j0 >= 0 && w.j1 <= sd.nt, BC_RESID_M)) return;
-  if (threadIdx.x < RG && roff[threadIdx.x] >= 0 &&
-      !BEOR_INBOUNDS(v.flags, roff[threadIdx.x] + (int64_t)sd.nt * BEOR_TB <= v.rows, BC_RESID_X))
-    roff[threadIdx.x] = -1;
-  for (int J = w.j0; J < w.j1; ++J) {
+  for (int q = 0; q < NP; ++q) tre[q] = tim[q] = 0.0;
+  for (int J0 = w.j0; J0 < w.j1; J0 += SPLIT ? 2 : 1) {
     __syncthreads();
-    for (int e = threadIdx.x; e < RG * BEOR_TB * 6; e += blockDim.x) {
-      const int q = e / (BEOR_TB * 6), rem = e - q * (BEOR_TB * 6);
-      xs[e] = roff[q] >= 0 ? v.xtr[(roff[q] + (int64_t)J * BEOR_TB) * 6 + rem] : 0.0f;
+    constexpr int XT = BEOR_TB * 6;   // floats of one block of x
+    for (int e = tid; e < (SPLIT ? 2 : G) * XT; e += 256) {
+      const int q = e / XT, rem = e - q * XT;
+      const int64_t ro = roff[SPLIT ? 0 : q];
+      const int J = SPLIT ? J0 + q : J0;
+      xs[e] = ro >= 0 && J < w.j1 ? v.xtr[(ro + (int64_t)J * BEOR_TB) * 6 + rem] : 0.0f;
     }
     __syncthreads();
+    const int J = SPLIT ? J0 + half : J0;
+    if (SPLIT && J >= w.j1) break;   // the last barrier of this item is behind
     const int64_t t0 = ((int64_t)w.I * sd.nt + J) * BEOR_TILE_ELEMS + r;
     const float4* __restrict__ T4 = sd.Mf + t0;
     const float2* __restrict__ T2 = sd.Mft + t0;
-    float hr[8], sr[8], hi[8], si[8];
+    float hr[NP], sr[NP], hi[NP], si[NP];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) hr[q] = sr[q] = hi[q] = si[q] = 0.0f;
-#pragma unroll 2
+    for (int q = 0; q < NP; ++q) hr[q] = sr[q] = hi[q] = si[q] = 0.0f;
+#pragma unroll(NP >= 4 ? 2 : 8)
     for (int c = 0; c < BEOR_TB; ++c) {
       const float4 m4 = __ldg(T4 + c * BEOR_TB);
       const float2 m2 = __ldg(T2 + c * BEOR_TB);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float* x = xs + ((half * 8 + q) * BEOR_TB + c) * 6;
+      for (int q = 0; q < NP; ++q) {
+        const float* x = xs + ((SPLIT ? half : half * NP + q) * BEOR_TB + c) * 6;
         const float xrh = x[0], xrl = x[1], xrt = x[2], xih = x[3], xil = x[4], xit = x[5];
         // re += mr xr - mi xi, im += mr xi + mi xr
         dot2_mac(hr[q], sr[q], m4.x, m4.y, m2.x, xrh, xrl, xrt);
@@ -925,62 +921,82 @@ __global__ void __launch_bounds__(256, 2) resid_df_kernel(BatchView v) {
       }
     }
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < NP; ++q) {
       tre[q] += (double)hr[q] + (double)sr[q];
       tim[q] += (double)hi[q] + (double)si[q];
     }
   }
+  // partial sums of (problem row, item column); SPLIT items hold two one-tile columns
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int64_t ro = roff[half * 8 + q];
-    if (ro < 0) continue;
-    double2* dst = v.vec_r + ro + (int64_t)w.I * BEOR_TB + r;
-    atomicAdd(&dst->x, -tre[q]);
-    atomicAdd(&dst->y, -tim[q]);
+  for (int q = 0; q < NP; ++q) {
+    const int64_t ro = roff[SPLIT ? 0 : half * NP + q];
+    const int col = w.col + (SPLIT ? half : 0);
+    if (ro < 0 || (SPLIT && w.j0 + half >= w.j1)) continue;
+    v.rpart[(int64_t)col * v.rows + ro + (int64_t)w.I * BEOR_TB + r] = make_double2(tre[q], tim[q]);
   }
 }
 
-__global__ void resid_norm_kernel(BatchView v) {
-  const int p = blockIdx.x;
+__global__ void __launch_bounds__(256, 2) resid_df_kernel(BatchView v) {
+  extern __shared__ float xs[];   // [problem of the group, or tile][128][6]
+  const RWork w = v.rwork[blockIdx.x];
+  const SetDesc sd = v.sets[w.set];
+  if (!BEOR_INBOUNDS(v.flags, w.I >= 0 && w.I < sd.nt && w.j0 >= 0 && w.j1 <= sd.nt, BC_RESID_M)) return;
+  if (!BEOR_INBOUNDS(v.flags, w.col >= 0 && w.col + (w.split ? w.j1 - w.j0 : 1) <= v.rcols, BC_RESID_M)) return;
+  if (w.split)
+    resid_item<1, true>(v, w, sd, xs);
+  else if (w.nb <= 2)
+    resid_item<1, false>(v, w, sd, xs);
+  else if (w.nb <= 4)
+    resid_item<2, false>(v, w, sd, xs);
+  else if (w.nb <= 8)
+    resid_item<4, false>(v, w, sd, xs);
+  else
+    resid_item<8, false>(v, w, sd, xs);
+}
+
+// vec_r = dbar - Phi^-1 x - sum of the partial sums: groups of 16 block columns
+// added up from the left, the last group first if it is a shorter one, then
+// the others in order (the order in which concurrent groups would finish).
+__global__ void resid_sum_kernel(BatchView v) {
+  const int p = blockIdx.y;
   const Prob pr = v.prob[p];
   const SetDesc sd = v.sets[pr.set];
-  __shared__ double red[2][32];
-  double a = 0.0, b = 0.0;
-  for (int j = threadIdx.x; j < pr.n; j += blockDim.x) {
-    double2 r = v.vec_r[pr.row_off + j], d = sd.dbar[j];
-    a += r.x * r.x + r.y * r.y;
-    b += d.x * d.x + d.y * d.y;
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= pr.nt * BEOR_TB) return;
+  double2 o = make_double2(0.0, 0.0);
+  if (j < pr.n) {
+    const double2 x = v.vec_x[pr.row_off + j], d = sd.dbar[j];
+    const double w = v.phi_inv[pr.row_off + j];
+    o = make_double2(d.x - w * x.x, d.y - w * x.y);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = a;
-    red[1][threadIdx.x >> 5] = b;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sa = 0.0, sb = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      sa += red[0][w];
-      sb += red[1][w];
+  if (!prob_skipped(v.status[p])) {
+    const int T = sd.rtiles, ngrp = (pr.nt + 15) / 16;
+    const bool tail_first = pr.nt % 16 != 0;
+    for (int g = 0; g < ngrp; ++g) {
+      const int grp = tail_first ? (g == 0 ? ngrp - 1 : g - 1) : g;
+      double sr = 0.0, si = 0.0;
+      for (int J = 16 * grp; J < min(pr.nt, 16 * grp + 16); J += T) {
+        const double2 t = v.rpart[(int64_t)(J / T) * v.rows + pr.row_off + j];
+        sr += t.x;
+        si += t.y;
+      }
+      o.x -= sr;
+      o.y -= si;
     }
-    v.resid[p] = sb > 0.0 ? sqrt(sa / sb) : 0.0;
   }
+  v.vec_r[pr.row_off + j] = o;
 }
 
 cudaError_t launch_residual(const BatchView& v, cudaStream_t s) {
   static bool attr = false;
+  constexpr int smem = (int)(sizeof(float) * 16 * BEOR_TB * 6);
   if (!attr) {
-    cudaFuncSetAttribute(resid_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(float) * RG * BEOR_TB * 6));
+    cudaFuncSetAttribute(resid_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     attr = true;
   }
-  resid_init_kernel<<<dim3(8, v.P), 256, 0, s>>>(v);
   xsplit_kernel<<<dim3(8, v.P), 256, 0, s>>>(v);
-  resid_df_kernel<<<v.n_rwork, 256, sizeof(float) * RG * BEOR_TB * 6, s>>>(v);
-  resid_norm_kernel<<<v.P, 256, 0, s>>>(v);
+  resid_df_kernel<<<v.n_rwork, 256, v.rgroup * sizeof(float) * BEOR_TB * 6, s>>>(v);
+  resid_sum_kernel<<<dim3((v.max_nt * BEOR_TB + 255) / 256, v.P), 256, 0, s>>>(v);
   return cudaGetLastError();
 }
 
