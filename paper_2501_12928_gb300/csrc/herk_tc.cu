@@ -155,7 +155,7 @@ __device__ __forceinline__ void hk_issue_half_stage(uint32_t tmem, uint32_t a0, 
 #pragma unroll
     for (int q = 0; q < slice_mma_count(sa, SLICE_PAIRS_FULL7); ++q) {
       const uint32_t acc = (first && sa == 0 && q < slice_mma_main(0)) ? 0u : 1u;
-      tc_mma(tmem + (uint32_t)slice_mma_col(sa, q), ad,
+      tc_mma(tc_a_use(q, slice_mma_count(sa, SLICE_PAIRS_FULL7)), tmem + (uint32_t)slice_mma_col(sa, q), ad,
              sdesc_kmajor(b0 + slice_mma_t(sa, q, SLICE_PAIRS_FULL7) * HK_SLICE),
              idesc_bf16(0, (uint32_t)slice_mma_n(sa, q)), acc);
     }

@@ -171,7 +171,7 @@ __device__ __forceinline__ void issue_half_stage(uint32_t tmem, uint64_t ad, uin
 #pragma unroll
     for (int q = 0; q < slice_mma_count(sa, SET); ++q) {
       const uint32_t acc = (first && sa == 0 && q < slice_mma_main(0)) ? 0u : 1u;
-      tc_mma(tmem + (uint32_t)slice_mma_col(sa, q), sdesc_add(ad, sa * MX_SLICE_A),
+      tc_mma(tc_a_use(q, slice_mma_count(sa, SET)), tmem + (uint32_t)slice_mma_col(sa, q), sdesc_add(ad, sa * MX_SLICE_A),
              sdesc_add(bd, slice_mma_t(sa, q, SET) * MX_SLICE_B), idesc_bf16(0, (uint32_t)slice_mma_n(sa, q)), acc);
     }
   }
