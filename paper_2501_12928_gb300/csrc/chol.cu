@@ -524,72 +524,63 @@ cudaError_t launch_diag(const BatchView& v, int k, bool mixed, int active, cudaS
 }
 
 // --------------------------------------------------------------------------
-// float64 panel: L_ik = A_ik Linv_kk^H for i > k (rows split in two halves)
+// float64 panel: L_ik = A_ik Linv_kk^H for i > k, R rows per CTA
+//
+// Bound by the float64 pipe.  Column c needs the terms m <= c only (Linv is
+// lower triangular; the terms left out are exact zeros): warp w takes the
+// eight-column groups w and 15 - w, which together have the same number of
+// terms for every w; lane = (row, part of the group's columns).  Few rows per
+// CTA where the batch is small, so that the work reaches every SM: one point of
+// 3280 modes took 26 ms in at most 50 CTAs of 64 rows (with the zeros) and takes
+// 3.3 ms with R = 8.
 // --------------------------------------------------------------------------
+template <int R>
 __global__ void __launch_bounds__(256) panel_f64_kernel(BatchView v, int kg) {
-  extern __shared__ double2 psm[];
-  double2* xs = psm;                  // [128 m][64 r]
-  double2* ys = psm + 128 * 64;       // [16 m][128 c]
+  __shared__ double2 xs[BEOR_TB][R];
+  constexpr int NC = R / 4;             // columns per thread and group
   const int p = blockIdx.y;
   const Prob pr = v.prob[p];
   const int k = kg - pr.k_off;
-  const int i = k + 1 + (blockIdx.x >> 1);
+  const int i = k + 1 + blockIdx.x / (BEOR_TB / R);
   if (k < 0 || i >= pr.nt || v.status[p] != 0) return;
-  const int r0 = (blockIdx.x & 1) * 64;
-  double2* tile = reinterpret_cast<double2*>(v.ws) + pr.ws_off + tri_index(i, k) * BEOR_TILE_ELEMS;
-  const double2* linv = v.dinv + pr.dinv_off + (int64_t)k * DG_PACK;
-  for (int e = threadIdx.x; e < 128 * 64; e += 256) {
-    int m = e / 64, r = e % 64;
-    xs[e] = tile[m * BEOR_TB + r0 + r];
+  const int r0 = (blockIdx.x % (BEOR_TB / R)) * R;
+  double2* tile = reinterpret_cast<double2*>(v.ws) + pr.ws_off + tri_index(i, k) * BEOR_TILE_ELEMS + r0;
+  const double2* __restrict__ linv = v.dinv + pr.dinv_off + (int64_t)k * DG_PACK;
+  for (int e = threadIdx.x; e < BEOR_TB * R; e += 256) xs[e / R][e % R] = tile[(e / R) * BEOR_TB + e % R];
+  __syncthreads();   // every element of these rows is read
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane % R, q = lane / R;
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    const int g = h ? 15 - warp : warp, c0 = 8 * g + q * NC;
+    double ar[NC], ai[NC];
+#pragma unroll
+    for (int b = 0; b < NC; ++b) ar[b] = ai[b] = 0.0;
+#pragma unroll 4
+    for (int m = 0; m < 8 * g + 8; ++m) {
+      const double2 x = xs[m][r];
+#pragma unroll
+      for (int b = 0; b < NC; ++b) {
+        const int c = c0 + b;
+        const double2 y = m <= c ? linv[pk(c, m)] : make_double2(0.0, 0.0);
+        // x * conj(y)
+        ar[b] = fma(x.x, y.x, fma(x.y, y.y, ar[b]));
+        ai[b] = fma(x.y, y.x, fma(-x.x, y.y, ai[b]));
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < NC; ++b) tile[(c0 + b) * BEOR_TB + r] = make_double2(ar[b], ai[b]);
   }
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double ar[4][8], ai[4][8];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 8; ++b) ar[a][b] = ai[a][b] = 0.0;
-  for (int m0 = 0; m0 < BEOR_TB; m0 += 16) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < 16 * 128; e += 256) {
-      int mm = e / 128, c = e % 128, m = m0 + mm;
-      ys[e] = m <= c ? linv[pk(c, m)] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    for (int mm = 0; mm < 16; ++mm) {
-      double2 x[4], y[8];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) x[a] = xs[(m0 + mm) * 64 + ty * 4 + a];
-#pragma unroll
-      for (int b = 0; b < 8; ++b) y[b] = ys[mm * 128 + tx * 8 + b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-          // x * conj(y)
-          ar[a][b] = fma(x[a].x, y[b].x, fma(x[a].y, y[b].y, ar[a][b]));
-          ai[a][b] = fma(x[a].y, y[b].x, fma(-x[a].x, y[b].y, ai[a][b]));
-        }
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      int r = r0 + ty * 4 + a, c = tx * 8 + b;
-      tile[c * BEOR_TB + r] = make_double2(ar[a][b], ai[a][b]);
-    }
 }
 
 cudaError_t launch_panel_f64(const BatchView& v, int k, cudaStream_t s) {
-  int nblk = 2 * (v.max_nt - 1 - k);
-  if (nblk <= 0) return cudaSuccess;
-  const size_t smem = sizeof(double2) * (128 * 64 + 16 * 128);
-  static bool init = false;
-  if (!init) {
-    cudaFuncSetAttribute(panel_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    init = true;
-  }
-  panel_f64_kernel<<<dim3(nblk, v.P), 256, smem, s>>>(v, k);
+  const int rows = v.max_nt - 1 - k;   // block rows
+  if (rows <= 0) return cudaSuccess;
+  // 32 rows per CTA read the inverse block (132 KB) a quarter as often; from
+  // four such CTAs per SM on
+  if ((int64_t)rows * 4 * v.P >= 4 * device_sms())
+    panel_f64_kernel<32><<<dim3(rows * 4, v.P), 256, 0, s>>>(v, k);
+  else
+    panel_f64_kernel<8><<<dim3(rows * 16, v.P), 256, 0, s>>>(v, k);
   return cudaGetLastError();
 }
 
