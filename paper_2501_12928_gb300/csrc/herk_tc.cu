@@ -51,10 +51,32 @@ constexpr int HK_KB_PASS = 64;                             // K-blocks of 128 pe
 constexpr int HK_JOBS = 4;
 enum { HK_ERR_TMA = 21, HK_ERR_MMA = 22, HK_ERR_ACC = 23, HK_ERR_EPI = 24 };
 
+// round-to-nearest-even of v 2^sh (|v| 2^sh < 2^55, sh <= 2 for normal v) by
+// integer operations; subnormal v: zero
+__device__ __forceinline__ long long hk_fixed(double v, int e) {
+  const long long bits = __double_as_longlong(v);
+  const int ex = (int)(bits >> 52) & 2047;
+  unsigned long long m = ex ? ((unsigned long long)bits & 0xfffffffffffffull) | 0x10000000000000ull : 0ull;
+  const int sh = ex - 1075 + 55 - e;
+  if (sh >= 0) {
+    m <<= min(sh, 2);
+  } else {
+    const int r = min(-sh, 60);
+    const unsigned long long low = m & ((1ull << r) - 1ull), half = 1ull << (r - 1);
+    m >>= r;
+    m += low > half || (low == half && (m & 1ull)) ? 1ull : 0ull;
+  }
+  return bits < 0 ? -(long long)m : (long long)m;
+}
+
 // ---------------------------------------------------------------------------
 // slicing: Y[j][v] = sqrt(w_v) T[v][j] for the K-blocks of one pass; block
 // (kb, 16 rows); digits of round(y 2^(55 - e_j)) for the row exponent e_j of
-// the block (largest |re|, |im| below 2^e_j)
+// the block (largest |re|, |im| below 2^e_j).  The float64 pipe forms the two
+// products of each element and nothing else: square roots once per visibility,
+// exponents, rounding and digits by integer operations (with a square root, a
+// scaling, a maximum and a conversion per element in float64, 90,972 x 3280
+// took 13.9 ms; now 2.7, the time of its 19 GB of traffic).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) herk_slice_kernel(const double2* __restrict__ T, int64_t ld,
                                                          const double* __restrict__ w, int64_t n_vis, int n,
@@ -63,32 +85,38 @@ __global__ void __launch_bounds__(256) herk_slice_kernel(const double2* __restri
                                                          int32_t* __restrict__ exps) {
   constexpr int R = 16;
   __shared__ double2 s[BEOR_TB][R + 1];   // [visibility][row]
+  __shared__ double s_sw[BEOR_TB];
   __shared__ int s_e[R];
   const int kb = blockIdx.x;
   const int64_t j0 = (int64_t)blockIdx.y * R;
   const int64_t vb = v0 + (int64_t)kb * BEOR_TB;
-  for (int e = threadIdx.x; e < BEOR_TB * R; e += 256) {
-    const int vl = e / R, jj = e % R;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double2 t[BEOR_TB * R / 256];
+#pragma unroll
+  for (int i = 0; i < BEOR_TB * R / 256; ++i) {   // every load in flight while the square roots are formed
+    const int e = threadIdx.x + 256 * i, vl = e / R, jj = e % R;
     const int64_t v = vb + vl, j = j0 + jj;
-    double2 y = make_double2(0.0, 0.0);
-    if (v < n_vis && j < n) {
-      const double2 t = T[v * ld + j];
-      const double sw = sqrt(w[v]);
-      y = make_double2(t.x * sw, t.y * sw);
-    }
-    s[vl][jj] = y;
+    t[i] = v < n_vis && j < n ? T[v * ld + j] : make_double2(0.0, 0.0);
+  }
+  if (threadIdx.x < BEOR_TB) s_sw[threadIdx.x] = vb + threadIdx.x < n_vis ? sqrt(w[vb + threadIdx.x]) : 0.0;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < BEOR_TB * R / 256; ++i) {
+    const int e = threadIdx.x + 256 * i, vl = e / R, jj = e % R;
+    const double sw = s_sw[vl];
+    s[vl][jj] = make_double2(t[i].x * sw, t[i].y * sw);
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int r = warp; r < R; r += 8) {
-    double mx = 0.0;
+    int mx = 0;   // high words: the exponent of the largest magnitude
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const double2 a = s[lane + 32 * q][r];
-      mx = fmax(mx, fmax(fabs(a.x), fabs(a.y)));
+      mx = max(mx, max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff));
     }
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    const int e = mx > 0.0 ? ilogb(mx) + 1 : -1000;
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    const int ex = mx >> 20;
+    const int e = ex > 22 && ex < 2047 ? ex - 1022 : -1000;   // below 2^-1000 (and not finite): no digits
     if (lane == 0) {
       s_e[r] = e;
       exps[(int64_t)kb * rows + j0 + r] = e;
@@ -100,49 +128,40 @@ __global__ void __launch_bounds__(256) herk_slice_kernel(const double2* __restri
   const int r = g * 8 + rr;
   const int c0 = warp * HK_KC + kh * 8;
   const int e = s_e[r];
-  uint32_t packed[HK_NPLANE][4];
-#pragma unroll
-  for (int q = 0; q < 8; q += 2) {
-    float val[2][HK_NPLANE];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const double2 a = s[c0 + q + u][r];
-#pragma unroll
-      for (int part = 0; part < 2; ++part) {   // 0: real, 1: imaginary
-        long long X = 0;
-        if (e > -1000) X = llrint(ldexp(part ? a.y : a.x, 55 - e));   // exact scaling; |X| < 2^55
-        int dg[HK_NS];
-#pragma unroll
-        for (int sl = HK_NS - 1; sl >= 1; --sl) {
-          const long long m = ((X + 128) & 255) - 128;
-          dg[sl] = (int)m;
-          X = (X - m) >> 8;
-        }
-        dg[0] = (int)X;
-#pragma unroll
-        for (int sl = 0; sl < HK_NS; ++sl) {
-          const float d = ldexpf((float)dg[sl], -8 * sl);
-          if (part == 0) {
-            val[u][slice_plane(sl, BEOR_PART_RE)] = d;
-          } else {
-            val[u][slice_plane(sl, BEOR_PART_IM)] = d;
-            val[u][slice_plane(sl, BEOR_PART_NEGIM)] = -d;
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int pl = 0; pl < HK_NPLANE; ++pl) {
-      const __nv_bfloat162 h2 = __floats2bfloat162_rn(val[0][pl], val[1][pl]);
-      packed[pl][q / 2] = *reinterpret_cast<const uint32_t*>(&h2);
-    }
-  }
   const int64_t plane_elems = rows * BEOR_TB * nkb_buf;
   const int64_t off = slice_elem_off(j0 + r, kb * BEOR_TB + c0, rows);   // 16-byte aligned
 #pragma unroll
-  for (int pl = 0; pl < HK_NPLANE; ++pl)
-    *reinterpret_cast<uint4*>(planes + (int64_t)pl * plane_elems + off) =
-        make_uint4(packed[pl][0], packed[pl][1], packed[pl][2], packed[pl][3]);
+  for (int part = 0; part < 2; ++part) {   // 0: real, 1: imaginary
+    uint32_t packed[HK_NS][4];
+#pragma unroll
+    for (int q = 0; q < 8; q += 2) {
+      unsigned long long x[2];   // + 128 in every digit but the first, so that each is a byte
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const double2 a = s[c0 + q + u][r];
+        x[u] = (unsigned long long)(e > -1000 ? hk_fixed(part ? a.y : a.x, e) : 0ll) + 0x0000808080808080ull;
+      }
+#pragma unroll
+      for (int sl = 0; sl < HK_NS; ++sl) {
+        uint32_t f[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int d = sl == 0 ? (int)((long long)x[u] >> 48) : (int)((x[u] >> (8 * (HK_NS - 1 - sl))) & 255) - 128;
+          // the digit's exact float without a conversion, scaled by 2^(-8 sl)
+          f[u] = __float_as_uint((__int_as_float(0x4B400000 + d) - 12582912.0f) * __int_as_float((127 - 8 * sl) << 23));
+        }
+        packed[sl][q / 2] = __byte_perm(f[0], f[1], 0x7632);
+      }
+    }
+#pragma unroll
+    for (int sl = 0; sl < HK_NS; ++sl) {
+      const uint4 v = make_uint4(packed[sl][0], packed[sl][1], packed[sl][2], packed[sl][3]);
+      *reinterpret_cast<uint4*>(planes + slice_plane(sl, part ? BEOR_PART_IM : BEOR_PART_RE) * plane_elems + off) = v;
+      if (part)
+        *reinterpret_cast<uint4*>(planes + slice_plane(sl, BEOR_PART_NEGIM) * plane_elems + off) =
+            make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
