@@ -1045,21 +1045,21 @@ int beor_get_M(beor_ctx* c, beor_c128* M_out) {
   if (r) return r;
   if (!c->have_pre || !M_out) return c->have_pre ? BEOR_EINVAL : BEOR_ESTATE;
   cudaSetDevice(c->device);
-  std::vector<double2> t((size_t)tri_count(c->nt) * BEOR_TILE_ELEMS);
-  CKC(c, cudaMemcpy(t.data(), c->M.p, sizeof(double2) * t.size(), cudaMemcpyDeviceToHost));
+  // unpacked on the device, by bands of rows of up to 256 MB for a host output
   const int64_t n = c->n;
-  std::vector<double2> full((size_t)n * n);
-  for (int64_t i = 0; i < n; ++i)
-    for (int64_t j = 0; j <= i; ++j) {
-      int I = (int)(i / BEOR_TB), J = (int)(j / BEOR_TB);
-      double2 v = t[(size_t)(tri_index(I, J) * BEOR_TILE_ELEMS + (j % BEOR_TB) * BEOR_TB + (i % BEOR_TB))];
-      full[(size_t)(i * n + j)] = v;
-      full[(size_t)(j * n + i)] = make_double2(v.x, -v.y);
-    }
+  double2* out = reinterpret_cast<double2*>(M_out);
   if (is_device_ptr(M_out)) {
-    CKC(c, cudaMemcpy(M_out, full.data(), sizeof(double2) * full.size(), cudaMemcpyHostToDevice));
-  } else {
-    std::memcpy(M_out, full.data(), sizeof(double2) * full.size());
+    CKC(c, unpack_hermitian(c->M.as<double2>(), c->n, 0, n, out, 0));
+    CKC(c, cudaDeviceSynchronize());
+    return BEOR_OK;
+  }
+  const int64_t band = std::max<int64_t>(1, std::min<int64_t>(n, ((int64_t)1 << 24) / n));
+  DevBuf buf;
+  CKC(c, buf.alloc(sizeof(double2) * (size_t)(band * n)));
+  for (int64_t r0 = 0; r0 < n; r0 += band) {
+    const int64_t rows = std::min(band, n - r0);
+    CKC(c, unpack_hermitian(c->M.as<double2>(), c->n, r0, rows, buf.as<double2>(), 0));
+    CKC(c, cudaMemcpy(out + r0 * n, buf.p, sizeof(double2) * (size_t)(rows * n), cudaMemcpyDeviceToHost));
   }
   return BEOR_OK;
 }

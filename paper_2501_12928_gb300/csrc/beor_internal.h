@@ -15,6 +15,8 @@ cudaError_t split_double_float(const double2* M, int64_t n, float4* out, cudaStr
 // Full nt x nt tile square of the packed lower M (n x n, padding zero), each
 // element split exactly into three floats per component.
 cudaError_t split_full_triple(const double2* M, int n, int nt, float4* hl, float2* t, cudaStream_t s);
+// Rows [r0, r0 + rows) of the full Hermitian n x n matrix, row-major, from its packed lower tiles.
+cudaError_t unpack_hermitian(const double2* M, int n, int64_t r0, int64_t rows, double2* out, cudaStream_t s);
 cudaError_t precompute_dense(const double2* T, int64_t n_vis, int n, int64_t ld, const double* w,
                              const double2* d, int nt, double2* Mt, double2* dbar, cudaStream_t s, bool tc);
 // herk_tc.cu: M (packed lower float64 tiles) = T^H diag(w) T on the tensor cores

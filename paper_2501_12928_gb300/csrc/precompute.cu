@@ -19,25 +19,18 @@
 namespace beor {
 
 // ---------------------------------------------------------------------------
-// C = X^H diag(w) X, X: K x n complex (row-major, leading dimension ldx),
-// batched over blockIdx.z with element strides.  Each CTA computes one
-// 64 x 64 sub-tile of a lower 128-tile.  mode 0: write packed tiles (the
-// factorisation layout); mode 1: write a dense row-major Hermitian matrix.
+// C = X^H diag(w) X, X: K x n complex (row-major, leading dimension ldx).  Each
+// CTA computes one 64 x 64 sub-tile of a lower 128-tile of C, in packed tiles
+// (the factorisation layout).
 // ---------------------------------------------------------------------------
 constexpr int HK_T = 64;   // sub-tile edge
 constexpr int HK_K = 16;   // K rows per smem stage
 
 __global__ void __launch_bounds__(256) herk_f64_kernel(const double2* __restrict__ X, int64_t ldx,
-                                                       int64_t x_batch_stride, const double* __restrict__ w,
-                                                       int64_t w_batch_stride, int64_t K, int n, int nt,
-                                                       double2* __restrict__ C, int64_t ldc,
-                                                       int64_t c_batch_stride, int mode) {
+                                                       const double* __restrict__ w, int64_t K, int n,
+                                                       double2* __restrict__ C) {
   __shared__ double2 sa[HK_K][HK_T];
   __shared__ double2 sb[HK_K][HK_T];
-  const int bz = blockIdx.z;
-  X += bz * x_batch_stride;
-  w += bz * w_batch_stride;
-  C += bz * c_batch_stride;
   // which 128-tile (I, J), I >= J, and which 64 sub-tile
   int t = blockIdx.x >> 2, sub = blockIdx.x & 3;
   int I = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
@@ -101,18 +94,81 @@ __global__ void __launch_bounds__(256) herk_f64_kernel(const double2* __restrict
       double vr = ar[p][q], vi = ai[p][q];
       if (r >= n || c >= n) { vr = 0.0; vi = 0.0; }
       if (r == c) vi = 0.0;
-      if (mode == 0) {
-        int64_t off = tri_index(I, J) * BEOR_TILE_ELEMS + (int64_t)(c - J * BEOR_TB) * BEOR_TB + (r - I * BEOR_TB);
-        C[off] = make_double2(vr, vi);
-      } else if (r < n && c < n) {
-        C[(int64_t)r * ldc + c] = make_double2(vr, vi);
-        if (I != J) C[(int64_t)c * ldc + r] = make_double2(vr, -vi);
-      }
+      C[tri_index(I, J) * BEOR_TILE_ELEMS + (int64_t)(c - J * BEOR_TB) * BEOR_TB + (r - I * BEOR_TB)] =
+          make_double2(vr, vi);
     }
 }
 
+// G_f = A_f^H diag(w_f) A_f of a factored instrument, f = blockIdx.y, lower
+// triangle of a row-major n x n matrix (n uv cells): one 16 x 16 tile per warp,
+// lane = (row, eight columns).  Bound by the float64 pipe (64 cycles per warp
+// instruction and sub-partition, so that the operands' way through shared
+// memory, eight rows at a time, costs nothing).  64 x 64 tiles left three
+// quarters of the work in padding and above the diagonal at 80 cells: 38
+// channels of 2394 rows 9.9 ms -> 2.85 (its floor is 2.7).  Each element sums the rows in
+// order, w on the column's side.
+constexpr int GK = 8;   // rows per step
+__global__ void __launch_bounds__(128) gram_cells_kernel(const double2* __restrict__ X, const double* __restrict__ w,
+                                                         int64_t K, int n, int ntiles, double2* __restrict__ G) {
+  __shared__ double2 sa[4][GK][16], sb[4][GK][16];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = blockIdx.x * 4 + warp;
+  if (t >= ntiles) return;
+  X += blockIdx.y * K * n;
+  w += blockIdx.y * K;
+  G += (int64_t)blockIdx.y * n * n;
+  int I = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while (I * (I + 1) / 2 > t) --I;
+  while ((I + 1) * (I + 2) / 2 <= t) ++I;
+  const int J = t - I * (I + 1) / 2;
+  const int r = lane >> 1, c0 = (lane & 1) * 8;
+  const int ca = min(16 * I + (lane & 15), n - 1), cb = min(16 * J + (lane & 15), n - 1), kl = lane >> 4;
+  double2 a[GK / 2], b[GK / 2];
+  auto load = [&](int64_t k0) {   // rows k0 + kl, + 2, ..; zeros beyond the last
+#pragma unroll
+    for (int i = 0; i < GK / 2; ++i) {
+      const int64_t k = k0 + kl + 2 * i, kc = min(k, K - 1);
+      a[i] = X[kc * n + ca];
+      b[i] = X[kc * n + cb];
+      const double ww = k < K ? w[kc] : 0.0;
+      b[i].x *= ww;
+      b[i].y *= ww;
+    }
+  };
+  double ar[8], ai[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) ar[q] = ai[q] = 0.0;
+  load(0);
+  for (int64_t k0 = 0; k0 < K; k0 += GK) {
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < GK / 2; ++i) {
+      sa[warp][kl + 2 * i][lane & 15] = a[i];
+      sb[warp][kl + 2 * i][lane & 15] = b[i];
+    }
+    __syncwarp();
+    if (k0 + GK < K) load(k0 + GK);
+    const int nk = (int)min((int64_t)GK, K - k0);
+#pragma unroll 2
+    for (int kk = 0; kk < nk; ++kk) {
+      const double2 x = sa[warp][kk][r];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const double2 y = sb[warp][kk][c0 + q];
+        // conj(x) * y
+        ar[q] = fma(x.x, y.x, fma(x.y, y.y, ar[q]));
+        ai[q] = fma(x.x, y.y, fma(-x.y, y.x, ai[q]));
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int i = 16 * I + r, j = 16 * J + c0 + q;
+    if (i < n && j <= i) G[(int64_t)i * n + j] = make_double2(ar[q], i == j ? 0.0 : ai[q]);
+  }
+}
+
 // u[b][j] = sum_k conj(X_b[k, j]) w_b[k] d_b[k]  (atomic accumulation over K chunks)
-__global__ void xh_w_d_kernel(const double2* __restrict__ X, int64_t ldx, int64_t x_batch_stride,
+__global__ void __launch_bounds__(256) xh_w_d_kernel(const double2* __restrict__ X, int64_t ldx, int64_t x_batch_stride,
                               const double* __restrict__ w, const double2* __restrict__ d,
                               int64_t vec_batch_stride, int64_t K, int n, int64_t kchunk,
                               double2* __restrict__ u, int64_t u_batch_stride) {
@@ -121,18 +177,30 @@ __global__ void xh_w_d_kernel(const double2* __restrict__ X, int64_t ldx, int64_
   w += bz * vec_batch_stride;
   d += bz * vec_batch_stride;
   u += bz * u_batch_stride;
-  int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  int64_t k0 = blockIdx.y * kchunk, k1 = min(K, k0 + kchunk);
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t k0 = blockIdx.y * kchunk, k1 = min(K, k0 + kchunk);
+  // w d of 256 rows at a time, formed once per CTA (two of six float64 products
+  // per element, on the pipe that bounds this kernel)
+  __shared__ double2 dw[256];
   double sr = 0.0, si = 0.0;
-  for (int64_t k = k0; k < k1; ++k) {
-    double2 x = X[k * ldx + j];
-    double2 dd = d[k];
-    double ww = w[k];
-    double dr = dd.x * ww, di = dd.y * ww;
-    sr = fma(x.x, dr, fma(x.y, di, sr));
-    si = fma(x.x, di, fma(-x.y, dr, si));
+  for (int64_t kb = k0; kb < k1; kb += 256) {
+    __syncthreads();
+    if (kb + threadIdx.x < k1) {
+      const double2 dd = d[kb + threadIdx.x];
+      const double ww = w[kb + threadIdx.x];
+      dw[threadIdx.x] = make_double2(dd.x * ww, dd.y * ww);
+    }
+    __syncthreads();
+    const int nk = (int)min((int64_t)256, k1 - kb);
+    const double2* __restrict__ x0 = X + kb * ldx + min(j, n - 1);
+#pragma unroll 8
+    for (int k = 0; k < nk; ++k) {
+      const double2 x = x0[k * ldx], q = dw[k];
+      sr = fma(x.x, q.x, fma(x.y, q.y, sr));
+      si = fma(x.x, q.y, fma(-x.y, q.x, si));
+    }
   }
+  if (j >= n) return;
   atomicAdd(&u[j].x, sr);
   atomicAdd(&u[j].y, si);
 }
@@ -225,6 +293,46 @@ __global__ void split_full_kernel(const double2* __restrict__ M, int n, int nt, 
   }
 }
 
+// Packed lower tiles -> rows of the full matrix, through 32 x 32 blocks in shared
+// memory (the tiles are column-major, the output row-major; blocks above the
+// diagonal are read from their mirror image).  86 MB read and 172 MB written at
+// 3280 modes; the host loop that did this took 60 ms.
+__global__ void __launch_bounds__(256) unpack_hermitian_kernel(const double2* __restrict__ M, int n, int64_t r0,
+                                                               int64_t rows, double2* __restrict__ out) {
+  __shared__ double2 s[32][33];
+  const int64_t rb = r0 + (int64_t)blockIdx.y * 32;   // the block's first row and column
+  const int cb = blockIdx.x * 32;
+  const int x = threadIdx.x & 31, y0 = threadIdx.x >> 5;
+  // source block: rows rs.., columns cs.. of the lower triangle
+  const bool mirror = rb + 31 < cb;
+  const int64_t rs = mirror ? cb : rb, cs = mirror ? rb : cb;
+  for (int y = y0; y < 32; y += 8) {   // x: row of the source (contiguous), y: column
+    int64_t i = rs + x, j = cs + y;
+    const bool flip = i < j;           // only in blocks that cross the diagonal
+    if (flip) {
+      const int64_t t = i;
+      i = j;
+      j = t;
+    }
+    double2 v = make_double2(0.0, 0.0);
+    if (i < n && j < n)
+      v = M[tri_index((int)(i / BEOR_TB), (int)(j / BEOR_TB)) * BEOR_TILE_ELEMS + (j % BEOR_TB) * BEOR_TB + i % BEOR_TB];
+    if (flip != mirror) v.y = -v.y;
+    s[y][x] = v;
+  }
+  __syncthreads();
+  for (int y = y0; y < 32; y += 8) {   // row y, column x of the output block
+    const int64_t r = rb + y;
+    if (r < r0 + rows && cb + x < n) out[(r - r0) * n + cb + x] = mirror ? s[y][x] : s[x][y];
+  }
+}
+
+cudaError_t unpack_hermitian(const double2* M, int n, int64_t r0, int64_t rows, double2* out, cudaStream_t s) {
+  const int nb = (n + 31) / 32;
+  unpack_hermitian_kernel<<<dim3(nb, (unsigned)((rows + 31) / 32)), 256, 0, s>>>(M, n, r0, rows, out);
+  return cudaGetLastError();
+}
+
 cudaError_t split_full_triple(const double2* M, int n, int nt, float4* hl, float2* t, cudaStream_t s) {
   split_full_kernel<<<nt * nt, 256, 0, s>>>(M, n, nt, hl, t);
   return cudaGetLastError();
@@ -243,12 +351,14 @@ cudaError_t precompute_dense(const double2* T, int64_t n_vis, int n, int64_t ld,
     e = herk_dense_tc(T, n_vis, n, ld, w, nt, Mt, s);   // seven-digit slice products (herk_tc.cu)
   } else {
     dim3 grid((unsigned)(tri_count(nt) * 4), 1, 1);
-    herk_f64_kernel<<<grid, 256, 0, s>>>(T, ld, 0, w, 0, n_vis, n, nt, Mt, 0, 0, 0);
+    herk_f64_kernel<<<grid, 256, 0, s>>>(T, ld, w, n_vis, n, Mt);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return e;
   cudaMemsetAsync(dbar, 0, sizeof(double2) * (size_t)nt * BEOR_TB, s);
-  int64_t kchunk = 4096;
+  // chunks of 1024 visibilities of a large T, so that its rows stream from memory on every SM
+  int64_t kchunk = n_vis <= 4096 ? 4096 : 1024;
+  while ((n_vis + kchunk - 1) / kchunk > 65535) kchunk *= 2;
   dim3 g2((n + 255) / 256, (unsigned)((n_vis + kchunk - 1) / kchunk), 1);
   xh_w_d_kernel<<<g2, 256, 0, s>>>(T, ld, 0, w, d, 0, n_vis, n, kchunk, dbar, 0);
   return cudaGetLastError();
@@ -258,10 +368,8 @@ cudaError_t precompute_factored(const double2* A, const double2* W, int nf, int6
                                 int nx, const double* w, const double2* d, int n, int nt,
                                 double2* G_scratch, double2* u_scratch, double2* Mt, double2* dbar,
                                 cudaStream_t s) {
-  int ntc = (ncells + BEOR_TB - 1) / BEOR_TB;
-  dim3 grid((unsigned)(tri_count(ntc) * 4), 1, (unsigned)nf);
-  herk_f64_kernel<<<grid, 256, 0, s>>>(A, ncells, ntb * ncells, w, ntb, ntb, ncells, ntc, G_scratch,
-                                        ncells, (int64_t)ncells * ncells, 1);
+  const int nb = (ncells + 15) / 16, tiles = nb * (nb + 1) / 2;
+  gram_cells_kernel<<<dim3((tiles + 3) / 4, nf), 128, 0, s>>>(A, w, ntb, ncells, tiles, G_scratch);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   int64_t total = tri_count(nt) * BEOR_TILE_ELEMS;
