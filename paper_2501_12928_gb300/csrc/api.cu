@@ -265,9 +265,10 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
       L += 1;
       if (mixed_tiles(pl.maps, 1, k) > 0) {
         // reserve_diag: leave free the SMs that step k + 1's diagonal blocks
-        // (one CTA each, running beside this launch) need
+        // (running beside this launch) need
         int cap = 0;
-        if (pl.sch.reserve_diag) cap = std::max(8, device_sms() - diag_tc_ctas(active(k + 1)));
+        if (pl.sch.reserve_diag)
+          cap = std::max(8, device_sms() - (v.mean ? DIAG_MEAN_CTAS : diag_tc_ctas(active(k + 1))));
         RUN_ON(KC_TRAIL, pl.side, launch_trail_mixed(v, pl.maps, k, TRAIL_REST, pl.side, 0, cap));
         L += trail_launch_count(pl.maps, k, TRAIL_REST);
       }

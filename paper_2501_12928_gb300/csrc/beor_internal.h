@@ -118,6 +118,9 @@ cudaError_t launch_diag(const BatchView& v, int k, bool mixed, int active, cudaS
 // diag_tc.cu: the mixed path's diagonal blocks of step k, of `active` problems
 cudaError_t launch_diag_tc(const BatchView& v, int k, int active, cudaStream_t s, int prio);
 int diag_tc_ctas(int active);   // CTAs of its launch
+constexpr int DIAG_MEAN_CTAS = 8;   // and of the posterior mean's
+// diag_cluster.cu: diagonal blocks of the float64 path and of the posterior mean
+cudaError_t launch_diag_cluster(const BatchView& v, int k, bool mixed, int active, cudaStream_t s, int prio);
 cudaError_t launch_panel_f64(const BatchView& v, int k, cudaStream_t s);
 cudaError_t launch_trail_f64(const BatchView& v, int k, cudaStream_t s);
 cudaError_t launch_solve(const BatchView& v, bool mixed, const double2* rhs, double2* out, cudaStream_t s);

@@ -17,22 +17,13 @@
 
 #include "beor_common.cuh"
 #include "beor_internal.h"
+#include "diag_common.cuh"
 
 namespace beor {
 
 // --------------------------------------------------------------------------
 // workspace element access
 // --------------------------------------------------------------------------
-__device__ __forceinline__ double2 ws_load(const double2* p) { return *p; }
-__device__ __forceinline__ double2 ws_load(const float4* p) {
-  float4 v = *p;
-  return make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
-}
-__device__ __forceinline__ void ws_store(double2* p, double2 v) { *p = v; }
-__device__ __forceinline__ void ws_store(float4* p, double2 v) {
-  float rh = (float)v.x, ih = (float)v.y;
-  *p = make_float4(rh, (float)(v.x - (double)rh), ih, (float)(v.y - (double)ih));
-}
 
 __device__ __forceinline__ void tile_of(int64_t t, int& I, int& J) {
   int i = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
@@ -171,356 +162,18 @@ cudaError_t launch_prior_init(const BatchView& v, bool mixed, cudaStream_t s) {
 }
 
 // --------------------------------------------------------------------------
-// diagonal block: float64 Cholesky, log-det, status, and the inverse of the
-// block (float64; on the mixed path formed on the fp32 pipe) with, on the
-// mixed path, the bf16 slices of its rows: value = 2^(e-7) sum_s sigma_s
-// 2^(-8 s), sigma_s integers with |sigma_s| <= 128.
-// --------------------------------------------------------------------------
-#define DG_PACK (BEOR_TB * (BEOR_TB + 1) / 2)
-__device__ __forceinline__ int pk(int i, int j) { return i * (i + 1) / 2 + j; }
-
-// Complex Dot2 accumulation of a b into c (c[0] + c[1] the real part,
-// c[2] + c[3] the imaginary part): a an element of L as double-float with
-// its third terms at, b a double-float element.
-__device__ __forceinline__ void cmac_l(dfl* c, float4 a, float2 at, float4 b) {
-  dot2_acc3(c[0], a.x, a.y, at.x, b.x, b.y);
-  dot2_acc3(c[1], -a.z, -a.w, -at.y, b.z, b.w);
-  dot2_acc3(c[2], a.x, a.y, at.x, b.z, b.w);
-  dot2_acc3(c[3], a.z, a.w, at.y, b.x, b.y);
-}
-__device__ __forceinline__ dfl df_add_quick(dfl x, dfl y) {
-  const dfl t = df_two_sum(x.hi, y.hi);
-  return dfl{t.hi, t.lo + (x.lo + y.lo)};
-}
-// Barrier of the 128 threads (four warps) of group id - 1.
-__device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
-
-// Block row I of the diagonal block's inverse, in place (512 threads): the
-// rows 32 I .. 32 I + 31 of L (packed, double-float plus third terms Lt),
-// every earlier block row and the diagonal block Linv_II already inverted.
-// Output (J, r, c) of the block row goes to thread o % 512 (o = 1024 J +
-// 32 r + c): lanes take consecutive columns, so a warp reads one element of
-// L (a broadcast) and 32 consecutive elements of Linv per step.
-template <int I>
-__device__ __forceinline__ void inv_block_row(float4* Af, const float2* Lt, int tid) {
-  constexpr int NQ = 2 * I;   // outputs per thread
-  dfl xr[NQ], xi[NQ];
-  // X_IJ = sum_{m = 32 J + c}^{32 I - 1} L[i][m] Linv[m][jj] (Linv_JJ is lower triangular)
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    const int o = tid + 512 * q, J = o >> 10, r = (o >> 5) & 31, c = o & 31;
-    const int i = 32 * I + r, jj = 32 * J + c;
-    dfl a[4] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
-    for (int m = jj; m < 32 * I; ++m) cmac_l(a, Af[pk(i, m)], Lt[pk(i, m)], Af[pk(m, jj)]);
-    xr[q] = df_add_quick(a[0], a[1]);
-    xi[q] = df_add_quick(a[2], a[3]);
-  }
-  __syncthreads();   // every read of block row I (as L) is done
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    const int o = tid + 512 * q, J = o >> 10, r = (o >> 5) & 31, c = o & 31;
-    const dfl ur = df_fast_two_sum(xr[q].hi, xr[q].lo), ui = df_fast_two_sum(xi[q].hi, xi[q].lo);
-    Af[pk(32 * I + r, 32 * J + c)] = make_float4(ur.hi, ur.lo, ui.hi, ui.lo);
-  }
-  __syncthreads();   // X in place of L_IJ
-  // Linv_IJ = -Linv_II X_IJ = -sum_{t <= r} Linv[i][32 I + t] X[32 I + t][jj]
-  const float2 zero = make_float2(0.0f, 0.0f);
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    const int o = tid + 512 * q, J = o >> 10, r = (o >> 5) & 31, c = o & 31;
-    const int i = 32 * I + r, jj = 32 * J + c;
-    dfl a[4] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
-    for (int t = 0; t <= r; ++t) cmac_l(a, Af[pk(i, 32 * I + t)], zero, Af[pk(32 * I + t, jj)]);
-    xr[q] = df_add_quick(a[0], a[1]);
-    xi[q] = df_add_quick(a[2], a[3]);
-  }
-  __syncthreads();   // every read of X is done
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    const int o = tid + 512 * q, J = o >> 10, r = (o >> 5) & 31, c = o & 31;
-    const dfl ur = df_fast_two_sum(xr[q].hi, xr[q].lo), ui = df_fast_two_sum(xi[q].hi, xi[q].lo);
-    Af[pk(32 * I + r, 32 * J + c)] = make_float4(-ur.hi, -ur.lo, -ui.hi, -ui.lo);
-  }
-  __syncthreads();
-}
-
-template <typename WS>
-__global__ void __launch_bounds__(512) diag_kernel(BatchView v, int kg, int mixed) {
-  extern __shared__ double2 dsm[];
-  double2* A = dsm;                    // packed lower 128x128
-  double2* col = dsm + DG_PACK;        // 128
-  __shared__ int s_fail;
-  __shared__ double s_rinv;            // 1 / L_jj of the current column
-  const int p = blockIdx.x;
-  const Prob pr = v.prob[p];
-  const int k = kg - pr.k_off;   // this problem's block step
-  if (k < 0 || k >= pr.nt) return;
-  if (v.status[p] != 0) return;
-  if (!BEOR_INBOUNDS(v.flags, pr.ws_off + (tri_index(k, k) + 1) * BEOR_TILE_ELEMS <= v.ws_elems, BC_DIAG_WS) ||
-      !BEOR_INBOUNDS(v.flags, pr.dinv_off + (int64_t)(k + 1) * DG_PACK <= v.dinv_elems, BC_DIAG_DINV) ||
-      !BEOR_INBOUNDS(v.flags, !mixed || (int64_t)(p + 1) * BEOR_TB <= (int64_t)v.P * BEOR_TB, BC_DIAG_LINV))
-    return;
-  WS* ws = reinterpret_cast<WS*>(v.ws) + pr.ws_off + tri_index(k, k) * BEOR_TILE_ELEMS;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  for (int e = tid; e < BEOR_TILE_ELEMS; e += nthr) {
-    int r = e % BEOR_TB, c = e / BEOR_TB;
-    if (r >= c) A[pk(r, c)] = ws_load(ws + e);
-  }
-  if (tid == 0) s_fail = 0;
-  __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31, nwarp = nthr >> 5;
-  // Right-looking Cholesky, two columns per pass (rank-2 updates): half the
-  // barriers and shared-memory round trips of one column per pass, with the
-  // same operations in the same order as the rank-1 sequence (identical
-  // results).  Thread 0 takes both pivots: L_jj, column j's element in row
-  // j+1 and its update of a_{j+1,j+1}, then L_{j+1,j+1}.
-  double2* col2 = col + BEOR_TB;   // column j+1 (this space later holds the mixed path's third terms of L)
-  __shared__ double s_rinv2;
-  for (int j = 0; j < BEOR_TB; j += 2) {
-    if (tid == 0) {
-      const double d = A[pk(j, j)].x;
-      if (!(d > 0.0) || !isfinite(d)) {
-        s_fail = k * BEOR_TB + j + 1;
-      } else {
-        const double l = sqrt(d);
-        A[pk(j, j)] = make_double2(l, 0.0);
-        const double rinv = 1.0 / l;
-        s_rinv = rinv;
-        double2 a = A[pk(j + 1, j)];
-        a.x *= rinv;
-        a.y *= rinv;
-        A[pk(j + 1, j)] = a;
-        col[j + 1] = a;
-        double2 x = A[pk(j + 1, j + 1)];
-        x.x = fma(-a.x, a.x, fma(-a.y, a.y, x.x));
-        x.y = fma(-a.y, a.x, fma(a.x, a.y, x.y));
-        const double d2 = x.x;
-        if (!(d2 > 0.0) || !isfinite(d2)) {
-          s_fail = k * BEOR_TB + j + 2;
-        } else {
-          const double l2 = sqrt(d2);
-          A[pk(j + 1, j + 1)] = make_double2(l2, 0.0);
-          s_rinv2 = 1.0 / l2;
-        }
-      }
-    }
-    __syncthreads();
-    if (s_fail) break;
-    const double inv = s_rinv, inv2 = s_rinv2;
-    const double2 lj1 = col[j + 1];   // L_{j+1,j}
-    // columns j and j+1 below the pair: scale column j, apply it to column
-    // j+1 (the rank-1 step's update of those elements), scale column j+1
-    for (int i = j + 2 + tid; i < BEOR_TB; i += nthr) {
-      double2 a = A[pk(i, j)];
-      a.x *= inv;
-      a.y *= inv;
-      A[pk(i, j)] = a;
-      col[i] = a;
-      double2 b = A[pk(i, j + 1)];
-      b.x = fma(-a.x, lj1.x, fma(-a.y, lj1.y, b.x));
-      b.y = fma(-a.y, lj1.x, fma(a.x, lj1.y, b.y));
-      b.x *= inv2;
-      b.y *= inv2;
-      A[pk(i, j + 1)] = b;
-      col2[i] = b;
-    }
-    __syncthreads();
-    // rank-2 update of the trailing lower triangle (rows and columns >= j+2):
-    // A_il -= L_ij conj(L_lj), then -= L_i,j+1 conj(L_l,j+1); the triangle's
-    // elements are dealt out in order, so every lane has work
-    {
-      const int nt2 = BEOR_TB - 2 - j;
-      const int total = nt2 * (nt2 + 1) / 2;
-      for (int e = tid; e < total; e += nthr) {
-        int a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-        while (a * (a + 1) / 2 > e) --a;
-        while ((a + 1) * (a + 2) / 2 <= e) ++a;
-        const int i = j + 2 + a, l = j + 2 + (e - a * (a + 1) / 2);
-        const double2 ai = col[i], al = col[l], bi = col2[i], bl = col2[l];
-        double2 x = A[pk(i, l)];
-        x.x = fma(-ai.x, al.x, fma(-ai.y, al.y, x.x));
-        x.y = fma(-ai.y, al.x, fma(ai.x, al.y, x.y));
-        x.x = fma(-bi.x, bl.x, fma(-bi.y, bl.y, x.x));
-        x.y = fma(-bi.y, bl.x, fma(bi.x, bl.y, x.y));
-        A[pk(i, l)] = x;
-      }
-    }
-    __syncthreads();
-  }
-  if (s_fail) {
-    if (tid == 0) v.status[p] = s_fail;
-    return;
-  }
-  // log-determinant contribution, 2 sum ln L_jj over the real rows, in parallel
-  {
-    __shared__ double red[32];
-    double ldp = 0.0;
-    if (tid < BEOR_TB && k * BEOR_TB + tid < pr.n) ldp = 2.0 * log(A[pk(tid, tid)].x);
-    for (int o = 16; o > 0; o >>= 1) ldp += __shfl_xor_sync(0xffffffffu, ldp, o);
-    if (lane == 0) red[warp] = ldp;
-    __syncthreads();
-    if (tid == 0) {
-      double s = 0.0;
-      for (int w = 0; w < nwarp; ++w) s += red[w];
-      v.logdet_sigma[p] += s;
-    }
-  }
-  // L_kk back to the workspace tile (upper part zero)
-  for (int e = tid; e < BEOR_TILE_ELEMS; e += nthr) {
-    int r = e % BEOR_TB, c = e / BEOR_TB;
-    ws_store(ws + e, r >= c ? A[pk(r, c)] : make_double2(0.0, 0.0));
-  }
-  __syncthreads();
-  if (!mixed) {
-    // in-place inverse, row by row: Linv[i][j] = -(sum_{m=j}^{i-1} L[i][m] Linv[m][j]) / L[i][i];
-    // four threads share each dot product (thread = 4 j + part)
-    const int jj = tid >> 2, part = tid & 3;
-    for (int i = 0; i < BEOR_TB; ++i) {
-      if (tid == 0) s_rinv = 1.0 / A[pk(i, i)].x;
-      double sr = 0.0, si = 0.0;
-      if (jj < i) {
-        for (int m = jj + part; m < i; m += 4) {
-          const double2 a = A[pk(i, m)], b = A[pk(m, jj)];
-          sr = fma(a.x, b.x, fma(-a.y, b.y, sr));
-          si = fma(a.x, b.y, fma(a.y, b.x, si));
-        }
-      }
-      sr += __shfl_xor_sync(0xffffffffu, sr, 1);
-      si += __shfl_xor_sync(0xffffffffu, si, 1);
-      sr += __shfl_xor_sync(0xffffffffu, sr, 2);
-      si += __shfl_xor_sync(0xffffffffu, si, 2);
-      __syncthreads();
-      if (jj < i && part == 0) {
-        const double inv = s_rinv;
-        A[pk(i, jj)] = make_double2(-sr * inv, -si * inv);
-      }
-      if (tid == 0) A[pk(i, i)] = make_double2(s_rinv, 0.0);
-      __syncthreads();
-    }
-    double2* dinv = v.dinv + pr.dinv_off + (int64_t)k * DG_PACK;
-    for (int e = tid; e < DG_PACK; e += nthr) dinv[e] = A[e];
-    return;
-  }
-  // Mixed path: the inverse feeds the 40-bit panel slices and the
-  // double-float solves only, so it is formed on the fp32 pipe instead of in
-  // float64, whose rate on this GPU is 1/64 of fp32.  L is split exactly into
-  // three floats per component: {re hi, re lo, im hi, im lo} in place (16
-  // bytes per element either way) and the third terms in Lt.  Each product
-  // L[i][m] Linv[m][j] keeps the terms down to 2^-48 of its leading part
-  // (Dot2 accumulation); Linv itself is held as double-float.
-  float4* Af = reinterpret_cast<float4*>(A);
-  float2* Lt = reinterpret_cast<float2*>(col + BEOR_TB);
-  for (int e = tid; e < DG_PACK; e += nthr) {
-    const double2 a = A[e];
-    const float rh = (float)a.x, ih = (float)a.y;
-    const double rd = a.x - (double)rh, id = a.y - (double)ih;
-    const float rl = (float)rd, il = (float)id;
-    Af[e] = make_float4(rh, rl, ih, il);
-    Lt[e] = make_float2((float)(rd - (double)rl), (float)(id - (double)il));
-  }
-  __shared__ dfl s_invs[BEOR_TB];      // 1 / L_ii for every row, formed in parallel
-  __syncthreads();                     // the split of L is complete
-  if (tid < BEOR_TB) {
-    const float4 d = Af[pk(tid, tid)];
-    s_invs[tid] = df_from_double(1.0 / ((double)d.x + (double)d.y + (double)Lt[pk(tid, tid)].x));
-  }
-  __syncthreads();
-  // Blocked inverse (four 32-row blocks): the diagonal blocks are inverted
-  // row by row, one block per 128 threads at once; then block row I = 1..3
-  // takes X_IJ = sum_{M=J}^{I-1} L_IM Linv_MJ for every J < I and
-  // Linv_IJ = -Linv_II X_IJ.  32 dependent row steps and 12 barriers instead
-  // of 128 row steps with two barriers each; the operations per element are
-  // those of the row recursion, with the division by L_ii of each step
-  // replaced by the product with the inverted diagonal block.
-  {
-    const int g = tid >> 7, lt = tid & 127, jl = lt >> 2, part = lt & 3;
-    const int jj = 32 * g + jl;
-    for (int il = 0; il < 32; ++il) {
-      const int i = 32 * g + il;
-      dfl c[4] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
-      if (jl < il)
-        for (int m = jj + part; m < i; m += 4) cmac_l(c, Af[pk(i, m)], Lt[pk(i, m)], Af[pk(m, jj)]);
-      dfl sr = df_add_quick(c[0], c[1]), si = df_add_quick(c[2], c[3]);
-#pragma unroll
-      for (int o = 1; o <= 2; o <<= 1) {
-        sr = df_add_quick(sr, dfl{__shfl_xor_sync(0xffffffffu, sr.hi, o), __shfl_xor_sync(0xffffffffu, sr.lo, o)});
-        si = df_add_quick(si, dfl{__shfl_xor_sync(0xffffffffu, si.hi, o), __shfl_xor_sync(0xffffffffu, si.lo, o)});
-      }
-      group_sync(1 + g);   // every read of row i (as L) is done
-      if (jl < il && part == 0) {
-        const dfl inv = s_invs[i];
-        const dfl qr = df_mul(df_fast_two_sum(sr.hi, sr.lo), inv);
-        const dfl qi = df_mul(df_fast_two_sum(si.hi, si.lo), inv);
-        Af[pk(i, jj)] = make_float4(-qr.hi, -qr.lo, -qi.hi, -qi.lo);
-      }
-      if (lt == 0) Af[pk(i, i)] = make_float4(s_invs[i].hi, s_invs[i].lo, 0.0f, 0.0f);
-      group_sync(1 + g);   // row i of Linv is complete
-    }
-  }
-  __syncthreads();
-  inv_block_row<1>(Af, Lt, tid);
-  inv_block_row<2>(Af, Lt, tid);
-  inv_block_row<3>(Af, Lt, tid);
-  double2* dinv = v.dinv + pr.dinv_off + (int64_t)k * DG_PACK;
-  for (int e = tid; e < DG_PACK; e += nthr) {
-    const float4 f = Af[e];
-    dinv[e] = make_double2((double)f.x + (double)f.y, (double)f.z + (double)f.w);
-  }
-  // slices of Linv rows (B operand of the panel product L_ik = A_ik Linv^H):
-  // balanced base-256 digits of round(x * 2^(39 - e)), x = hi + lo (scaled
-  // exactly by a power of two, rounded once)
-  const int64_t lrows = (int64_t)v.P * BEOR_TB;
-  const int64_t ps = lrows * BEOR_TB;   // one plane; plane index slice_plane(slice, part)
-  for (int c = warp; c < BEOR_TB; c += nwarp) {
-    float mx = 0.0f;
-    for (int m = lane; m <= c; m += 32) {
-      const float4 a = Af[pk(c, m)];
-      mx = fmaxf(mx, fmaxf(fabsf(a.x), fabsf(a.z)));
-    }
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    const int e = mx > 0.0f ? ilogbf(mx) + 1 : -1000;
-    const int64_t row = (int64_t)p * BEOR_TB + c;
-    if (lane == 0) v.linv_exp[row] = e;
-    for (int m = lane; m < BEOR_TB; m += 32) {
-      const float4 a = m <= c ? Af[pk(c, m)] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-      for (int part = 0; part < 2; ++part) {
-        const float hi = part ? a.z : a.x, lo = part ? a.w : a.y;
-        float dv[BEOR_NSLICE];
-        balanced_digits5(hi, lo, e, dv);
-        __nv_bfloat16* dst = v.linv_sl + slice_elem_off(row, m, lrows);
-#pragma unroll
-        for (int sl = 0; sl < BEOR_NSLICE; ++sl) {
-          const float d = dv[sl];
-          if (part == 0) {
-            dst[slice_plane(sl, BEOR_PART_RE) * ps] = __float2bfloat16_rn(d);
-          } else {
-            dst[slice_plane(sl, BEOR_PART_IM) * ps] = __float2bfloat16_rn(d);
-            dst[slice_plane(sl, BEOR_PART_NEGIM) * ps] = __float2bfloat16_rn(-d);
-          }
-        }
-      }
-    }
-  }
-}
-
-// Mixed plans of lnL factor their diagonal blocks in diag_tc.cu.  The
-// posterior mean keeps this kernel: its amplitudes are Sigma^-1 times the
+// diagonal blocks: Cholesky factor, log-det, status, and the inverse of the
+// block, with, on the mixed path, the bf16 slices of its rows
+//
+// lnL on the mixed path factors them in fixed point (diag_tc.cu).  The posterior
+// mean stays with float64: its amplitudes are Sigma^-1 times the
 // float64-accurate residual's rounding (relative 5e-8 at kappa ~ 1e8, 3280
 // modes), so that any other rounding of the factor moves them by as much,
 // while the quadratic form of lnL does not see it (1e-10).
+// --------------------------------------------------------------------------
 cudaError_t launch_diag(const BatchView& v, int k, bool mixed, int active, cudaStream_t s, int prio) {
   if (mixed && !v.mean) return launch_diag_tc(v, k, active, s, prio);
-  // packed block, one column, and (mixed) the third float terms of L
-  const size_t smem = sizeof(double2) * (DG_PACK + BEOR_TB) + sizeof(float2) * DG_PACK;
-  static bool init = false;
-  if (!init) {
-    cudaFuncSetAttribute(diag_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(diag_kernel<float4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    init = true;
-  }
-  if (mixed) return launch_prio(diag_kernel<float4>, dim3(v.P), dim3(512), smem, s, prio, v, k, 1);
-  return launch_prio(diag_kernel<double2>, dim3(v.P), dim3(512), smem, s, prio, v, k, 0);
+  return launch_diag_cluster(v, k, mixed, active, s, prio);
 }
 
 // --------------------------------------------------------------------------

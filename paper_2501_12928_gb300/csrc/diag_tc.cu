@@ -55,8 +55,7 @@
 
 #include <cmath>
 
-#include "beor_common.cuh"
-#include "beor_internal.h"
+#include "diag_common.cuh"
 #include "diag_fixed.cuh"
 
 namespace beor {
@@ -67,12 +66,11 @@ constexpr int DT_P = 16;                         // panel width and row block
 constexpr int DT_NPAN = BEOR_TB / DT_P;
 constexpr int DT_THREADS = 512;
 constexpr int DT_WARPS = DT_THREADS / 32;
-constexpr int DT_PACK = BEOR_TB * (BEOR_TB + 1) / 2;
 constexpr int DT_SLICE = BEOR_TB * 64;           // bytes of one digit of 128 rows x 32 (K)
 constexpr int DT_ZERO_E = -400;                  // exponent of an all-zero column
 
 struct DtSmem {
-  longlong2 s[DT_PACK];        // packed lower: fixed point (columns not yet eliminated) or Linv~ as float4
+  longlong2 s[DG_PACK];        // packed lower: fixed point (columns not yet eliminated) or Linv~ as float4
   unsigned char dg[FX_ND * DT_SLICE];   // digits: row i of L~ (i below the panel) or column i of Y (up to the panel)
   int ex[BEOR_TB];             // their exponents
   int es[BEOR_TB];             // e_i
@@ -91,7 +89,6 @@ struct DtSmem {
   int tile;                    // next tile of the rank-16 update
 };
 
-__device__ __forceinline__ int dt_pk(int i, int j) { return i * (i + 1) / 2 + j; }
 // byte offset of 16-byte chunk (2 K step + component) of a row in one digit:
 // 64 bytes per row, chunks permuted so that ldmatrix reads eight rows without
 // bank conflicts
@@ -227,7 +224,7 @@ __device__ __forceinline__ void dt_update(DtSmem& sm, int pan, int R, int cb, in
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int i = i0 + (q & 2 ? 8 : 0), c = c0 + (q & 1);
-      float4* f = reinterpret_cast<float4*>(&sm.s[dt_pk(i, c)]);
+      float4* f = reinterpret_cast<float4*>(&sm.s[pk(i, c)]);
       const pow2 ps = make_pow2(sm.ex[i] + sm.ex[c] - 60);
       const dfl wr = df_from_fixed(vre[q], ps), wi = df_from_fixed(vim[q], ps);
       const float4 o = c >= s0 ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : *f;   // the panel's own columns start at zero
@@ -243,12 +240,12 @@ __device__ __forceinline__ void dt_update(DtSmem& sm, int pan, int R, int cb, in
       const int i = i0 + (q & 2 ? 8 : 0), c = c0 + (q & 1);
       if (c > i) continue;
       const int sh = 60 - FX_FRAC - (sm.ex[i] + sm.ex[c]);   // -7 .. 53
-      longlong2 o = sm.s[dt_pk(i, c)];
+      longlong2 o = sm.s[pk(i, c)];
       const long long half = sh > 0 ? 1ll << (sh - 1) : 0;
       const int rsh = max(sh, 0), lsh = max(-sh, 0);
       o.x -= shl64((vre[q] + half) >> rsh, lsh);
       o.y -= shl64((vim[q] + half) >> rsh, lsh);
-      sm.s[dt_pk(i, c)] = o;
+      sm.s[pk(i, c)] = o;
       if (i == c && o.x <= 0) sm.bad[i] = 1;   // pivots only decrease from here on
     }
   }
@@ -293,9 +290,9 @@ __device__ __forceinline__ void dt_factor(DtSmem& sm, float4* __restrict__ ws, i
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int c = c0 + 8 * h;
-    x[h] = c <= r ? sm.s[dt_pk(s0 + r, s0 + c)] : make_longlong2(0, 0);
+    x[h] = c <= r ? sm.s[pk(s0 + r, s0 + c)] : make_longlong2(0, 0);
   }
-  long long d = sm.s[dt_pk(s0, s0)].x;
+  long long d = sm.s[pk(s0, s0)].x;
 #pragma unroll 1
   for (int j = 0; j < DT_P; ++j) {
     int g;
@@ -388,7 +385,7 @@ __device__ __forceinline__ void dt_solve(DtSmem& sm, float4* __restrict__ ws, in
   longlong2 x[NC];
   bool bad = sm.bad[row];
 #pragma unroll
-  for (int h = 0; h < NC; ++h) x[h] = sm.s[dt_pk(row, s0 + q + LPR * h)];
+  for (int h = 0; h < NC; ++h) x[h] = sm.s[pk(row, s0 + q + LPR * h)];
 #pragma unroll
   for (int h0 = 0; h0 < NC; ++h0) {
 #pragma unroll 1
@@ -483,14 +480,14 @@ __device__ __forceinline__ void dt_inverse_rows(DtSmem& sm, int pan, int j, int 
   for (int r = 0; r < DT_P; ++r) {
     dfl c0{j == s0 + r && !comp ? 1.0f : 0.0f, 0.0f}, c1{0.0f, 0.0f};
     if (j < s0) {
-      const float2 b = reinterpret_cast<const float2*>(&own->s[dt_pk(s0 + r, j)])[comp];
+      const float2 b = reinterpret_cast<const float2*>(&own->s[pk(s0 + r, j)])[comp];
       c0 = dfl{b.x, b.y};
     }
 #pragma unroll 2
     for (int m = m0; m < r; ++m) {
       const float4 a = sm.lpf[r][m];
       const float2 at = sm.lpt[r][m];
-      const float4 y = *reinterpret_cast<const float4*>(&sm.s[dt_pk(s0 + m, j)]);
+      const float4 y = *reinterpret_cast<const float4*>(&sm.s[pk(s0 + m, j)]);
       const float yh = comp ? y.z : y.x, yl = comp ? y.w : y.y, zh = comp ? y.x : y.z, zl = comp ? y.y : y.w;
       dot2_acc3(c0, a.x, a.y, at.x, yh, yl);
       dot2_acc3(c1, sg * a.z, sg * a.w, sg * at.y, zh, zl);
@@ -499,8 +496,8 @@ __device__ __forceinline__ void dt_inverse_rows(DtSmem& sm, int pan, int j, int 
     const dfl y = df_mul(df_fast_two_sum(s.hi, s.lo + (c0.lo + c1.lo)), sm.rinvf[r]);
     mx = fmaxf(mx, fabsf(y.hi));
     if (r >= m0) {
-      reinterpret_cast<float2*>(&sm.s[dt_pk(s0 + r, j)])[comp] = make_float2(y.hi, y.lo);
-      if (C > 1 && own != &sm) reinterpret_cast<float2*>(&own->s[dt_pk(s0 + r, j)])[comp] = make_float2(y.hi, y.lo);
+      reinterpret_cast<float2*>(&sm.s[pk(s0 + r, j)])[comp] = make_float2(y.hi, y.lo);
+      if (C > 1 && own != &sm) reinterpret_cast<float2*>(&own->s[pk(s0 + r, j)])[comp] = make_float2(y.hi, y.lo);
     }
     __syncwarp();
   }
@@ -517,7 +514,7 @@ __device__ __forceinline__ void dt_inverse_rows(DtSmem& sm, int pan, int j, int 
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int r = 8 * u + 2 * q + h;
-        const float2 y = r >= m0 ? reinterpret_cast<const float2*>(&sm.s[dt_pk(s0 + r, j)])[comp] : make_float2(0.0f, 0.0f);
+        const float2 y = r >= m0 ? reinterpret_cast<const float2*>(&sm.s[pk(s0 + r, j)])[comp] : make_float2(0.0f, 0.0f);
         xv[h] = fx_from_scaled(scale2f(y.x, ps), scale2f(y.y, ps));
       }
       dt_digits2(xv[0], xv[1], dg[q]);
@@ -545,7 +542,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) diag_tc_kernel(BatchView v, int
   if (k < 0 || k >= pr.nt) return;
   if (v.status[p] != 0) return;
   if (!BEOR_INBOUNDS(v.flags, pr.ws_off + (tri_index(k, k) + 1) * BEOR_TILE_ELEMS <= v.ws_elems, BC_DIAG_WS) ||
-      !BEOR_INBOUNDS(v.flags, pr.dinv_off + (int64_t)(k + 1) * DT_PACK <= v.dinv_elems, BC_DIAG_DINV) ||
+      !BEOR_INBOUNDS(v.flags, pr.dinv_off + (int64_t)(k + 1) * DG_PACK <= v.dinv_elems, BC_DIAG_DINV) ||
       !BEOR_INBOUNDS(v.flags, (int64_t)(p + 1) * BEOR_TB <= (int64_t)v.P * BEOR_TB, BC_DIAG_LINV))
     return;
   float4* ws = reinterpret_cast<float4*>(v.ws) + pr.ws_off + tri_index(k, k) * BEOR_TILE_ELEMS;
@@ -574,7 +571,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) diag_tc_kernel(BatchView v, int
       x = make_longlong2(fx_from_float(a.x, sh) + fx_from_float(a.y, sh), fx_from_float(a.z, sh) + fx_from_float(a.w, sh));
     else
       sm.bad[r] = 1;
-    sm.s[dt_pk(r, c)] = x;
+    sm.s[pk(r, c)] = x;
   }
   dt_sync<C>();   // every CTA's shared memory is ready for its peers
   if (warp < DT_FW && rank == 0) dt_factor<C>(sm, ws, 0, tid);
@@ -637,13 +634,13 @@ __global__ void __launch_bounds__(DT_THREADS, 1) diag_tc_kernel(BatchView v, int
   }
   // Linv = Linv~ diag(2^-e_j) (double-float) for the solves, and its rows'
   // exponents for the slices
-  float4* dinv = reinterpret_cast<float4*>(v.dinv) + pr.dinv_off + (int64_t)k * DT_PACK;
+  float4* dinv = reinterpret_cast<float4*>(v.dinv) + pr.dinv_off + (int64_t)k * DG_PACK;
   float4* Af = reinterpret_cast<float4*>(sm.s);
   for (int w = warp; w < BEOR_TB / C; w += DT_WARPS) {
     const int r = ((w >> 4) * C + rank) * 16 + (w & 15);
     float mx = 0.0f;
     for (int c = lane; c <= r; c += 32) {
-      const int e = dt_pk(r, c);
+      const int e = pk(r, c);
       const float4 f = Af[e];
       const pow2 ps = make_pow2(-sm.es[c]);
       const float4 g = make_float4(scale2f(f.x, ps), scale2f(f.y, ps), scale2f(f.z, ps), scale2f(f.w, ps));
@@ -665,57 +662,14 @@ __global__ void __launch_bounds__(DT_THREADS, 1) diag_tc_kernel(BatchView v, int
   // work item (own block of 16 rows, K-chunk of 16); lane = (8-row group, K
   // half, row), 16-byte chunks of eight columns, a warp writing 512 contiguous
   // bytes of every plane
-  const int64_t lrows = (int64_t)v.P * BEOR_TB;
-  const int64_t ps = lrows * BEOR_TB;   // one plane; plane index slice_plane(slice, part)
   for (int w = warp; w < 64 / C; w += DT_WARPS) {
-    const int R = (w >> 3) * C + rank, kc = w & 7;
-    const int r = R * 16 + (lane >> 4) * 8 + (lane & 7), c0 = kc * 16 + ((lane >> 3) & 1) * 8;
-    const int e = sm.ex[r];
-    const int64_t off = slice_elem_off((int64_t)p * BEOR_TB + r, c0, lrows);   // 16-byte aligned
-    if (kc > R) {   // above the diagonal
-#pragma unroll
-      for (int pl = 0; pl < BEOR_NPLANE; ++pl)
-        *reinterpret_cast<uint4*>(v.linv_sl + (int64_t)pl * ps + off) = make_uint4(0u, 0u, 0u, 0u);
-      continue;
-    }
-    uint32_t packed[BEOR_NPLANE][4];
-#pragma unroll
-    for (int q = 0; q < 8; q += 2) {
-      float val[2][BEOR_NPLANE];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int m = c0 + q + u;
-        const float4 a = m <= r ? Af[dt_pk(r, m)] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-        for (int part = 0; part < 2; ++part) {
-          float dv[BEOR_NSLICE];
-          balanced_digits5(part ? a.z : a.x, part ? a.w : a.y, e, dv);
-#pragma unroll
-          for (int sl = 0; sl < BEOR_NSLICE; ++sl) {
-            if (part == 0) {
-              val[u][slice_plane(sl, BEOR_PART_RE)] = dv[sl];
-            } else {
-              val[u][slice_plane(sl, BEOR_PART_IM)] = dv[sl];
-              val[u][slice_plane(sl, BEOR_PART_NEGIM)] = -dv[sl];
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int pl = 0; pl < BEOR_NPLANE; ++pl) {
-        const __nv_bfloat162 h2 = __floats2bfloat162_rn(val[0][pl], val[1][pl]);
-        packed[pl][q / 2] = *reinterpret_cast<const uint32_t*>(&h2);
-      }
-    }
-#pragma unroll
-    for (int pl = 0; pl < BEOR_NPLANE; ++pl)
-      *reinterpret_cast<uint4*>(v.linv_sl + (int64_t)pl * ps + off) =
-          make_uint4(packed[pl][0], packed[pl][1], packed[pl][2], packed[pl][3]);
+    const int r = ((w >> 3) * C + rank) * 16 + (lane >> 4) * 8 + (lane & 7);
+    linv_slice_chunk(v, p, Af, r, (w & 7) * 16 + ((lane >> 3) & 1) * 8, sm.ex[r]);
   }
 }
 
 template <int C>
-static cudaError_t launch_diag_cluster(const BatchView& v, int k, cudaStream_t s, int prio) {
+static cudaError_t launch_dt(const BatchView& v, int k, cudaStream_t s, int prio) {
   static bool init = false;
   if (!init) {
     cudaFuncSetAttribute(diag_tc_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DtSmem));
@@ -734,9 +688,9 @@ int diag_tc_ctas(int active) { return active * cluster_size(active); }
 
 cudaError_t launch_diag_tc(const BatchView& v, int k, int active, cudaStream_t s, int prio) {
   switch (cluster_size(active)) {
-    case 4: return launch_diag_cluster<4>(v, k, s, prio);
-    case 2: return launch_diag_cluster<2>(v, k, s, prio);
-    default: return launch_diag_cluster<1>(v, k, s, prio);
+    case 4: return launch_dt<4>(v, k, s, prio);
+    case 2: return launch_dt<2>(v, k, s, prio);
+    default: return launch_dt<1>(v, k, s, prio);
   }
 }
 
