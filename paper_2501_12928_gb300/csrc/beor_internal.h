@@ -106,6 +106,27 @@ static cudaError_t launch_cluster(void (*kern)(Exp...), dim3 grid, dim3 block, s
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Act>(args)...);
 }
+// Clusters of `cluster` CTAs of a kernel that the GPU holds at once: fewer than
+// the SMs alone would allow, since a cluster stays within one GPC.
+template <typename... Exp>
+static int max_clusters(void (*kern)(Exp...), int threads, size_t smem, int cluster) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(cluster);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cluster;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
 template <typename... Exp, typename... Act>
 static cudaError_t launch_prio(void (*kern)(Exp...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int prio,
                                Act&&... args) {

@@ -73,18 +73,10 @@ template <int C>
 __device__ __forceinline__ int dc_block(int rank, int q) {
   return q / 2 * 2 * C + (q & 1 ? 2 * C - 1 - rank : rank);
 }
-template <int C, typename T>
+template <typename T>
 __device__ __forceinline__ T* dc_peer(T* p, int rank) {
-  return C == 1 ? p : cg::this_cluster().map_shared_rank(p, rank);
+  return cg::this_cluster().map_shared_rank(p, rank);
 }
-template <int C>
-__device__ __forceinline__ void dc_sync() {
-  if (C == 1)
-    __syncthreads();
-  else
-    cg::this_cluster().sync();
-}
-
 // Complex Dot2 accumulation of a b into c (c[0] + c[1] the real part,
 // c[2] + c[3] the imaginary part): a an element of L as double-float with
 // its third terms at, b a double-float element.
@@ -206,7 +198,7 @@ __global__ void __launch_bounds__(DC_THREADS, 1) diag_cluster_kernel(BatchView v
   }
   if (tid < DC_P * DC_P && tid % DC_P >= tid / DC_P)
     A[pk(tid % DC_P, tid / DC_P)] = dc_load(ws + tid / DC_P * BEOR_TB + tid % DC_P);
-  dc_sync<C>();
+  cg::this_cluster().sync();
 
   for (int s0 = 0; s0 < BEOR_TB; s0 += DC_P) {
     const int s1 = s0 + DC_P;
@@ -236,12 +228,12 @@ __global__ void __launch_bounds__(DC_THREADS, 1) diag_cluster_kernel(BatchView v
       }
 #pragma unroll
       for (int c = 0; c < C; ++c) {
-        double2* o = dc_peer<C>(A, c);
+        double2* o = dc_peer(A, c);
         o[pk(row, s0 + q)] = x[0];
         o[pk(row, s0 + q + 8)] = x[1];
       }
     }
-    dc_sync<C>();
+    cg::this_cluster().sync();
     // rank-16 update of the own rows, 8 x 8 tiles; the next panel's diagonal block goes to every CTA
     int t = warp;
     for (int q = q0; q < NBLK; ++q) {
@@ -262,18 +254,18 @@ __global__ void __launch_bounds__(DC_THREADS, 1) diag_cluster_kernel(BatchView v
 #pragma unroll
           for (int o = 0; o < C; ++o) {
             if (o == rank) continue;
-            double2* B = dc_peer<C>(A, o);
+            double2* B = dc_peer(A, o);
             if (on0) B[pk(i, c)] = x0;
             if (on1) B[pk(i, c + 4)] = x1;
           }
       }
       t -= b - b1 + 1;
     }
-    dc_sync<C>();
+    cg::this_cluster().sync();
   }
   if (sm.fail) {
     if (tid == 0 && rank == 0) v.status[p] = sm.fail;
-    dc_sync<C>();
+    cg::this_cluster().sync();
     return;
   }
 
@@ -375,7 +367,7 @@ __global__ void __launch_bounds__(DC_THREADS, 1) diag_cluster_kernel(BatchView v
     // then X_IJ = sum_{M=J}^{I-1} L_IM Linv_MJ and Linv_IJ = -Linv_II X_IJ for
     // the own columns (blocks of eight, dealt like the rows).
     float4* Af = reinterpret_cast<float4*>(A);
-    dc_sync<C>();   // L is written out everywhere
+    cg::this_cluster().sync();   // L is written out everywhere
     for (int e = tid + rank * DC_THREADS; e < DG_PACK; e += C * DC_THREADS) {
       const double2 a = A[e];
       const float rh = (float)a.x, ih = (float)a.y;
@@ -385,11 +377,11 @@ __global__ void __launch_bounds__(DC_THREADS, 1) diag_cluster_kernel(BatchView v
       const float2 l3 = make_float2((float)(rd - (double)rl), (float)(id - (double)il));
 #pragma unroll
       for (int c = 0; c < C; ++c) {
-        dc_peer<C>(Af, c)[e] = f;
-        dc_peer<C>(Lt, c)[e] = l3;
+        dc_peer(Af, c)[e] = f;
+        dc_peer(Lt, c)[e] = l3;
       }
     }
-    dc_sync<C>();
+    cg::this_cluster().sync();
     if (tid < BEOR_TB) {
       const float4 d = Af[pk(tid, tid)];
       sm.invs[tid] = df_from_double(1.0 / ((double)d.x + (double)d.y + (double)Lt[pk(tid, tid)].x));
@@ -445,9 +437,9 @@ __global__ void __launch_bounds__(DC_THREADS, 1) diag_cluster_kernel(BatchView v
         }
       }
 #pragma unroll
-      for (int c = 0; c < C; ++c) dc_peer<C>(&sm, c)->rmax[rank][tid] = mx;
+      for (int c = 0; c < C; ++c) dc_peer(&sm, c)->rmax[rank][tid] = mx;
     }
-    dc_sync<C>();
+    cg::this_cluster().sync();
     if (tid < BEOR_TB) {
       float mx = 0.0f;
 #pragma unroll
@@ -464,32 +456,194 @@ __global__ void __launch_bounds__(DC_THREADS, 1) diag_cluster_kernel(BatchView v
   }
 }
 
-template <typename WS, int C>
-static cudaError_t launch_dc(const BatchView& v, int k, cudaStream_t s, int prio) {
-  constexpr size_t smem = dc_smem<std::is_same<WS, float4>::value>();
-  static bool init = false;
-  if (!init) {
-    cudaFuncSetAttribute(diag_cluster_kernel<WS, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    init = true;
+// One CTA per block, for batches that have more blocks than the GPU holds
+// clusters of two: the float64 pipe (0.87 ms of it per block and SM) bounds it,
+// and the finer steps of the cluster's kernel cost more of its instructions
+// (1.33 ms a block with C = 1, 1.17 here).
+__global__ void __launch_bounds__(512) diag_f64_kernel(BatchView v, int kg) {
+  extern __shared__ double2 dsm[];
+  double2* A = dsm;                    // packed lower 128x128
+  double2* col = dsm + DG_PACK;        // 128
+  __shared__ int s_fail;
+  __shared__ double s_rinv;            // 1 / L_jj of the current column
+  const int p = blockIdx.x;
+  const Prob pr = v.prob[p];
+  const int k = kg - pr.k_off;   // this problem's block step
+  if (k < 0 || k >= pr.nt) return;
+  if (v.status[p] != 0) return;
+  if (!BEOR_INBOUNDS(v.flags, pr.ws_off + (tri_index(k, k) + 1) * BEOR_TILE_ELEMS <= v.ws_elems, BC_DIAG_WS) ||
+      !BEOR_INBOUNDS(v.flags, pr.dinv_off + (int64_t)(k + 1) * DG_PACK <= v.dinv_elems, BC_DIAG_DINV))
+    return;
+  double2* ws = reinterpret_cast<double2*>(v.ws) + pr.ws_off + tri_index(k, k) * BEOR_TILE_ELEMS;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  for (int e = tid; e < BEOR_TILE_ELEMS; e += nthr) {
+    int r = e % BEOR_TB, c = e / BEOR_TB;
+    if (r >= c) A[pk(r, c)] = ws[e];
   }
-  return launch_cluster(diag_cluster_kernel<WS, C>, dim3(C * v.P), dim3(DC_THREADS), smem, s, prio, C, v, k);
+  if (tid == 0) s_fail = 0;
+  __syncthreads();
+  const int warp = tid >> 5, lane = tid & 31, nwarp = nthr >> 5;
+  // Right-looking Cholesky, two columns per pass (rank-2 updates): half the
+  // barriers and shared-memory round trips of one column per pass, with the
+  // same operations in the same order as the rank-1 sequence (identical
+  // results).  Thread 0 takes both pivots: L_jj, column j's element in row
+  // j+1 and its update of a_{j+1,j+1}, then L_{j+1,j+1}.
+  double2* col2 = col + BEOR_TB;   // column j+1
+  __shared__ double s_rinv2;
+  for (int j = 0; j < BEOR_TB; j += 2) {
+    if (tid == 0) {
+      const double d = A[pk(j, j)].x;
+      if (!(d > 0.0) || !isfinite(d)) {
+        s_fail = k * BEOR_TB + j + 1;
+      } else {
+        const double l = sqrt(d);
+        A[pk(j, j)] = make_double2(l, 0.0);
+        const double rinv = 1.0 / l;
+        s_rinv = rinv;
+        double2 a = A[pk(j + 1, j)];
+        a.x *= rinv;
+        a.y *= rinv;
+        A[pk(j + 1, j)] = a;
+        col[j + 1] = a;
+        double2 x = A[pk(j + 1, j + 1)];
+        x.x = fma(-a.x, a.x, fma(-a.y, a.y, x.x));
+        x.y = fma(-a.y, a.x, fma(a.x, a.y, x.y));
+        const double d2 = x.x;
+        if (!(d2 > 0.0) || !isfinite(d2)) {
+          s_fail = k * BEOR_TB + j + 2;
+        } else {
+          const double l2 = sqrt(d2);
+          A[pk(j + 1, j + 1)] = make_double2(l2, 0.0);
+          s_rinv2 = 1.0 / l2;
+        }
+      }
+    }
+    __syncthreads();
+    if (s_fail) break;
+    const double inv = s_rinv, inv2 = s_rinv2;
+    const double2 lj1 = col[j + 1];   // L_{j+1,j}
+    // columns j and j+1 below the pair: scale column j, apply it to column
+    // j+1 (the rank-1 step's update of those elements), scale column j+1
+    for (int i = j + 2 + tid; i < BEOR_TB; i += nthr) {
+      double2 a = A[pk(i, j)];
+      a.x *= inv;
+      a.y *= inv;
+      A[pk(i, j)] = a;
+      col[i] = a;
+      double2 b = A[pk(i, j + 1)];
+      b.x = fma(-a.x, lj1.x, fma(-a.y, lj1.y, b.x));
+      b.y = fma(-a.y, lj1.x, fma(a.x, lj1.y, b.y));
+      b.x *= inv2;
+      b.y *= inv2;
+      A[pk(i, j + 1)] = b;
+      col2[i] = b;
+    }
+    __syncthreads();
+    // rank-2 update of the trailing lower triangle (rows and columns >= j+2):
+    // A_il -= L_ij conj(L_lj), then -= L_i,j+1 conj(L_l,j+1); the triangle's
+    // elements are dealt out in order, so every lane has work
+    {
+      const int nt2 = BEOR_TB - 2 - j;
+      const int total = nt2 * (nt2 + 1) / 2;
+      for (int e = tid; e < total; e += nthr) {
+        int a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+        while (a * (a + 1) / 2 > e) --a;
+        while ((a + 1) * (a + 2) / 2 <= e) ++a;
+        const int i = j + 2 + a, l = j + 2 + (e - a * (a + 1) / 2);
+        const double2 ai = col[i], al = col[l], bi = col2[i], bl = col2[l];
+        double2 x = A[pk(i, l)];
+        x.x = fma(-ai.x, al.x, fma(-ai.y, al.y, x.x));
+        x.y = fma(-ai.y, al.x, fma(ai.x, al.y, x.y));
+        x.x = fma(-bi.x, bl.x, fma(-bi.y, bl.y, x.x));
+        x.y = fma(-bi.y, bl.x, fma(bi.x, bl.y, x.y));
+        A[pk(i, l)] = x;
+      }
+    }
+    __syncthreads();
+  }
+  if (s_fail) {
+    if (tid == 0) v.status[p] = s_fail;
+    return;
+  }
+  // log-determinant contribution, 2 sum ln L_jj over the real rows, in parallel
+  {
+    __shared__ double red[32];
+    double ldp = 0.0;
+    if (tid < BEOR_TB && k * BEOR_TB + tid < pr.n) ldp = 2.0 * log(A[pk(tid, tid)].x);
+    for (int o = 16; o > 0; o >>= 1) ldp += __shfl_xor_sync(0xffffffffu, ldp, o);
+    if (lane == 0) red[warp] = ldp;
+    __syncthreads();
+    if (tid == 0) {
+      double s = 0.0;
+      for (int w = 0; w < nwarp; ++w) s += red[w];
+      v.logdet_sigma[p] += s;
+    }
+  }
+  // L_kk back to the workspace tile (upper part zero)
+  for (int e = tid; e < BEOR_TILE_ELEMS; e += nthr) {
+    int r = e % BEOR_TB, c = e / BEOR_TB;
+    ws[e] = r >= c ? A[pk(r, c)] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  // in-place inverse, row by row: Linv[i][j] = -(sum_{m=j}^{i-1} L[i][m] Linv[m][j]) / L[i][i];
+  // four threads share each dot product (thread = 4 j + part)
+  const int jj = tid >> 2, part = tid & 3;
+  for (int i = 0; i < BEOR_TB; ++i) {
+    if (tid == 0) s_rinv = 1.0 / A[pk(i, i)].x;
+    double sr = 0.0, si = 0.0;
+    if (jj < i) {
+      for (int m = jj + part; m < i; m += 4) {
+        const double2 a = A[pk(i, m)], b = A[pk(m, jj)];
+        sr = fma(a.x, b.x, fma(-a.y, b.y, sr));
+        si = fma(a.x, b.y, fma(a.y, b.x, si));
+      }
+    }
+    sr += __shfl_xor_sync(0xffffffffu, sr, 1);
+    si += __shfl_xor_sync(0xffffffffu, si, 1);
+    sr += __shfl_xor_sync(0xffffffffu, sr, 2);
+    si += __shfl_xor_sync(0xffffffffu, si, 2);
+    __syncthreads();
+    if (jj < i && part == 0) {
+      const double inv = s_rinv;
+      A[pk(i, jj)] = make_double2(-sr * inv, -si * inv);
+    }
+    if (tid == 0) A[pk(i, i)] = make_double2(s_rinv, 0.0);
+    __syncthreads();
+  }
+  double2* dinv = v.dinv + pr.dinv_off + (int64_t)k * DG_PACK;
+  for (int e = tid; e < DG_PACK; e += nthr) dinv[e] = A[e];
 }
 
-// Float64: the largest cluster, of up to eight CTAs, with which the batch fits
-// the GPU's SMs.  The posterior mean is of one point, and always takes eight.
-static int cluster_size(int active) {
-  int c = 8;
-  while (c > 1 && c * active > device_sms()) c /= 2;
-  return c;
+template <typename WS, int C>
+static int dc_fit() {   // blocks that are factored at once
+  constexpr size_t smem = dc_smem<std::is_same<WS, float4>::value>();
+  static const int n = [] {   // once: the kernel's attribute, and the device's answer
+    cudaFuncSetAttribute(diag_cluster_kernel<WS, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return max_clusters(diag_cluster_kernel<WS, C>, DC_THREADS, smem, C);
+  }();
+  return n;
 }
+template <typename WS, int C>
+static cudaError_t launch_dc(const BatchView& v, int k, cudaStream_t s, int prio) {
+  dc_fit<WS, C>();
+  return launch_cluster(diag_cluster_kernel<WS, C>, dim3(C * v.P), dim3(DC_THREADS),
+                        dc_smem<std::is_same<WS, float4>::value>(), s, prio, C, v, k);
+}
+
+// Float64: the largest cluster, of up to eight CTAs, of which the GPU holds the
+// whole batch at once (15 clusters of eight, 36 of four and 76 of two on a GB300:
+// 0.39, 0.50 and 0.77 ms a block), else one CTA per block (1.17 ms).  The
+// posterior mean is of one point, and always takes eight.
 cudaError_t launch_diag_cluster(const BatchView& v, int k, bool mixed, int active, cudaStream_t s, int prio) {
   if (mixed) return launch_dc<float4, DIAG_MEAN_CTAS>(v, k, s, prio);
-  switch (cluster_size(active)) {
-    case 8: return launch_dc<double2, 8>(v, k, s, prio);
-    case 4: return launch_dc<double2, 4>(v, k, s, prio);
-    case 2: return launch_dc<double2, 2>(v, k, s, prio);
-    default: return launch_dc<double2, 1>(v, k, s, prio);
-  }
+  if (active <= dc_fit<double2, 8>()) return launch_dc<double2, 8>(v, k, s, prio);
+  if (active <= dc_fit<double2, 4>()) return launch_dc<double2, 4>(v, k, s, prio);
+  if (active <= dc_fit<double2, 2>()) return launch_dc<double2, 2>(v, k, s, prio);
+  constexpr size_t smem = sizeof(double2) * (DG_PACK + 2 * BEOR_TB);   // packed block and two columns
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(diag_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (attr != cudaSuccess) return attr;
+  return launch_prio(diag_f64_kernel, dim3(v.P), dim3(512), smem, s, prio, v, k);
 }
 
 }  // namespace beor

@@ -669,21 +669,22 @@ __global__ void __launch_bounds__(DT_THREADS, 1) diag_tc_kernel(BatchView v, int
 }
 
 template <int C>
-static cudaError_t launch_dt(const BatchView& v, int k, cudaStream_t s, int prio) {
-  static bool init = false;
-  if (!init) {
+static int dt_fit() {   // blocks that are factored at once
+  static const int n = [] {   // once: the kernel's attribute, and the device's answer
     cudaFuncSetAttribute(diag_tc_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DtSmem));
-    init = true;
-  }
+    return C == 1 ? device_sms() : max_clusters(diag_tc_kernel<C>, DT_THREADS, sizeof(DtSmem), C);
+  }();
+  return n;
+}
+template <int C>
+static cudaError_t launch_dt(const BatchView& v, int k, cudaStream_t s, int prio) {
+  dt_fit<C>();
   return launch_cluster(diag_tc_kernel<C>, dim3(C * v.P), dim3(DT_THREADS), sizeof(DtSmem), s, prio, C, v, k);
 }
 
-// Clusters of four CTAs per block while they fit the GPU's SMs, else of two,
-// else single CTAs.
-static int cluster_size(int active) {
-  const int sms = device_sms();
-  return 4 * active <= sms ? 4 : 2 * active <= sms ? 2 : 1;
-}
+// Clusters of four CTAs per block, or of two, while the GPU holds the batch's at
+// once (36 and 76 on a GB300), else single CTAs.
+static int cluster_size(int active) { return active <= dt_fit<4>() ? 4 : active <= dt_fit<2>() ? 2 : 1; }
 int diag_tc_ctas(int active) { return active * cluster_size(active); }
 
 cudaError_t launch_diag_tc(const BatchView& v, int k, int active, cudaStream_t s, int prio) {

@@ -1,5 +1,5 @@
-"""Float64 diagonal blocks at every cluster size (eight CTAs per block up to 19
-problems, four up to 38, two up to 76, one beyond): the operations on an element
+"""Float64 diagonal blocks at every cluster size (eight CTAs per block up to 15
+problems, four up to 36, two up to 76, one beyond): the operations on an element
 do not depend on it, so lnL and the factor are the same bits; a point that is not
 positive definite fails at its column without touching the others."""
 
@@ -31,7 +31,7 @@ def test_same_bits_at_every_cluster_size(n):
     M, db = O.herm_dense(p["T"], p["noise_var"]), O.dbar_dense(p["T"], p["noise_var"], p["d"])
     ref = O.evaluate(M, db, p["kbin"], ph[0], 2.0)["lnl"]
     base = None
-    for B in (1, 19, 20, 38, 39, 76, 77, 90):
+    for B in (1, 15, 16, 36, 37, 76, 77, 90):
         lnl, st = lk.lnl(ph[:B])
         assert np.all(st == 0)
         assert abs(lnl[0] - ref) <= 1e-9 * abs(ref)
