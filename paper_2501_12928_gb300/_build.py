@@ -10,7 +10,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libbeor.so")
 LIB_CHECKED = os.path.join(OUT_DIR, "libbeor_checked.so")
 SOURCES = ["api.cu", "precompute.cu", "chol.cu", "mixed.cu", "mlp.cu", "noalloc.cu", "autotune.cu", "instrument.cu", "herk_tc.cu",
-           "diag_tc.cu", "diag_cluster.cu"]
+           "diag_tc.cu", "diag_cluster.cu", "solve.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-Xptxas", "-warn-spills"]

@@ -310,336 +310,6 @@ cudaError_t launch_trail_f64(const BatchView& v, int k, cudaStream_t s) {
 }
 
 // --------------------------------------------------------------------------
-// Triangular solves with the factor: out = L^-H L^-1 rhs, blocked by 128.
-// One launch per block step covers every problem: CTA (i, p) applies the
-// update of block row i with the block just solved; the CTA that completes
-// the next block row also applies that block's float64 inverse, so a step's
-// critical path is one tile update plus one 128 x 128 float64 matvec.
-// Off-diagonal products: float64 for the float64 path, double-float (fp32
-// pairs) for the mixed path's double-float factor.
-// --------------------------------------------------------------------------
-struct CAcc {          // complex accumulator
-  double2 d;           // float64 path
-  dfl re, im;          // double-float path: hi = error-free running sum, lo = its accumulated errors
-};
-
-__device__ __forceinline__ void cacc_zero(CAcc& a) {
-  a.d = make_double2(0.0, 0.0);
-  a.re = dfl{0.0f, 0.0f};
-  a.im = dfl{0.0f, 0.0f};
-}
-// a += L * y (conj_l: a += conj(L) * y); y given as double2 and as double-float pairs
-__device__ __forceinline__ void cacc_mac(CAcc& a, const double2* L, double2 y, dfl, dfl, bool conj_l) {
-  const double2 l = *L;
-  const double li = conj_l ? -l.y : l.y;
-  a.d.x = fma(l.x, y.x, fma(-li, y.y, a.d.x));
-  a.d.y = fma(l.x, y.y, fma(li, y.x, a.d.y));
-}
-__device__ __forceinline__ void cacc_mac(CAcc& a, const float4* L, double2, dfl yr, dfl yi, bool conj_l) {
-  const float4 l = *L;
-  const float lih = conj_l ? -l.z : l.z, lil = conj_l ? -l.w : l.w;
-  // re += lr yr - li yi, im += lr yi + li yr
-  dot2_acc(a.re, l.x, l.y, yr.hi, yr.lo);
-  dot2_acc(a.re, -lih, -lil, yi.hi, yi.lo);
-  dot2_acc(a.im, l.x, l.y, yi.hi, yi.lo);
-  dot2_acc(a.im, lih, lil, yr.hi, yr.lo);
-}
-__device__ __forceinline__ double2 cacc_get(const CAcc& a, const double2*) { return a.d; }
-__device__ __forceinline__ double2 cacc_get(const CAcc& a, const float4*) {
-  return make_double2((double)a.re.hi + (double)a.re.lo, (double)a.im.hi + (double)a.im.lo);
-}
-__device__ __forceinline__ void cacc_add(CAcc& a, const CAcc& b) {
-  a.d.x += b.d.x;
-  a.d.y += b.d.y;
-  dfl s = df_two_sum(a.re.hi, b.re.hi);
-  a.re = dfl{s.hi, s.lo + (a.re.lo + b.re.lo)};
-  s = df_two_sum(a.im.hi, b.im.hi);
-  a.im = dfl{s.hi, s.lo + (a.im.lo + b.im.lo)};
-}
-
-// sum over the 8 lanes of an aligned lane octet (xor 1, 2, 4)
-__device__ __forceinline__ void cacc_reduce8(CAcc& a, const double2*) {
-#pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-    a.d.x += __shfl_xor_sync(0xffffffffu, a.d.x, o);
-    a.d.y += __shfl_xor_sync(0xffffffffu, a.d.y, o);
-  }
-}
-__device__ __forceinline__ void cacc_reduce8(CAcc& a, const float4*) {
-#pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-    CAcc b;
-    b.d = make_double2(0.0, 0.0);
-    b.re.hi = __shfl_xor_sync(0xffffffffu, a.re.hi, o);
-    b.re.lo = __shfl_xor_sync(0xffffffffu, a.re.lo, o);
-    b.im.hi = __shfl_xor_sync(0xffffffffu, a.im.hi, o);
-    b.im.lo = __shfl_xor_sync(0xffffffffu, a.im.lo, o);
-    cacc_add(a, b);
-  }
-}
-
-// The inverse diagonal block times a block of the right-hand side, y = Linv rk
-// or (herm) Linv^H rk, into out; 256 threads.  Float64 blocks (the float64 path
-// and the posterior mean): one thread per row, the loads unrolled ahead of the
-// chain of float64 products.
-__device__ __forceinline__ void diag_apply(const double2* __restrict__ li, const double2* rk, const dfl*, const dfl*,
-                                           CAcc*, double2* out, bool herm) {
-  const int t = threadIdx.x;
-  if (t >= BEOR_TB) return;
-  double sr = 0.0, si = 0.0;
-  const int m0 = herm ? t : 0, m1 = herm ? BEOR_TB - 1 : t;
-  constexpr int U = 8;
-  double2 a[U];
-#pragma unroll
-  for (int u = 0; u < U; ++u) a[u] = li[herm ? pk(min(m0 + u, m1), t) : pk(t, min(m0 + u, m1))];
-  for (int m = m0; m <= m1; m += U) {
-    double2 n[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) n[u] = li[herm ? pk(min(m + U + u, m1), t) : pk(t, min(m + U + u, m1))];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (m + u > m1) break;
-      const double2 q = rk[m + u];
-      const double ai = herm ? -a[u].y : a[u].y;
-      sr = fma(a[u].x, q.x, fma(-ai, q.y, sr));
-      si = fma(a[u].x, q.y, fma(ai, q.x, si));
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) a[u] = n[u];
-  }
-  out[t] = make_double2(sr, si);
-}
-// Double-float blocks (lnL on the mixed path): compensated products on the fp32
-// pipe, as for the off-diagonal tiles.  33,000 float64 products of one block
-// take 10 us on one SM, and as a chain per row with uncoalesced loads they took
-// 40 us of a step; eight lanes per row (forward) or two threads per column
-// (backward) read the block coalesced.
-__device__ __forceinline__ void diag_apply(const float4* __restrict__ li, const double2*, const dfl* rkr,
-                                           const dfl* rki, CAcc* part, double2* out, bool herm) {
-  const int tid = threadIdx.x;
-  if (!herm) {
-    const int lane8 = tid & 7;
-    for (int t = tid >> 3; t < BEOR_TB; t += 32) {
-      CAcc a;
-      cacc_zero(a);
-#pragma unroll 4
-      for (int m = lane8; m <= t; m += 8)
-        cacc_mac(a, li + pk(t, m), make_double2(0.0, 0.0), rkr[m], rki[m], false);
-      cacc_reduce8(a, li);
-      if (lane8 == 0) out[t] = cacc_get(a, li);
-    }
-  } else {
-    const int t = tid & 127, half = tid >> 7;
-    CAcc a;
-    cacc_zero(a);
-#pragma unroll 4
-    for (int m = t + half; m < BEOR_TB; m += 2)
-      cacc_mac(a, li + pk(m, t), make_double2(0.0, 0.0), rkr[m], rki[m], true);
-    if (half) part[t] = a;
-    __syncthreads();
-    if (!half) {
-      cacc_add(a, part[t]);
-      out[t] = cacc_get(a, li);
-    }
-  }
-}
-
-// Forward step k (k = -1: only y_0).  CTA (i, p), i = k+1 .. nt-1:
-// r_i -= L_ik y_k; the CTA with i == k+1 then sets y_{k+1} = Linv r_{k+1}.
-// DV: element type of the inverse diagonal blocks.
-template <typename WS, typename DV>
-__global__ void __launch_bounds__(256) fwd_step_kernel(BatchView v, int kg, const double2* __restrict__ rhs) {
-  __shared__ double2 yk[BEOR_TB];
-  __shared__ dfl ykr[BEOR_TB], yki[BEOR_TB];
-  __shared__ CAcc part[BEOR_TB];
-  __shared__ double2 rk[BEOR_TB];
-  __shared__ dfl rkr[BEOR_TB], rki[BEOR_TB];
-  auto set_rk = [&](int t, double2 q) {
-    rk[t] = q;
-    if (std::is_same<DV, float4>::value) {
-      rkr[t] = df_from_double(q.x);
-      rki[t] = df_from_double(q.y);
-    }
-  };
-  const int p = blockIdx.y;
-  const Prob pr = v.prob[p];
-  const int k = kg - pr.k_off;   // this problem's step (-1: start)
-  if (k < -1) return;
-  const int i = k + 1 + blockIdx.x;
-  if (i >= pr.nt || prob_skipped(v.status[p])) return;
-  if (!BEOR_INBOUNDS(v.flags, pr.row_off + (int64_t)pr.nt * BEOR_TB <= v.rows, BC_SOLVE_VEC) ||
-      !BEOR_INBOUNDS(v.flags, k < 0 || pr.ws_off + (tri_index(i, k) + 1) * BEOR_TILE_ELEMS <= v.ws_elems, BC_SOLVE_VEC))
-    return;
-  const int tid = threadIdx.x;
-  double2* r = v.vec_t + pr.row_off;
-  double2* y = v.vec_y + pr.row_off;
-  if (k < 0) {
-    // initial step: r = rhs for all rows of block 0 handled here, other rows by their own CTAs
-    if (tid < BEOR_TB) r[i * BEOR_TB + tid] = rhs[pr.row_off + i * BEOR_TB + tid];
-    if (i != 0) return;
-    __syncthreads();
-    if (tid < BEOR_TB) set_rk(tid, r[tid]);
-    __syncthreads();
-    diag_apply(reinterpret_cast<const DV*>(v.dinv) + pr.dinv_off, rk, rkr, rki, part, yk, false);
-    __syncthreads();
-    if (tid < BEOR_TB) y[tid] = yk[tid];
-    return;
-  }
-  if (tid < BEOR_TB) {
-    const double2 q = y[k * BEOR_TB + tid];
-    yk[tid] = q;
-    ykr[tid] = df_from_double(q.x);
-    yki[tid] = df_from_double(q.y);
-  }
-  __syncthreads();
-  const WS* t = reinterpret_cast<const WS*>(v.ws) + pr.ws_off + tri_index(i, k) * BEOR_TILE_ELEMS;
-  const int row = tid & 127, half = tid >> 7;
-  CAcc a;
-  cacc_zero(a);
-#pragma unroll 4
-  for (int m = half * 64; m < half * 64 + 64; ++m)
-    cacc_mac(a, t + m * BEOR_TB + row, yk[m], ykr[m], yki[m], false);
-  if (half) part[row] = a;
-  __syncthreads();
-  if (!half) {
-    cacc_add(a, part[row]);
-    const double2 s = cacc_get(a, t);
-    double2 cur = r[i * BEOR_TB + row];
-    cur.x -= s.x;
-    cur.y -= s.y;
-    r[i * BEOR_TB + row] = cur;
-    if (i == k + 1) set_rk(row, cur);
-  }
-  if (i != k + 1) return;
-  __syncthreads();
-  diag_apply(reinterpret_cast<const DV*>(v.dinv) + pr.dinv_off + (int64_t)i * DG_PACK, rk, rkr, rki, part, yk, false);
-  __syncthreads();
-  if (tid < BEOR_TB) y[i * BEOR_TB + tid] = yk[tid];
-}
-
-// Backward step k (k = nt: only x_{nt-1} for each problem).  CTA (i, p),
-// i = 0 .. k-1: r_i -= L_ki^H x_k; the CTA with i == k-1 then sets
-// x_{k-1} = Linv^H r_{k-1}.  Steps run from the largest nt down; problems
-// with fewer tiles join when k < their nt.
-template <typename WS, typename DV>
-__global__ void __launch_bounds__(256) bwd_step_kernel(BatchView v, int k, double2* __restrict__ out) {
-  __shared__ double2 xk[BEOR_TB];
-  __shared__ dfl xkr[BEOR_TB], xki[BEOR_TB];
-  __shared__ double2 rk[BEOR_TB];
-  __shared__ dfl rkr[BEOR_TB], rki[BEOR_TB];
-  __shared__ CAcc part[BEOR_TB];
-  auto set_rk = [&](int t, double2 q) {
-    rk[t] = q;
-    if (std::is_same<DV, float4>::value) {
-      rkr[t] = df_from_double(q.x);
-      rki[t] = df_from_double(q.y);
-    }
-  };
-  const int p = blockIdx.y;
-  const Prob pr = v.prob[p];
-  if (prob_skipped(v.status[p])) return;
-  if (!BEOR_INBOUNDS(v.flags, pr.row_off + (int64_t)pr.nt * BEOR_TB <= v.rows, BC_SOLVE_VEC)) return;
-  const int tid = threadIdx.x;
-  double2* r = v.vec_t + pr.row_off;
-  double2* x = out + pr.row_off;
-  const double2* y = v.vec_y + pr.row_off;
-  if (k >= pr.nt) {
-    // start: r = y; the CTA for the last block applies Linv^H
-    const int i = blockIdx.x;
-    if (i >= pr.nt) return;
-    if (tid < BEOR_TB) r[i * BEOR_TB + tid] = y[i * BEOR_TB + tid];
-    if (k != pr.nt || i != pr.nt - 1) return;
-    __syncthreads();
-    if (tid < BEOR_TB) set_rk(tid, r[i * BEOR_TB + tid]);
-    __syncthreads();
-    diag_apply(reinterpret_cast<const DV*>(v.dinv) + pr.dinv_off + (int64_t)i * DG_PACK, rk, rkr, rki, part, xk, true);
-    __syncthreads();
-    if (tid < BEOR_TB) x[i * BEOR_TB + tid] = xk[tid];
-    return;
-  }
-  const int i = blockIdx.x;
-  if (i >= k) return;
-  if (tid < BEOR_TB) {
-    const double2 q = x[k * BEOR_TB + tid];
-    xk[tid] = q;
-    xkr[tid] = df_from_double(q.x);
-    xki[tid] = df_from_double(q.y);
-  }
-  __syncthreads();
-  // r_i[c] -= sum_m conj(L_ki[m][c]) x_k[m]: tile (k, i) is column-major, so
-  // column c is 128 contiguous elements.  A warp takes 4 columns at a time,
-  // 8 lanes per column on interleaved m (each load instruction reads four
-  // 128-byte segments), and sums the 8 partials by shuffles.
-  const WS* t = reinterpret_cast<const WS*>(v.ws) + pr.ws_off + tri_index(k, i) * BEOR_TILE_ELEMS;
-  const int warp = tid >> 5, lane = tid & 31, cl = lane >> 3, mo = lane & 7;
-#pragma unroll 1
-  for (int it = 0; it < 4; ++it) {
-    const int c = warp * 16 + it * 4 + cl;
-    CAcc a;
-    cacc_zero(a);
-#pragma unroll 4
-    for (int u = 0; u < 16; ++u) {
-      const int m = mo + 8 * u;
-      cacc_mac(a, t + c * BEOR_TB + m, xk[m], xkr[m], xki[m], true);
-    }
-    cacc_reduce8(a, t);
-    if (mo == 0) {
-      const double2 sv = cacc_get(a, t);
-      double2 cur = r[i * BEOR_TB + c];
-      cur.x -= sv.x;
-      cur.y -= sv.y;
-      r[i * BEOR_TB + c] = cur;
-      if (i == k - 1) set_rk(c, cur);
-    }
-  }
-  if (i != k - 1) return;
-  __syncthreads();
-  diag_apply(reinterpret_cast<const DV*>(v.dinv) + pr.dinv_off + (int64_t)i * DG_PACK, rk, rkr, rki, part, xk, true);
-  __syncthreads();
-  if (tid < BEOR_TB) x[i * BEOR_TB + tid] = xk[tid];
-}
-
-
-// Forward step k of y = L^-1 rhs (k = -1: r = rhs and y_0), every problem.
-cudaError_t launch_fwd_step(const BatchView& v, bool mixed, const double2* rhs, int k, cudaStream_t s, int prio) {
-  const int nb = k < 0 ? v.max_nt : v.max_nt - k - 1;
-  if (nb <= 0) return cudaSuccess;
-  auto kern = !mixed ? fwd_step_kernel<double2, double2>
-                     : v.mean ? fwd_step_kernel<float4, double2> : fwd_step_kernel<float4, float4>;
-  return launch_prio(kern, dim3(nb, v.P), dim3(256), 0, s, prio, v, k, rhs);
-}
-
-// out = L^-H y (y in vec_y), every problem.
-template <typename WS, typename DV>
-static cudaError_t bwd_impl(const BatchView& v, double2* out, cudaStream_t s) {
-  const int nt = v.max_nt;
-  bwd_step_kernel<WS, DV><<<dim3(nt, v.P), 256, 0, s>>>(v, nt, out);
-  for (int k = nt - 1; k >= 1; --k) {
-    // problems whose last block is k-1 (nt_p == k) start here
-    bwd_step_kernel<WS, DV><<<dim3(k, v.P), 256, 0, s>>>(v, k, out);
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_bwd(const BatchView& v, bool mixed, double2* out, cudaStream_t s) {
-  if (!mixed) return bwd_impl<double2, double2>(v, out, s);
-  return v.mean ? bwd_impl<float4, double2>(v, out, s) : bwd_impl<float4, float4>(v, out, s);
-}
-
-cudaError_t launch_solve_fwd(const BatchView& v, bool mixed, const double2* rhs, cudaStream_t s) {
-  cudaError_t e = cudaSuccess;
-  for (int k = -1; k + 1 < v.max_nt && e == cudaSuccess; ++k) e = launch_fwd_step(v, mixed, rhs, k, s, 0);
-  return e;
-}
-
-cudaError_t launch_solve(const BatchView& v, bool mixed, const double2* rhs, double2* out, cudaStream_t s) {
-  cudaError_t e = launch_solve_fwd(v, mixed, rhs, s);
-  return e == cudaSuccess ? launch_bwd(v, mixed, out, s) : e;
-}
-
-int solve_launch_count(int max_nt) { return 2 * max_nt; }
-
-// --------------------------------------------------------------------------
 // dbar of each problem's set into the right-hand-side vector
 // --------------------------------------------------------------------------
 __global__ void copy_dbar_kernel(BatchView v) {
