@@ -503,20 +503,19 @@ __global__ void __launch_bounds__(MX_THREADS, 1)
 // slicing of the panel rows: rows of tiles (i, k), i > k, of every problem
 // ---------------------------------------------------------------------------
 constexpr int SL_R = 16;                                    // rows per group
-constexpr int SL_GROUPS = 4;                                // groups per CTA (half a block row)
-constexpr int SL_CTAS = BEOR_TB / (SL_R * SL_GROUPS);       // CTAs per block row
 constexpr int SL_BUF = BEOR_TB * (SL_R + 1);                // float4 per buffer: [column][row], padded
-constexpr int SL_SMEM = 2 * SL_BUF * (int)sizeof(float4);   // double buffer: 69632 bytes
 
 __device__ __forceinline__ void cp_async16(float4* dst, const float4* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
-// Two CTAs per block row i of every problem, each taking four groups of 16
-// rows in turn: the next group's double-float rows are copied into shared
+// CTAs of SL_GROUPS groups of 16 rows in turn (two or eight per block row i of
+// every problem): the next group's double-float rows are copied into shared
 // memory (cp.async) while the current group is sliced.
+template <int SL_GROUPS>
 __global__ void __launch_bounds__(256)
     slice_panel_kernel(BatchView v, int kg, __nv_bfloat16* __restrict__ panel_sl, int32_t* __restrict__ panel_exp) {
+  constexpr int SL_CTAS = BEOR_TB / (SL_R * SL_GROUPS);   // CTAs per block row
   extern __shared__ float4 sl_smem[];
   __shared__ int s_e[SL_R];
   const int p = blockIdx.y;
@@ -616,21 +615,33 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+static int num_sms();
 static __nv_bfloat16* slice_buf(const BatchView& v, int k) {
   return v.panel_sl + (size_t)(k & 1) * BEOR_NPLANE * v.rows * BEOR_TB;
 }
 static int32_t* exp_buf(const BatchView& v, int k) { return v.panel_exp + (size_t)(k & 1) * v.rows; }
 
-cudaError_t launch_slice_panel(const BatchView& v, int k, cudaStream_t s, int prio) {
-  const int nblk = SL_CTAS * (v.max_nt - 1 - k);   // block rows below block column k
-  if (nblk <= 0) return cudaSuccess;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(slice_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SL_SMEM);
-    attr = true;
-  }
-  return launch_prio(slice_panel_kernel, dim3(nblk, v.P), dim3(256), (size_t)SL_SMEM, s, prio, v, k,
+template <int SL_GROUPS>
+static cudaError_t launch_slice(const BatchView& v, int k, cudaStream_t s, int prio) {
+  constexpr int smem = (SL_GROUPS > 1 ? 2 : 1) * SL_BUF * (int)sizeof(float4);   // one group, or two in turn
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(slice_panel_kernel<SL_GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (attr != cudaSuccess) return attr;
+  const int nblk = BEOR_TB / (SL_R * SL_GROUPS) * (v.max_nt - 1 - k);   // CTAs of the block rows below block column k
+  return launch_prio(slice_panel_kernel<SL_GROUPS>, dim3(nblk, v.P), dim3(256), (size_t)smem, s, prio, v, k,
                      slice_buf(v, k), exp_buf(v, k));
+}
+cudaError_t launch_slice_panel(const BatchView& v, int k, cudaStream_t s, int prio) {
+  if (k + 1 >= v.max_nt) return cudaSuccess;
+  // One group of rows per CTA while the step has few of them: the launch is then
+  // a chain of loads and digits (10.7 us for 25 block rows, 21 with four groups
+  // in turn).  Many groups go four to a CTA, whose loads run ahead of its digits
+  // and which take fewer of the resident CTAs of the trailing update's time.
+  // lnL of 3280 modes in ms (one / four): 1 point 7.06 / 7.55, 8 points 11.05 /
+  // 11.26, 12 points 14.28 / 14.28, 32 points 27.9 / 27.2; 700 modes, 32 points
+  // 2.30 / 2.33.
+  return (int64_t)(BEOR_TB / SL_R) * (v.max_nt - 1 - k) * v.P <= 12 * num_sms() ? launch_slice<1>(v, k, s, prio)
+                                                                                  : launch_slice<4>(v, k, s, prio);
 }
 
 // ---------------------------------------------------------------------------
