@@ -33,7 +33,7 @@
 //    scaled per column, the 21 pairs s + t <= 5: 2^-51) into double-float
 //    elements; column j of Linv~ takes the storage that column j of the block
 //    no longer needs.
-//  * Four warps update and factor the next panel's diagonal while the others
+//  * Eight warps update and factor the next panel's diagonal while the others
 //    do the rest of the rank-16 update.  The panel loops are kept rolled: a
 //    warp alone runs straight-line code at the rate of instruction fetches
 //    (6-8 cycles per instruction when they were unrolled).
@@ -43,10 +43,10 @@
 //    per panel.
 //
 // Measured per launch (3280 modes): 0.79 ms before (float64 factor, fp32
-// inverse), now 0.205 ms with one problem (clusters of four) and 0.23 ms with
-// 64 (clusters of two).  In a cluster of four, of 408,000 cycles: 160,000 the
-// chain of 128 columns in the panel factors, 150,000 the substitutions, 55,000
-// updates and barriers, 25,000 loading and output.
+// inverse), now 0.185 ms with one problem (clusters of four), 0.225 ms with 64
+// (clusters of two) and 0.295 ms with 100 (single CTAs).  Most of it is the
+// chain of 128 columns in the panel factors and, between them, the
+// substitutions; loading and output take 13 us.
 //
 // tcgen05 is not used: its smallest tile (M = 64 or 128 of one CTA, operands
 // by descriptor, accumulators in tensor memory) does not fit a triangle of
@@ -275,39 +275,32 @@ __device__ __forceinline__ void dt_sync() {
     cg::this_cluster().sync();
 }
 
-// Factor of the 16 x 16 diagonal block of panel pan by four warps of its
-// owner: thread = (row r, columns c0 and c0 + 8).  Square-root-free
+// Factor of the 16 x 16 diagonal block of panel pan by eight warps of its
+// owner: thread = element (row r, column c); a warp's rows are consecutive, so
+// that finished rows cost nothing.  Square-root-free
 // elimination, a_rc -= z~_r conj(z~_c) / D, so that only a reciprocal lies
 // between two pivots (beside the products, which do not need it), and every
 // thread forms the next pivot itself: one barrier per column.  The square
 // roots follow for all columns at once.  The factor goes to every CTA.
-constexpr int DT_FW = 4;   // warps
+constexpr int DT_FW = 8;   // warps
 __device__ __forceinline__ void dt_fsync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * DT_FW) : "memory"); }
 template <int C>
 __device__ __forceinline__ void dt_factor(DtSmem& sm, float4* __restrict__ ws, int pan, int tid) {
-  const int s0 = pan * DT_P, r = tid >> 3, c0 = tid & 7;
-  longlong2 x[2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int c = c0 + 8 * h;
-    x[h] = c <= r ? sm.s[pk(s0 + r, s0 + c)] : make_longlong2(0, 0);
-  }
+  const int s0 = pan * DT_P, r = tid >> 4, c = tid & 15;
+  longlong2 x = c <= r ? sm.s[pk(s0 + r, s0 + c)] : make_longlong2(0, 0);
   long long d = sm.s[pk(s0, s0)].x;
 #pragma unroll 1
   for (int j = 0; j < DT_P; ++j) {
     int g;
     const long long D = fx_normalise(d > 0 ? d : FX_ONE / 2, g);
     bool over;
-    const longlong2 z = dt_shift(j < 8 ? x[0] : x[1], g, over);
-    if (c0 == (j & 7) && r > j) {
-      if (j < 8)
-        x[0] = z;
-      else
-        x[1] = z;
+    const longlong2 z = dt_shift(x, g, over);
+    if (c == j && r > j) {
+      x = z;
       sm.zb[j & 1][r] = z;
       if (over) sm.bad[s0 + r] = 1;
     }
-    if (r == j + 1 && c0 == ((j + 1) & 7)) sm.pub[j & 1] = j + 1 < 8 ? x[0].x : x[1].x;
+    if (r == j + 1 && c == j + 1) sm.pub[j & 1] = x.x;
     const fxs w = fx_split(fx_recip(D));
     dt_fsync();
     if (d <= 0 || sm.bad[s0 + j]) {
@@ -319,18 +312,14 @@ __device__ __forceinline__ void dt_factor(DtSmem& sm, float4* __restrict__ ws, i
     const longlong2* zb = sm.zb[j & 1];
     const fxs nx = fx_split(zb[j + 1].x), ny = fx_split(zb[j + 1].y);
     d = sm.pub[j & 1] - fx_mul<2>(fx_dot2(nx, nx, ny, ny), w);
-    const longlong2 zr = zb[r];
-    const fxs ar = fx_split(zr.x), ai = fx_split(zr.y), nr = fx_split(-zr.x);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int c = c0 + 8 * h;
-      if (c > j && c <= r) {
-        const fxs br = fx_split(zb[c].x), bi = fx_split(zb[c].y);
-        const long long re = fx_dot2(ar, br, ai, bi), im = fx_dot2(ai, br, nr, bi);
-        if (c == r && re > D + (1ll << 45)) sm.bad[s0 + r] = 1;   // |L~_rj| > 1
-        x[h].x -= fx_mul<2>(re, w);
-        x[h].y -= fx_mul<2>(im, w);
-      }
+    if (c > j && c <= r) {
+      const longlong2 zr = zb[r];
+      const fxs ar = fx_split(zr.x), ai = fx_split(zr.y), nr = fx_split(-zr.x);
+      const fxs br = fx_split(zb[c].x), bi = fx_split(zb[c].y);
+      const long long re = fx_dot2(ar, br, ai, bi), im = fx_dot2(ai, br, nr, bi);
+      if (c == r && re > D + (1ll << 45)) sm.bad[s0 + r] = 1;   // |L~_rj| > 1
+      x.x -= fx_mul<2>(re, w);
+      x.y -= fx_mul<2>(im, w);
     }
   }
   dt_fsync();   // every pivot is written
@@ -350,12 +339,9 @@ __device__ __forceinline__ void dt_factor(DtSmem& sm, float4* __restrict__ ws, i
   }
   dt_fsync();
   const pow2 pe = make_pow2(sm.es[s0 + r] - FX_FRAC);
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int c = c0 + 8 * h;
-    if (c >= r) continue;
+  if (c < r) {
     const fxs y = fx_split(sm.y[c]);
-    const longlong2 l = make_longlong2(fx_mul<1>(x[h].x, y), fx_mul<1>(x[h].y, y));
+    const longlong2 l = make_longlong2(fx_mul<1>(x.x, y), fx_mul<1>(x.y, y));
     // L~ y, 60 fractional bits: the multipliers of the rows below
     const fxs re = fx_split(fx_mul<0>(l.x, y)), im = fx_split(fx_mul<0>(l.y, y));
     // -L~ as three floats per component, exactly (24, 24 and 14 bits)
@@ -375,12 +361,17 @@ __device__ __forceinline__ void dt_factor(DtSmem& sm, float4* __restrict__ ws, i
   }
 }
 
-// Rows below the panel, 4 C lanes per row (columns q, q + 4 C, ..: more lanes
-// where a CTA has fewer rows): substitution with the panel's factor, digits to
+// Lanes per row of the rows below a panel: more where a CTA has fewer rows,
+// while that shortens the chain (16 lanes with C = 4 took 3 % longer a block).
+template <int C>
+constexpr int dt_lpr() {
+  return C == 1 ? 4 : 8;
+}
+// Rows below the panel, dt_lpr lanes per row (columns q, q + LPR, ..): substitution with the panel's factor, digits to
 // every CTA, L to the workspace.
 template <int C>
 __device__ __forceinline__ void dt_solve(DtSmem& sm, float4* __restrict__ ws, int s0, int row, int lane) {
-  constexpr int LPR = 4 * C, NC = DT_P / LPR;
+  constexpr int LPR = dt_lpr<C>(), NC = DT_P / LPR;
   const int q = lane & (LPR - 1);
   longlong2 x[NC];
   bool bad = sm.bad[row];
@@ -467,24 +458,27 @@ __device__ __forceinline__ void dt_solve(DtSmem& sm, float4* __restrict__ ws, in
   if (q < C) dt_peer<C>(sm, q)->ex[row] = lb - 59;
 }
 
+constexpr int DT_IP = 4;   // lanes per sum
 // The panel's rows of the inverse, column j, component comp (0 re, 1 im; the
-// other component is the neighbouring lane's): Y = L_pp^-1 B, row by row.  A
+// other component is the neighbouring lane's): Y = L_pp^-1 B, row by row, each
+// sum over four lanes (one lane took 18,000 cycles a panel, the longest of the
+// chain).  A
 // CTA that does not own the rows keeps its columns of Y in its own copy too.
 template <int C>
-__device__ __forceinline__ void dt_inverse_rows(DtSmem& sm, int pan, int j, int comp) {
+__device__ __forceinline__ void dt_inverse_rows(DtSmem& sm, int pan, int j, int part, int comp) {
   const int s0 = pan * DT_P, m0 = max(0, j - s0);   // rows above column j are zero
   DtSmem* own = dt_peer<C>(sm, pan % C);            // holds the rows
   const float sg = comp ? 1.0f : -1.0f;
   float mx = 0.0f;
 #pragma unroll 1
   for (int r = 0; r < DT_P; ++r) {
-    dfl c0{j == s0 + r && !comp ? 1.0f : 0.0f, 0.0f}, c1{0.0f, 0.0f};
-    if (j < s0) {
+    dfl c0{j == s0 + r && !comp && !part ? 1.0f : 0.0f, 0.0f}, c1{0.0f, 0.0f};
+    if (j < s0 && !part) {
       const float2 b = reinterpret_cast<const float2*>(&own->s[pk(s0 + r, j)])[comp];
       c0 = dfl{b.x, b.y};
     }
 #pragma unroll 2
-    for (int m = m0; m < r; ++m) {
+    for (int m = m0 + part; m < r; m += DT_IP) {
       const float4 a = sm.lpf[r][m];
       const float2 at = sm.lpt[r][m];
       const float4 y = *reinterpret_cast<const float4*>(&sm.s[pk(s0 + m, j)]);
@@ -492,10 +486,17 @@ __device__ __forceinline__ void dt_inverse_rows(DtSmem& sm, int pan, int j, int 
       dot2_acc3(c0, a.x, a.y, at.x, yh, yl);
       dot2_acc3(c1, sg * a.z, sg * a.w, sg * at.y, zh, zl);
     }
-    const dfl s = df_two_sum(c0.hi, c1.hi);
-    const dfl y = df_mul(df_fast_two_sum(s.hi, s.lo + (c0.lo + c1.lo)), sm.rinvf[r]);
+    dfl s = df_two_sum(c0.hi, c1.hi);
+    s.lo += c0.lo + c1.lo;
+#pragma unroll
+    for (int o = 2; o < 2 * DT_IP; o <<= 1) {   // the same bits in every lane
+      const dfl t{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)};
+      const dfl u = df_two_sum(s.hi, t.hi);
+      s = dfl{u.hi, u.lo + (s.lo + t.lo)};
+    }
+    const dfl y = df_mul(df_fast_two_sum(s.hi, s.lo), sm.rinvf[r]);
     mx = fmaxf(mx, fabsf(y.hi));
-    if (r >= m0) {
+    if (r >= m0 && !part) {
       reinterpret_cast<float2*>(&sm.s[pk(s0 + r, j)])[comp] = make_float2(y.hi, y.lo);
       if (C > 1 && own != &sm) reinterpret_cast<float2*>(&own->s[pk(s0 + r, j)])[comp] = make_float2(y.hi, y.lo);
     }
@@ -505,15 +506,16 @@ __device__ __forceinline__ void dt_inverse_rows(DtSmem& sm, int pan, int j, int 
   const bool zero = !(mx > 0x1p-120f);
   const int eu = zero ? DT_ZERO_E : ilogbf(mx) + 4;   // two powers of two of headroom; hi + lo may round up to one more
   const pow2 ps = zero ? pow2{0.0f, 0.0f} : make_pow2(55 - eu);
-#pragma unroll 1
-  for (int u = 0; u < 2; ++u) {
-    uint32_t dg[4][FX_ND];
+  // digits of the eight pairs of rows, two of them by each lane
+  {
+    const int p0 = part * 2;
+    uint32_t dg[2][FX_ND];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 2; ++q) {
       long long xv[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int r = 8 * u + 2 * q + h;
+        const int r = 2 * (p0 + q) + h;
         const float2 y = r >= m0 ? reinterpret_cast<const float2*>(&sm.s[pk(s0 + r, j)])[comp] : make_float2(0.0f, 0.0f);
         xv[h] = fx_from_scaled(scale2f(y.x, ps), scale2f(y.y, ps));
       }
@@ -521,15 +523,12 @@ __device__ __forceinline__ void dt_inverse_rows(DtSmem& sm, int pan, int j, int 
     }
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      unsigned char* o = dt_peer<C>(sm, c)->dg + dt_off(j, 2 * u + comp);
+      unsigned char* o = dt_peer<C>(sm, c)->dg + dt_off(j, 2 * (p0 >> 2) + comp) + 4 * (p0 & 3);
 #pragma unroll
-      for (int d = 0; d < FX_ND; ++d)
-        *reinterpret_cast<uint4*>(o + d * DT_SLICE) = make_uint4(dg[0][d], dg[1][d], dg[2][d], dg[3][d]);
+      for (int d = 0; d < FX_ND; ++d) *reinterpret_cast<uint2*>(o + d * DT_SLICE) = make_uint2(dg[0][d], dg[1][d]);
     }
   }
-#pragma unroll
-  for (int c = 0; c < C; c += 2)
-    if (c + comp < C) dt_peer<C>(sm, c + comp)->ex[j] = eu;
+  if (2 * part + comp < C) dt_peer<C>(sm, 2 * part + comp)->ex[j] = eu;
 }
 
 template <int C>
@@ -580,17 +579,17 @@ __global__ void __launch_bounds__(DT_THREADS, 1) diag_tc_kernel(BatchView v, int
     const int s0 = pan * DT_P;
     dt_sync<C>();   // the panel's factor, the updated rows
     if (sm.fail) break;
-    // own row blocks below the panel, 2 C warps each; then one warp per 16 columns of the panel's rows of the inverse
+    // own row blocks below the panel, WB warps each; then one warp per four columns of the panel's rows of the inverse
     const int first = pan + 1 + (rank - (pan + 1) % C + C) % C;   // first own block below the panel
     const int nblk = first < DT_NPAN ? (DT_NPAN - 1 - first) / C + 1 : 0;
-    constexpr int WB = 2 * C;   // warps per block of 16 rows
+    constexpr int LPR = dt_lpr<C>(), WB = LPR / 2;   // warps per block of 16 rows
     if (tid == 0) sm.tile = 0;
     if (warp < WB * nblk) {
       const int R = first + (warp / WB) * C;
-      dt_solve<C>(sm, ws, s0, 16 * R + (warp % WB) * (DT_P / WB) + lane / (4 * C), lane);
+      dt_solve<C>(sm, ws, s0, 16 * R + (warp % WB) * (DT_P / WB) + lane / LPR, lane);
     } else {
-      const int b = (warp - WB * nblk) * C + rank;
-      if (b <= pan) dt_inverse_rows<C>(sm, pan, 16 * b + (lane >> 1), lane & 1);
+      for (int w = warp - WB * nblk; w / 4 * C + rank <= pan; w += DT_WARPS - WB * nblk)
+        dt_inverse_rows<C>(sm, pan, 16 * (w / 4 * C + rank) + 4 * (w & 3) + (lane >> 3), (lane >> 1) & 3, lane & 1);
     }
     dt_sync<C>();   // digits and exponents
     if (pan + 1 == DT_NPAN) break;
