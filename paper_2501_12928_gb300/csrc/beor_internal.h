@@ -159,10 +159,10 @@ struct MixedMaps;  // opaque TMA descriptors of one batch
 cudaError_t mixed_maps_create(const BatchView& v, MixedMaps** out);
 void mixed_maps_destroy(MixedMaps* m);
 // Block step k of the mixed factorisation: slicing of the panel column (buffer k % 2),
-// the panel product, and the trailing update, whole or split into the next block
-// column (j = k + 1) and the rest (j >= k + 2) so that step k + 1 can start early.
+// the panel product, and the trailing update, whole or split into the next diagonal
+// block, the tiles below it and the rest (j >= k + 2) so that step k + 1 can start early.
 // prio: launch priority (0: the stream's).
-enum { TRAIL_ALL = 0, TRAIL_NEXT_COL = 1, TRAIL_REST = 2 };
+enum { TRAIL_ALL = 0, TRAIL_NEXT_DIAG = 1, TRAIL_NEXT_BELOW = 2, TRAIL_REST = 3 };
 cudaError_t mixed_reset_counters(const MixedMaps* m, cudaStream_t s);   // before every evaluation
 int64_t mixed_tiles(const MixedMaps* m, int kind, int k);               // kind 0 next col, 1 rest, 2 panel, 3 all
 cudaError_t launch_slice_panel(const BatchView& v, int k, cudaStream_t s, int prio = 0);

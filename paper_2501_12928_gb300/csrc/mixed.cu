@@ -810,21 +810,26 @@ cudaError_t launch_panel_mixed(const BatchView& v, const MixedMaps* m, int k, cu
   return launch_gemm(v, m, k, KIND_PANEL, s, prio);
 }
 
-// The off-diagonal tiles (reduced pair set), then the diagonal ones (full
-// set), on the same stream.
+// Kinds of a part's off-diagonal tiles (reduced pair set) and diagonal ones
+// (full set), -1: none.
+static int part_kind(int part) {
+  return part == TRAIL_NEXT_BELOW ? KIND_COL : part == TRAIL_REST ? KIND_REST : part == TRAIL_ALL ? KIND_ALL : -1;
+}
+static int part_diag(int part) {
+  return part == TRAIL_NEXT_DIAG ? KIND_DCOL : part == TRAIL_REST ? KIND_DREST : part == TRAIL_ALL ? KIND_DALL : -1;
+}
+// Off-diagonal tiles, then the diagonal ones, on the same stream.
 cudaError_t launch_trail_mixed(const BatchView& v, const MixedMaps* m, int k, int part, cudaStream_t s, int prio,
                                int max_ctas) {
-  const int kind = part == TRAIL_NEXT_COL ? KIND_COL : part == TRAIL_REST ? KIND_REST : KIND_ALL;
-  const int diag = part == TRAIL_NEXT_COL ? KIND_DCOL : part == TRAIL_REST ? KIND_DREST : KIND_DALL;
-  cudaError_t e = launch_gemm(v, m, k, kind, s, prio, max_ctas);
-  if (e == cudaSuccess) e = launch_gemm(v, m, k, diag, s, prio, max_ctas);
+  const int kind = part_kind(part), diag = part_diag(part);
+  cudaError_t e = kind >= 0 ? launch_gemm(v, m, k, kind, s, prio, max_ctas) : cudaSuccess;
+  if (e == cudaSuccess && diag >= 0) e = launch_gemm(v, m, k, diag, s, prio, max_ctas);
   return e;
 }
 
 int trail_launch_count(const MixedMaps* m, int k, int part) {
-  const int kind = part == TRAIL_NEXT_COL ? KIND_COL : part == TRAIL_REST ? KIND_REST : KIND_ALL;
-  const int diag = part == TRAIL_NEXT_COL ? KIND_DCOL : part == TRAIL_REST ? KIND_DREST : KIND_DALL;
-  return (mixed_tiles_kind(m, kind, k) > 0) + (mixed_tiles_kind(m, diag, k) > 0);
+  const int kind = part_kind(part), diag = part_diag(part);
+  return (kind >= 0 && mixed_tiles_kind(m, kind, k) > 0) + (diag >= 0 && mixed_tiles_kind(m, diag, k) > 0);
 }
 
 int device_sms() { return num_sms(); }
