@@ -162,9 +162,12 @@ int beor_precompute(beor_ctx *ctx, void *stream);
  * n_model = 3280, 1.07 GB at 11,424) plus bf16 slices and vectors -- and
  * captures its CUDA graph (BEOR_ENOMEM if they do not fit).  Both are kept
  * for later calls of the same shape and released when one of its contexts
- * is re-set (beor_set_T, beor_set_instrument, beor_set_data,
- * beor_precompute) or destroyed, so callers with varying B should use a
- * few sizes (e.g. pad to powers of two).
+ * takes another model (beor_set_T, beor_set_instrument) or is destroyed, so
+ * callers with varying B should use a few sizes (e.g. pad to powers of two).
+ * New data (beor_set_data, beor_precompute) only end the results' validity:
+ * the next call of the shape takes the batch up again.  Such idle batches
+ * hold at most a sixteenth of the device's memory in all, and give it back
+ * when an allocation of the library does not fit otherwise.
  * Mixed precision: the quadratic form q = dbar^H Sigma^-1 dbar is evaluated
  * from the first solution x~ of the approximate factor L~ and one float64
  * residual r = dbar - Sigma x~ as q = dbar^H x~ + x~^H r + |L~^-1 r|^2

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <string>
@@ -47,6 +48,8 @@ cudaError_t from_device(void* dst, const void* src, size_t n, cudaStream_t s) {
   return cudaMemcpyAsync(dst, src, n, is_device_ptr(dst) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
 }
 
+bool release_retired_plans();   // frees their memory; false: there was none
+
 struct DevBuf {
   void* p = nullptr;
   size_t n = 0;
@@ -60,12 +63,44 @@ struct DevBuf {
     release();
     if (bytes == 0) return cudaSuccess;
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && release_retired_plans()) {
+      cudaGetLastError();
+      e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
       p = nullptr;
       return e;
     }
     n = bytes;
     return cudaSuccess;
+  }
+  // as alloc, but a buffer of that size stays (its contents are undefined)
+  cudaError_t ensure(size_t bytes) { return p && n == bytes ? cudaSuccess : alloc(bytes); }
+  template <typename T>
+  T* as() const { return reinterpret_cast<T*>(p); }
+};
+
+// Host memory for small copies, page-locked where that succeeds (a pageable
+// copy takes 15 us more).
+struct HostBuf {
+  void* p = nullptr;
+  bool pinned = false;
+  HostBuf() = default;
+  HostBuf(const HostBuf&) = delete;
+  HostBuf& operator=(const HostBuf&) = delete;
+  ~HostBuf() {
+    if (pinned)
+      cudaFreeHost(p);
+    else
+      std::free(p);
+  }
+  bool alloc(size_t bytes) {   // once
+    pinned = cudaHostAlloc(&p, bytes, cudaHostAllocDefault) == cudaSuccess;
+    if (!pinned) {
+      cudaGetLastError();
+      p = std::malloc(bytes);
+    }
+    return p != nullptr;
   }
   template <typename T>
   T* as() const { return reinterpret_cast<T*>(p); }
@@ -102,7 +137,7 @@ struct beor_ctx {
 
 namespace {
 
-std::mutex g_mu;
+std::recursive_mutex g_mu;   // an allocation under it may release retired plans
 std::vector<Plan*> g_plans;
 
 struct Plan {
@@ -115,7 +150,7 @@ struct Plan {
   std::vector<Prob> h_prob;
   std::vector<SetDesc> h_sets;
   std::vector<int> first;   // first problem index of each set
-  DevBuf d_prob, d_sets, ws, dinv, phi_inv, vecs, scal, flags, phis, panel_sl, panel_exp, linv_sl, linv_exp;
+  DevBuf d_prob, d_sets, ws, dinv, phi_inv, vecs, scal, phis, panel_sl, panel_exp, linv_sl, linv_exp;
   DevBuf xtr, rwork, rpart;         // float32-pipe residual: x triples, work items, partial sums
   int n_rwork = 0, rcols = 0, rgroup = 0;
   std::vector<int64_t> phi_off;
@@ -124,6 +159,9 @@ struct Plan {
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
   int64_t launches = 0;
+  bool retired = false;             // its data set was replaced; the next call of its shape takes it up again
+  HostBuf h_phi, h_out;             // phi of host callers; the results, read by one copy
+  size_t out_off = 0, out_bytes = 0, status_off = 0, flags_off = 0;   // in scal (bytes); out: from lnl to the flags
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   bool prof = false;
   bool refine_x = false;            // mixed: refine the solution (posterior mean) rather than correct q
@@ -430,8 +468,13 @@ int build_plan(beor_ctx* const* ctxs, int nsets, const int* Bs, bool need_x, int
   chk(pl->dinv.alloc(sizeof(double2) * (size_t)dinv_elems));
   chk(pl->phi_inv.alloc(sizeof(double) * (size_t)rows));
   chk(pl->vecs.alloc(sizeof(double2) * (size_t)rows * 6));
-  chk(pl->scal.alloc(sizeof(double) * (size_t)pl->P * 6 + sizeof(int32_t) * pl->P));
-  chk(pl->flags.alloc(sizeof(Flags)));
+  pl->out_off = sizeof(double) * (size_t)pl->P * 3;
+  pl->status_off = sizeof(double) * (size_t)pl->P * 6;
+  pl->flags_off = (pl->status_off + sizeof(int32_t) * (size_t)pl->P + 15) & ~(size_t)15;
+  pl->out_bytes = pl->flags_off + sizeof(Flags) - pl->out_off;
+  chk(pl->scal.alloc(pl->flags_off + sizeof(Flags)));
+  if (!pl->h_phi.alloc(sizeof(double) * std::max<int64_t>(1, phi_total)) || !pl->h_out.alloc(pl->out_bytes))
+    chk(cudaErrorMemoryAllocation);
   if (pl->mixed) {
     chk(pl->panel_sl.alloc(sizeof(__nv_bfloat16) * 2 * (size_t)BEOR_NPLANE * rows * BEOR_TB));
     chk(pl->panel_exp.alloc(sizeof(int32_t) * 2 * (size_t)rows));
@@ -477,7 +520,7 @@ int build_plan(beor_ctx* const* ctxs, int nsets, const int* Bs, bool need_x, int
   }
   chk(cudaMemcpy(pl->d_prob.p, pl->h_prob.data(), sizeof(Prob) * pl->P, cudaMemcpyHostToDevice));
   chk(cudaMemcpy(pl->d_sets.p, pl->h_sets.data(), sizeof(SetDesc) * nsets, cudaMemcpyHostToDevice));
-  chk(cudaMemset(pl->flags.p, 0, sizeof(Flags)));
+  chk(cudaMemset(pl->scal.as<char>() + pl->flags_off, 0, sizeof(Flags)));
   BatchView& v = pl->view;
   v.P = pl->P;
   v.nsets = nsets;
@@ -500,8 +543,8 @@ int build_plan(beor_ctx* const* ctxs, int nsets, const int* Bs, bool need_x, int
   v.q = sc + 2 * pl->P;
   v.lnl = sc + 3 * pl->P;
   v.resid = sc + 4 * pl->P;
-  v.status = reinterpret_cast<int32_t*>(sc + 6 * pl->P);
-  v.flags = pl->flags.as<Flags>();
+  v.status = reinterpret_cast<int32_t*>(pl->scal.as<char>() + pl->status_off);
+  v.flags = reinterpret_cast<Flags*>(pl->scal.as<char>() + pl->flags_off);
   v.panel_sl = pl->panel_sl.as<__nv_bfloat16>();
   v.panel_exp = pl->panel_exp.as<int32_t>();
   v.linv_sl = pl->linv_sl.as<__nv_bfloat16>();
@@ -572,7 +615,7 @@ void drop_plans_with_stale_schedule() {
 }
 
 void drop_plans_of(beor_ctx* c) {
-  std::lock_guard<std::mutex> lk(g_mu);
+  std::lock_guard<std::recursive_mutex> lk(g_mu);
   std::vector<Plan*> keep;
   for (Plan* p : g_plans) {
     if (std::find(p->ctxs.begin(), p->ctxs.end(), c) != p->ctxs.end()) {
@@ -587,6 +630,89 @@ void drop_plans_of(beor_ctx* c) {
     }
   }
   g_plans.swap(keep);
+}
+
+// Plans of a context whose data set is about to change: nothing may read their
+// results any more, but buffers and graph stay for the next call of the shape
+// (building them again took 4 of the 28 ms of a data set of 3280 modes with 16
+// points).  They hold a sixteenth of the device's memory at most; an allocation
+// that fails releases them.
+void retire_plans_of(beor_ctx* c) {
+  std::lock_guard<std::recursive_mutex> lk(g_mu);
+  static const size_t limit = [] {
+    size_t avail = 0, total = 0;
+    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
+      cudaGetLastError();
+      total = 0;
+    }
+    return total / 16;
+  }();
+  auto bytes = [](const Plan* p) {
+    size_t n = 0;
+    for (const DevBuf* b : {&p->d_prob, &p->d_sets, &p->ws, &p->dinv, &p->phi_inv, &p->vecs, &p->scal, &p->phis, &p->panel_sl,
+                            &p->panel_exp, &p->linv_sl, &p->linv_exp, &p->xtr, &p->rwork, &p->rpart})
+      n += b->n;
+    return n;
+  };
+  size_t held = 0;
+  for (const Plan* p : g_plans)
+    if (p->retired) held += bytes(p);
+  bool synced = false;
+  std::vector<Plan*> keep;
+  for (Plan* p : g_plans) {
+    if (p->retired || std::find(p->ctxs.begin(), p->ctxs.end(), c) == p->ctxs.end()) {
+      keep.push_back(p);
+      continue;
+    }
+    if (!synced) {   // no evaluation of the plan may still be running
+      cudaDeviceSynchronize();
+      synced = true;
+    }
+    for (beor_ctx* o : p->ctxs)
+      if (o->last_plan == p) o->last_plan = nullptr;
+    p->retired = true;
+    held += bytes(p);
+    if (held <= limit) {
+      keep.push_back(p);
+    } else {
+      held -= bytes(p);
+      delete p;
+    }
+  }
+  g_plans.swap(keep);
+}
+
+bool release_retired_plans() {
+  std::lock_guard<std::recursive_mutex> lk(g_mu);
+  std::vector<Plan*> keep;
+  for (Plan* p : g_plans) {
+    if (p->retired)
+      delete p;
+    else
+      keep.push_back(p);
+  }
+  const bool any = keep.size() < g_plans.size();
+  g_plans.swap(keep);
+  return any;
+}
+
+// The set descriptors follow the contexts' buffers when a retired plan is
+// taken up again (the graph reads them from device memory).
+cudaError_t refresh_sets(Plan& pl) {
+  bool changed = false;
+  for (size_t s = 0; s < pl.ctxs.size(); ++s) {
+    const beor_ctx* c = pl.ctxs[s];
+    SetDesc sd = pl.h_sets[s];
+    sd.M = c->M.as<double2>();
+    sd.Mdf = c->Mdf.as<float4>();
+    sd.Mf = c->Mf.as<float4>();
+    sd.Mft = c->Mft.as<float2>();
+    sd.dbar = c->dbar.as<double2>();
+    changed = changed || std::memcmp(&sd, &pl.h_sets[s], sizeof(sd)) != 0;
+    pl.h_sets[s] = sd;
+  }
+  return changed ? cudaMemcpy(pl.d_sets.p, pl.h_sets.data(), sizeof(SetDesc) * pl.h_sets.size(), cudaMemcpyHostToDevice)
+                 : cudaSuccess;
 }
 
 int check_ready(const beor_ctx* c) {
@@ -759,14 +885,14 @@ int beor_set_data(beor_ctx* c, const beor_c128* d, const double* noise_var) {
   for (double x : nv)
     if (!(x > 0.0) || !std::isfinite(x)) return BEOR_EINVAL;
   for (double& x : nv) x = 1.0 / x;
-  CKC(c, c->w.alloc(sizeof(double) * c->n_vis));
+  CKC(c, c->w.ensure(sizeof(double) * c->n_vis));
   CKC(c, cudaMemcpy(c->w.p, nv.data(), sizeof(double) * c->n_vis, cudaMemcpyHostToDevice));
-  CKC(c, c->d.alloc(sizeof(double2) * c->n_vis));
+  CKC(c, c->d.ensure(sizeof(double2) * c->n_vis));
   CKC(c, to_device(c->d.p, d, sizeof(double2) * c->n_vis, 0));
   CKC(c, cudaDeviceSynchronize());
   c->have_data = true;
   c->have_pre = false;
-  drop_plans_of(c);
+  retire_plans_of(c);
   return BEOR_OK;
 }
 
@@ -776,9 +902,9 @@ int beor_precompute(beor_ctx* c, void* stream) {
   if (!c->have_data) return BEOR_ESTATE;
   cudaSetDevice(c->device);
   cudaStream_t s = (cudaStream_t)stream;
-  drop_plans_of(c);
-  CKC(c, c->M.alloc(sizeof(double2) * (size_t)tri_count(c->nt) * BEOR_TILE_ELEMS));
-  CKC(c, c->dbar.alloc(sizeof(double2) * (size_t)c->nt * BEOR_TB));
+  retire_plans_of(c);
+  CKC(c, c->M.ensure(sizeof(double2) * (size_t)tri_count(c->nt) * BEOR_TILE_ELEMS));
+  CKC(c, c->dbar.ensure(sizeof(double2) * (size_t)c->nt * BEOR_TB));
   if (c->model_kind == 1) {
     CKC(c, precompute_dense(c->T.as<double2>(), c->n_vis, c->n, c->ld, c->w.as<double>(), c->d.as<double2>(), c->nt,
                             c->M.as<double2>(), c->dbar.as<double2>(), s, c->precision == BEOR_PREC_MIXED));
@@ -793,11 +919,11 @@ int beor_precompute(beor_ctx* c, void* stream) {
   }
   if (c->precision == BEOR_PREC_MIXED) {
     const int64_t ne = tri_count(c->nt) * BEOR_TILE_ELEMS;
-    CKC(c, c->Mdf.alloc(sizeof(float4) * (size_t)ne));
+    CKC(c, c->Mdf.ensure(sizeof(float4) * (size_t)ne));
     CKC(c, split_double_float(c->M.as<double2>(), ne, c->Mdf.as<float4>(), s));
     const int64_t nf = (int64_t)c->nt * c->nt * BEOR_TILE_ELEMS;
-    CKC(c, c->Mf.alloc(sizeof(float4) * (size_t)nf));
-    CKC(c, c->Mft.alloc(sizeof(float2) * (size_t)nf));
+    CKC(c, c->Mf.ensure(sizeof(float4) * (size_t)nf));
+    CKC(c, c->Mft.ensure(sizeof(float2) * (size_t)nf));
     CKC(c, split_full_triple(c->M.as<double2>(), c->n, c->nt, c->Mf.as<float4>(), c->Mft.as<float2>(), s));
   }
   CKC(c, cudaStreamSynchronize(s));
@@ -826,7 +952,7 @@ static int lnl_multi_impl(beor_ctx* const* ctxs, int nsets, const double* const*
   beor_ctx* c0 = ctxs[0];
   cudaSetDevice(c0->device);
   cudaStream_t st = (cudaStream_t)stream;
-  std::lock_guard<std::mutex> lk(g_mu);
+  std::lock_guard<std::recursive_mutex> lk(g_mu);
   need_x = need_x && ctxs[0]->precision == BEOR_PREC_MIXED;
   Plan* pl = find_plan(ctxs, nsets, B, need_x, slot);
   if (!pl) {
@@ -834,16 +960,35 @@ static int lnl_multi_impl(beor_ctx* const* ctxs, int nsets, const double* const*
     if (r) return r;
     g_plans.push_back(pl);
   }
-  for (int s = 0; s < nsets; ++s) {
-    // validate phi values (finite) on the host when possible
-    size_t bytes = sizeof(double) * (size_t)B[s] * ctxs[s]->n_k;
-    if (!is_device_ptr(phi[s])) {
-      for (size_t i = 0; i < (size_t)B[s] * ctxs[s]->n_k; ++i)
-        if (!std::isfinite(phi[s][i])) return BEOR_EINVAL;
-    }
-    CKC(c0, to_device(pl->phis.as<double>() + pl->phi_off[s], phi[s], bytes, st));
+  const bool first_use = !pl->exec || pl->retired;
+  if (pl->retired) {
+    CKC(c0, refresh_sets(*pl));
+    pl->retired = false;
   }
-  const bool first_use = !pl->exec;
+  size_t on_host = 0, phi_end = 0;   // sets, values
+  for (int s = 0; s < nsets; ++s) {
+    const size_t off = (size_t)pl->phi_off[s], cnt = (size_t)B[s] * ctxs[s]->n_k;
+    phi_end = off + cnt;
+    if (is_device_ptr(phi[s])) {
+      CKC(c0, cudaMemcpyAsync(pl->phis.as<double>() + off, phi[s], sizeof(double) * cnt, cudaMemcpyDeviceToDevice, st));
+      continue;
+    }
+    // validate phi values (finite) on the host when possible
+    for (size_t i = 0; i < cnt; ++i)
+      if (!std::isfinite(phi[s][i])) return BEOR_EINVAL;
+    std::memcpy(pl->h_phi.as<double>() + off, phi[s], sizeof(double) * cnt);
+    ++on_host;
+  }
+  if (on_host == (size_t)nsets) {
+    CKC(c0, cudaMemcpyAsync(pl->phis.p, pl->h_phi.p, sizeof(double) * phi_end, cudaMemcpyHostToDevice, st));
+  } else {
+    for (int s = 0; s < nsets && on_host; ++s) {
+      const size_t off = (size_t)pl->phi_off[s];
+      if (!is_device_ptr(phi[s]))
+        CKC(c0, cudaMemcpyAsync(pl->phis.as<double>() + off, pl->h_phi.as<double>() + off,
+                                sizeof(double) * (size_t)B[s] * ctxs[s]->n_k, cudaMemcpyHostToDevice, st));
+    }
+  }
   if (!pl->exec) {
     // first use: run once directly (sets kernel attributes), then capture
     int64_t nl = 0;
@@ -875,23 +1020,35 @@ static int lnl_multi_impl(beor_ctx* const* ctxs, int nsets, const double* const*
     CKC(c0, cudaGraphLaunch(pl->exec, st));
     CKC(c0, cudaEventRecord(pl->ev1, st));
   }
-  for (int s = 0; s < nsets; ++s) {
-    int f = pl->first[s];
-    if (lnl_out && lnl_out[s]) CKC(c0, from_device(lnl_out[s], pl->view.lnl + f, sizeof(double) * B[s], st));
-    if (status_out && status_out[s])
-      CKC(c0, from_device(status_out[s], pl->view.status + f, sizeof(int32_t) * B[s], st));
+  auto lnl_at = [&](int s) { return lnl_out ? lnl_out[s] : nullptr; };
+  auto status_at = [&](int s) { return status_out ? status_out[s] : nullptr; };
+  for (int s = 0; s < nsets; ++s) {   // results to device memory
+    const int f = pl->first[s];
+    if (lnl_at(s) && is_device_ptr(lnl_at(s)))
+      CKC(c0, from_device(lnl_at(s), pl->view.lnl + f, sizeof(double) * B[s], st));
+    if (status_at(s) && is_device_ptr(status_at(s)))
+      CKC(c0, from_device(status_at(s), pl->view.status + f, sizeof(int32_t) * B[s], st));
   }
   // asynchronous call on a captured batch: done once the work is enqueued
   // (errors of bounded device waits are reported by beor_lnl_multi_wait)
   if (async && pl->launches > 0 && pl->exec && !first_use) return BEOR_OK;
+  // lnL, residuals, status and flags by one copy, then to the caller's host memory
+  CKC(c0, cudaMemcpyAsync(pl->h_out.p, pl->scal.as<char>() + pl->out_off, pl->out_bytes, cudaMemcpyDeviceToHost, st));
   CKC(c0, cudaStreamSynchronize(st));
   CKC(c0, cudaGetLastError());
+  const double* h_lnl = pl->h_out.as<double>();
+  const double* resid = h_lnl + pl->P;
+  const int32_t* h_status = reinterpret_cast<int32_t*>(pl->h_out.as<char>() + (pl->status_off - pl->out_off));
+  const Flags* fl = reinterpret_cast<Flags*>(pl->h_out.as<char>() + (pl->flags_off - pl->out_off));
+  for (int s = 0; s < nsets; ++s) {
+    const int f = pl->first[s];
+    if (lnl_at(s) && !is_device_ptr(lnl_at(s))) std::copy(h_lnl + f, h_lnl + f + B[s], lnl_at(s));
+    if (status_at(s) && !is_device_ptr(status_at(s))) std::copy(h_status + f, h_status + f + B[s], status_at(s));
+  }
   int bounds = 0;
   {
-    int fl[2] = {0, 0};   // error, bounds
-    CKC(c0, cudaMemcpy(fl, pl->view.flags, sizeof(fl), cudaMemcpyDeviceToHost));
-    const int err = fl[0];
-    bounds = fl[1];
+    const int err = fl->error;
+    bounds = fl->bounds;
     if (err) {
       for (int s = 0; s < nsets; ++s) {
         ctxs[s]->poisoned = true;
@@ -954,8 +1111,6 @@ static int lnl_multi_impl(beor_ctx* const* ctxs, int nsets, const double* const*
     }
   }
   // diagnostics
-  std::vector<double> resid(pl->P);
-  CKC(c0, cudaMemcpy(resid.data(), pl->view.resid, sizeof(double) * pl->P, cudaMemcpyDeviceToHost));
   for (int s = 0; s < nsets; ++s) {
     beor_ctx* c = ctxs[s];
     c->stats.ms_last = ms;
@@ -993,8 +1148,9 @@ int beor_lnl_multi_wait(beor_ctx* const* ctxs, int nsets, const int* B, int slot
   if (!ctxs || nsets <= 0 || !B || slot < 0 || slot >= 4) return BEOR_EINVAL;
   Plan* pl = nullptr;
   {
-    std::lock_guard<std::mutex> lk(g_mu);
+    std::lock_guard<std::recursive_mutex> lk(g_mu);
     pl = find_plan(ctxs, nsets, B, false, slot);
+    if (pl && pl->retired) pl = nullptr;
   }
   if (!pl) return BEOR_ESTATE;
   beor_ctx* c0 = ctxs[0];
@@ -1094,14 +1250,14 @@ static void drop_stale_graphs() {
 }
 
 int beor_set_profiling(int on) {
-  std::lock_guard<std::mutex> lk(g_mu);
+  std::lock_guard<std::recursive_mutex> lk(g_mu);
   g_profiling = on != 0;
   drop_stale_graphs();
   return BEOR_OK;
 }
 
 int beor_set_lookahead(int on) {
-  std::lock_guard<std::mutex> lk(g_mu);
+  std::lock_guard<std::recursive_mutex> lk(g_mu);
   g_lookahead = on != 0;
   drop_plans_with_stale_schedule();
   return BEOR_OK;
@@ -1121,7 +1277,7 @@ int beor_set_schedule(beor_ctx* const* ctxs, int nsets, const int* B, const beor
   if (r) return r;
   if (sch && (sch->rest_ctas < 0 || sch->col_ctas < 0 || sch->rest_ctas > 65535 || sch->col_ctas > 65535))
     return BEOR_EINVAL;
-  std::lock_guard<std::mutex> lk(g_mu);
+  std::lock_guard<std::recursive_mutex> lk(g_mu);
   const std::string key = shape_key(ctxs, nsets, B, false);
   if (sch) {
     beor_schedule c = *sch;
@@ -1140,14 +1296,14 @@ int beor_get_schedule(beor_ctx* const* ctxs, int nsets, const int* B, beor_sched
   int r = check_shape(ctxs, nsets, B);
   if (r) return r;
   if (!out) return BEOR_EINVAL;
-  std::lock_guard<std::mutex> lk(g_mu);
+  std::lock_guard<std::recursive_mutex> lk(g_mu);
   *out = schedule_of(shape_key(ctxs, nsets, B, false));
   return BEOR_OK;
 }
 
 int beor_set_wait_test(int skip_one_copy, double limit_ms) {
   if (!(limit_ms >= 0.0) || limit_ms > 60000.0) return BEOR_EINVAL;
-  std::lock_guard<std::mutex> lk(g_mu);
+  std::lock_guard<std::recursive_mutex> lk(g_mu);
   g_skip_copy = skip_one_copy != 0;
   g_wait_ns = (unsigned long long)(limit_ms * 1e6);
   drop_stale_graphs();
