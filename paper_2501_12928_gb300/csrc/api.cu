@@ -909,11 +909,13 @@ int beor_precompute(beor_ctx* c, void* stream) {
     CKC(c, precompute_dense(c->T.as<double2>(), c->n_vis, c->n, c->ld, c->w.as<double>(), c->d.as<double2>(), c->nt,
                             c->M.as<double2>(), c->dbar.as<double2>(), s, c->precision == BEOR_PREC_MIXED));
   } else {
-    DevBuf G, u;
+    DevBuf G, u, wp;
     CKC(c, G.alloc(sizeof(double2) * (size_t)c->nf * c->ncells * c->ncells));
     CKC(c, u.alloc(sizeof(double2) * (size_t)c->nf * c->ncells));
+    // products of weights, where they are small beside G; without them if they do not fit
+    if (c->nx <= c->ncells && wp.alloc(sizeof(double2) * (size_t)c->nf * c->nx * c->nx) != cudaSuccess) cudaGetLastError();
     CKC(c, precompute_factored(c->A.as<double2>(), c->W.as<double2>(), c->nf, c->ntb, c->ncells, c->nx,
-                               c->w.as<double>(), c->d.as<double2>(), c->n, c->nt, G.as<double2>(), u.as<double2>(),
+                               c->w.as<double>(), c->d.as<double2>(), c->n, c->nt, G.as<double2>(), u.as<double2>(), wp.as<double2>(),
                                c->M.as<double2>(), c->dbar.as<double2>(), s));
     CKC(c, cudaStreamSynchronize(s));
   }

@@ -22,9 +22,10 @@ cudaError_t precompute_dense(const double2* T, int64_t n_vis, int n, int64_t ld,
 // herk_tc.cu: M (packed lower float64 tiles) = T^H diag(w) T on the tensor cores
 cudaError_t herk_dense_tc(const double2* T, int64_t n_vis, int n, int64_t ld, const double* w, int nt,
                           double2* Mt, cudaStream_t s);
+// P_scratch: nf nx^2 elements for the products of weights, or null
 cudaError_t precompute_factored(const double2* A, const double2* W, int nf, int64_t ntb, int ncells,
                                 int nx, const double* w, const double2* d, int n, int nt,
-                                double2* G_scratch, double2* u_scratch, double2* Mt, double2* dbar,
+                                double2* G_scratch, double2* u_scratch, double2* P_scratch, double2* Mt, double2* dbar,
                                 cudaStream_t s);
 
 // Device-side view of one batched evaluation (all problems of all sets).

@@ -71,3 +71,21 @@ def test_normal_matrix_in_bands_and_on_the_device(P, n):
     out = torch.empty((n, n), dtype=torch.complex128, device="cuda")
     assert P.beor._lib().beor_get_M(lk._h, ctypes.c_void_p(out.data_ptr())) == 0
     np.testing.assert_array_equal(out.cpu().numpy(), M)
+
+
+@pytest.mark.parametrize("ncells,nx", [(2, 3), (3, 2), (9, 40), (40, 9), (41, 41)])
+def test_factored_weights(P, ncells, nx):
+    """The products of weights from a table (nx <= ncells) and formed per element,
+    over one tile and over several with a ragged last one."""
+    nf, ntb = 5, 11
+    g = np.random.default_rng(100 * ncells + nx)
+
+    def cn(*shape):
+        return g.standard_normal(shape) + 1j * g.standard_normal(shape)
+    A, W, d = cn(nf, ntb, ncells), cn(nf, nx), cn(nf * ntb)
+    var = 0.5 + g.random(nf * ntb)
+    lk = P.Likelihood("fp64")
+    lk.set_instrument(A, W, np.zeros(ncells * nx, np.int32), 1, 2.0)
+    lk.set_data(d, var)
+    lk.precompute()
+    _close(lk.get_M(), O.herm_structured(A, W, var))
