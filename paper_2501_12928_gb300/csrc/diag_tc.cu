@@ -43,7 +43,7 @@
 //    per panel.
 //
 // Measured per launch (3280 modes): 0.79 ms before (float64 factor, fp32
-// inverse), now 0.185 ms with one problem (clusters of four), 0.225 ms with 64
+// inverse), now 0.181 ms with one problem (clusters of four), 0.225 ms with 64
 // (clusters of two) and 0.295 ms with 100 (single CTAs).  Most of it is the
 // chain of 128 columns in the panel factors and, between them, the
 // substitutions; loading and output take 13 us.
@@ -276,8 +276,8 @@ __device__ __forceinline__ void dt_sync() {
 }
 
 // Factor of the 16 x 16 diagonal block of panel pan by eight warps of its
-// owner: thread = element (row r, column c); a warp's rows are consecutive, so
-// that finished rows cost nothing.  Square-root-free
+// owner: thread = element (row r, column c); a warp whose two rows have been
+// pivots is done.  Square-root-free
 // elimination, a_rc -= z~_r conj(z~_c) / D, so that only a reciprocal lies
 // between two pivots (beside the products, which do not need it), and every
 // thread forms the next pivot itself: one barrier per column.  The square
@@ -291,6 +291,7 @@ __device__ __forceinline__ void dt_factor(DtSmem& sm, float4* __restrict__ ws, i
   long long d = sm.s[pk(s0, s0)].x;
 #pragma unroll 1
   for (int j = 0; j < DT_P; ++j) {
+    if ((r | 1) < j) break;   // both rows of the warp have been pivots
     int g;
     const long long D = fx_normalise(d > 0 ? d : FX_ONE / 2, g);
     bool over;
@@ -301,28 +302,31 @@ __device__ __forceinline__ void dt_factor(DtSmem& sm, float4* __restrict__ ws, i
       if (over) sm.bad[s0 + r] = 1;
     }
     if (r == j + 1 && c == j + 1) sm.pub[j & 1] = x.x;
-    const fxs w = fx_split(fx_recip(D));
-    dt_fsync();
+    // the warps with row j or rows below it
+    asm volatile("bar.sync 2, %0;" ::"r"(32 * (DT_FW - j / 2)) : "memory");
     if (d <= 0 || sm.bad[s0 + j]) {
-      if (tid < C) dt_peer<C>(sm, tid)->fail = s0 + j + 1;
-      return;
+      if (r == DT_P - 1 && c < C) dt_peer<C>(sm, c)->fail = s0 + j + 1;
+      break;
     }
-    if (tid == 0) sm.piv[s0 + j] = d;
-    if (j == DT_P - 1) break;
+    if (tid == 32 * DT_FW - 1) sm.piv[s0 + j] = d;
+    // the reciprocal beside the products, which do not need it
     const longlong2* zb = sm.zb[j & 1];
-    const fxs nx = fx_split(zb[j + 1].x), ny = fx_split(zb[j + 1].y);
-    d = sm.pub[j & 1] - fx_mul<2>(fx_dot2(nx, nx, ny, ny), w);
+    const longlong2 zn = zb[min(j + 1, DT_P - 1)], zr = zb[r], zc = zb[c];
+    const long long pub = sm.pub[j & 1];
+    const fxs w = fx_split(fx_recip(D));
+    const fxs nx = fx_split(zn.x), ny = fx_split(zn.y);
+    const fxs ar = fx_split(zr.x), ai = fx_split(zr.y), nr = fx_split(-zr.x);
+    const fxs br = fx_split(zc.x), bi = fx_split(zc.y);
+    const long long nn = fx_dot2(nx, nx, ny, ny), re = fx_dot2(ar, br, ai, bi), im = fx_dot2(ai, br, nr, bi);
+    d = pub - fx_mul<2>(nn, w);
     if (c > j && c <= r) {
-      const longlong2 zr = zb[r];
-      const fxs ar = fx_split(zr.x), ai = fx_split(zr.y), nr = fx_split(-zr.x);
-      const fxs br = fx_split(zb[c].x), bi = fx_split(zb[c].y);
-      const long long re = fx_dot2(ar, br, ai, bi), im = fx_dot2(ai, br, nr, bi);
       if (c == r && re > D + (1ll << 45)) sm.bad[s0 + r] = 1;   // |L~_rj| > 1
       x.x -= fx_mul<2>(re, w);
       x.y -= fx_mul<2>(im, w);
     }
   }
   dt_fsync();   // every pivot is written
+  if (sm.fail) return;
   if (tid < DT_P) {
     int g;
     const long long piv = sm.piv[s0 + tid];
@@ -470,11 +474,21 @@ __device__ __forceinline__ void dt_inverse_rows(DtSmem& sm, int pan, int j, int 
   DtSmem* own = dt_peer<C>(sm, pan % C);            // holds the rows
   const float sg = comp ? 1.0f : -1.0f;
   float mx = 0.0f;
+  if (C > 1 && own != &sm && j < s0) {   // the column so far, all rows in flight at once
+    float2 b[DT_P / DT_IP];
+#pragma unroll
+    for (int q = 0; q < DT_P / DT_IP; ++q)
+      b[q] = reinterpret_cast<const float2*>(&own->s[pk(s0 + part * (DT_P / DT_IP) + q, j)])[comp];
+#pragma unroll
+    for (int q = 0; q < DT_P / DT_IP; ++q)
+      reinterpret_cast<float2*>(&sm.s[pk(s0 + part * (DT_P / DT_IP) + q, j)])[comp] = b[q];
+    __syncwarp();
+  }
 #pragma unroll 1
   for (int r = 0; r < DT_P; ++r) {
     dfl c0{j == s0 + r && !comp && !part ? 1.0f : 0.0f, 0.0f}, c1{0.0f, 0.0f};
     if (j < s0 && !part) {
-      const float2 b = reinterpret_cast<const float2*>(&own->s[pk(s0 + r, j)])[comp];
+      const float2 b = reinterpret_cast<const float2*>(&sm.s[pk(s0 + r, j)])[comp];
       c0 = dfl{b.x, b.y};
     }
 #pragma unroll 2
