@@ -7,8 +7,9 @@
 // pipe.
 //
 // What bounds it: one SM issues a float64 warp instruction every 19 cycles, so
-// that a block's 44,000 take 0.42 ms there; the chain of 128 square roots and
-// reciprocals (1,000 cycles each pair) takes 0.08 ms on any number of SMs.  The
+// that a block's 44,000 take 0.42 ms there; the chain of 128 pivots takes 0.06 ms
+// on any number of SMs (their square roots and reciprocals from integers, 450
+// cycles a pair; 1,000 with float64's).  The
 // rows are dealt to the CTAs in blocks of eight (zigzag, so that each has short
 // and long ones); per panel of 16 columns every CTA factors the 16 x 16
 // diagonal (the same operations everywhere, cheaper than an exchange per
@@ -16,13 +17,14 @@
 // The inverse goes by columns, which do not depend on each other, from the copy
 // of L that every CTA then has.  One point of 3280 modes, one CTA with barriers
 // per column -> eight: float64 1.16 ms -> 0.39 per block, posterior mean 0.79 ->
-// 0.33.
+// 0.33; with the pivots' square roots and reciprocals from integers 0.35 and 0.30.
 #include <cooperative_groups.h>
 
 #include <cmath>
 #include <type_traits>
 
 #include "diag_common.cuh"
+#include "diag_fixed.cuh"
 
 namespace beor {
 
@@ -136,8 +138,17 @@ __device__ __forceinline__ void dc_factor(double2* A, DcCommon& sm, int s0, int 
   for (int j = 0; j < DC_P; ++j) {
     if (chain) {
       const bool ok = d > 0.0 && isfinite(d);
-      const double l = sqrt(d);
-      const double rinv = 1.0 / l;
+      double l, rinv;
+      const int ef = __double2hiint(d) >> 20;
+      if (ef >= 1 && ef < 2047) {
+        long long lb, rb;
+        fx_sqrt_rcp(__double_as_longlong(d), lb, rb);
+        l = __longlong_as_double(lb);
+        rinv = __longlong_as_double(rb);
+      } else {
+        l = sqrt(d);
+        rinv = 1.0 / l;
+      }
       if (tid == 128) {
         if (!ok) sm.fail = col0 + s0 + j + 1;
         A[pk(s0 + j, s0 + j)] = make_double2(l, 0.0);
@@ -632,7 +643,7 @@ static cudaError_t launch_dc(const BatchView& v, int k, cudaStream_t s, int prio
 
 // Float64: the largest cluster, of up to eight CTAs, of which the GPU holds the
 // whole batch at once (15 clusters of eight, 36 of four and 76 of two on a GB300:
-// 0.39, 0.50 and 0.77 ms a block), else one CTA per block (1.17 ms).  The
+// 0.35, 0.46 and 0.73 ms a block), else one CTA per block (1.17 ms).  The
 // posterior mean is of one point, and always takes eight.
 cudaError_t launch_diag_cluster(const BatchView& v, int k, bool mixed, int active, cudaStream_t s, int prio) {
   if (mixed) return launch_dc<float4, DIAG_MEAN_CTAS>(v, k, s, prio);

@@ -101,6 +101,26 @@ __host__ __device__ __forceinline__ long long fx_rsqrt(long long D) {
   return (((long long)yh << 32) + (fx_mulhi((long long)yh << 32, c << 22) >> 18) + 1) >> 1;
 }
 
+// l = sqrt(d) and 1 / l, both correctly rounded, of a normal d > 0, by integer
+// operations: 53-bit candidates from the reciprocal square root above, then the
+// sign of the exact remainder, whose magnitude leaves the low 64 bits of each
+// product to decide it.  Half the latency of float64's square root and division.
+__host__ __device__ __forceinline__ void fx_sqrt_rcp(long long bits, long long& l, long long& rinv) {
+  const int e = (int)(bits >> 52) - 1023, odd = e & 1, h = (e - odd) / 2;
+  const long long one = 1ll << 52;
+  const long long m = ((bits & (one - 1)) | one) << odd;       // d = m 2^(2 h - 52), 2^52 <= m < 2^54
+  const long long y = fx_rsqrt(m << 7);                        // 1 / sqrt(m 2^-54), 60 fractional bits
+  const unsigned long long p = fx_umulhi((unsigned long long)m << 10, (unsigned long long)y << 2);
+  long long s = (long long)((p + 256) >> 9);                   // sqrt(m 2^52), within 1 of its rounding
+  const long long r = (long long)(((unsigned long long)m << 52) - (unsigned long long)s * (unsigned long long)s);
+  s += (r > s) - (r <= -s);                                    // (s - 1/2)^2 < m 2^52 < (s + 1/2)^2
+  l = ((long long)(h + 1023) << 52) + (s - one);
+  long long t = y >> 8;                                        // 2^105 / s, within 2 of its rounding
+  const long long q = 2 * -(long long)((unsigned long long)t * (unsigned long long)s);   // 2 (2^105 - t s)
+  t += (q > s) + (q > 3 * s) - (q < -s) - (q < -3 * s);        // no ties: s would have to divide a power of two
+  rinv = ((long long)(1022 - h) << 52) + (t - one);
+}
+
 // Balanced base-512 digits of X, |X| <= 2^53: X = sum_s d[s] 512^(5 - s),
 // d[1..5] in [-256, 255], |d[0]| <= 256: each exact in bf16.
 __host__ __device__ __forceinline__ void fx_digits(long long x, int* d) {
