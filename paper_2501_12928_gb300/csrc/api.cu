@@ -285,8 +285,6 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
     RUN(KC_DIAG, launch_diag(v, 0, true, active(0), s, hi));
     L += 1;
     if ((e = fwd_after_diag()) != cudaSuccess) return e;
-    RUN_ON(KC_SOLVE, pl.side2, launch_fwd_step(v, true, v.vec_b, -1, pl.side2));
-    L += 1;
     if (pl.max_nt > 1) {
       RUN(KC_SLICE, launch_slice_panel(v, 0, s, hi));
       RUN(KC_PANEL, launch_panel_mixed(v, pl.maps, 0, s, hi));
@@ -304,7 +302,7 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
       L += 1;
       if ((e = fwd_after_diag()) != cudaSuccess) return e;
       RUN_ON(KC_SOLVE, pl.side2, launch_fwd_step(v, true, v.vec_b, k, pl.side2));
-      L += 1;
+      L += fwd_step_launches(v, k);
       if (mixed_tiles(pl.maps, 1, k) > 0) {
         // reserve_diag: leave free the SMs that step k + 1's diagonal blocks
         // (running beside this launch) need
@@ -324,6 +322,8 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
       }
       if ((e = cudaStreamWaitEvent(s, pl.ev_rest, 0)) != cudaSuccess) return e;
     }
+    RUN_ON(KC_SOLVE, pl.side2, launch_fwd_step(v, true, v.vec_b, pl.max_nt - 1, pl.side2));
+    L += fwd_step_launches(v, pl.max_nt - 1);
     if ((e = cudaEventRecord(pl.ev_fwd, pl.side2)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(s, pl.ev_fwd, 0)) != cudaSuccess) return e;
   } else {
@@ -347,10 +347,10 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
   }
   if (la) {
     RUN(KC_SOLVE, launch_bwd(v, true, v.vec_x, s));   // the forward half ran during the factorisation
-    L += pl.max_nt;
+    L += solve_pass_launches(v);
   } else {
     RUN(KC_SOLVE, launch_solve(v, pl.mixed, v.vec_b, v.vec_x, s));
-    L += solve_launch_count(pl.max_nt);
+    L += 2 * solve_pass_launches(v);
   }
   const bool corr = pl.mixed && !pl.refine_x;
   if (pl.mixed && pl.refine_x) {
@@ -359,14 +359,14 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
       RUN(KC_REFINE, launch_residual(v, s));
       RUN(KC_SOLVE, launch_solve(v, true, v.vec_r, v.vec_d, s));
       RUN(KC_REFINE, launch_refine_update(v, s));
-      L += 4 + solve_launch_count(pl.max_nt);
+      L += 4 + 2 * solve_pass_launches(v);
     }
   } else if (corr) {
     // lnL only: one float64 residual r = dbar - Sigma x~ and y = L~^-1 r
     // correct the quadratic form (see lnl_kernel)
     RUN(KC_REFINE, launch_residual(v, s));
     RUN(KC_SOLVE, launch_solve_fwd(v, true, v.vec_r, s));
-    L += 3 + pl.max_nt;
+    L += 3 + solve_pass_launches(v);
   }
   RUN(KC_LNL, launch_lnl(v, s, corr ? 1 : 0));
   L += 1;

@@ -146,11 +146,12 @@ cudaError_t launch_diag_cluster(const BatchView& v, int k, bool mixed, int activ
 cudaError_t launch_panel_f64(const BatchView& v, int k, cudaStream_t s);
 cudaError_t launch_trail_f64(const BatchView& v, int k, cudaStream_t s);
 cudaError_t launch_solve(const BatchView& v, bool mixed, const double2* rhs, double2* out, cudaStream_t s);
-// The solve's two halves: forward step k (k = -1: start) of vec_y = L^-1 rhs,
-// and the whole backward pass out = L^-H vec_y.
-cudaError_t launch_fwd_step(const BatchView& v, bool mixed, const double2* rhs, int k, cudaStream_t s, int prio = 0);
+// The solve's two halves: forward step k (0 .. max_nt - 1) of vec_y = L^-1 rhs, the
+// whole forward pass, and the whole backward pass out = L^-H vec_y.
+cudaError_t launch_fwd_step(const BatchView& v, bool mixed, const double2* rhs, int k, cudaStream_t s);
+int fwd_step_launches(const BatchView& v, int k);
 cudaError_t launch_bwd(const BatchView& v, bool mixed, double2* out, cudaStream_t s);
-int solve_launch_count(int max_nt);
+int solve_pass_launches(const BatchView& v);   // of a whole pass
 cudaError_t launch_lnl(const BatchView& v, cudaStream_t s, int corr);   // corr: residual-corrected q
 cudaError_t launch_solve_fwd(const BatchView& v, bool mixed, const double2* rhs, cudaStream_t s);   // vec_y = L^-1 rhs
 cudaError_t launch_copy_dbar(const BatchView& v, cudaStream_t s);
