@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
+#include <utility>
 
 #include "diag_common.cuh"
 
@@ -10,13 +11,13 @@ namespace beor {
 // --------------------------------------------------------------------------
 // Triangular solves with the factor: out = L^-H L^-1 rhs, blocked by 128.  Step k
 // has two parts: its block of the solution, y_k = Linv_k r_k, and the update of
-// the other blocks, r_i -= L_ik y_k (backward: with L_ki^H), a quarter of a tile
-// (32 rows, or columns) per CTA.
+// the other blocks, r_i -= L_ik y_k (backward: with L_ki^H).
 //   - Large batches launch one after the other: a CTA per problem, then a CTA per
-//     quarter tile.  Small ones do both in one launch, every CTA forming y_k for
-//     itself (33,000 products, cheaper than a launch that waits for one CTA).
-//   - Tile and inverse block are copied to shared memory by cp.async, all in
-//     flight at once, before the step waits for the one before (programmatic
+//     tile.  Small ones do both in one launch, a CTA per quarter tile, every one
+//     forming y_k for itself (33,000 products, cheaper than a launch that waits
+//     for one CTA).
+//   - Inverse block and quarter tile are copied to shared memory by cp.async, all
+//     in flight at once, before the step waits for the one before (programmatic
 //     dependent launch): the factor is final by then.
 //   - Real and imaginary part of a sum go to two threads.
 // Off-diagonal products: float64 for the float64 path, double-float (fp32 pairs,
@@ -26,13 +27,12 @@ namespace beor {
 // Bound by memory in large batches, by the launch and by the chains of dependent
 // products in small ones.  A step with one CTA per tile and 16 rounds of loads,
 // the inverse block in one CTA at its end, took 35 us with one point of 3280
-// modes and 71 with 64; now 5 and 62.  Float64, one point of 2000 modes: 38
+// modes and 71 with 64; now 5 and 60.  Float64, one point of 2000 modes: 38
 // -> 30 us, whose chains of 128 dependent pairs of products alone are 9 us.
 // --------------------------------------------------------------------------
 constexpr int SOLVE_SPLIT = 4;                       // CTAs per tile
 constexpr int SOLVE_ROWS = BEOR_TB / SOLVE_SPLIT;
 constexpr int SOLVE_THREADS = 512;
-enum { PART_BOTH = 0, PART_BLOCK = 1, PART_UPDATE = 2 };
 template <typename V>   // V: the factor's real type, double or dfl
 struct SolveVecs {
   double2 yk[BEOR_TB];
@@ -43,11 +43,9 @@ struct SolveVecs {
 };
 // shared memory: Linv_k, packed (double2 or float4 elements); the quarter tile,
 // forward [column][own row], backward [own column][row]; the vectors
-constexpr int solve_li(int part) { return part == PART_UPDATE ? 0 : DG_PACK; }
-constexpr int solve_tile(int part) { return part == PART_BLOCK ? 0 : BEOR_TB * SOLVE_ROWS; }
 template <typename V>
-constexpr size_t solve_smem(int part) {
-  return sizeof(double2) * (size_t)(solve_li(part) + solve_tile(part)) + sizeof(SolveVecs<V>);
+constexpr size_t solve_smem(bool both) {
+  return sizeof(double2) * (size_t)(DG_PACK + (both ? BEOR_TB * SOLVE_ROWS : 0)) + sizeof(SolveVecs<V>);
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -130,33 +128,32 @@ __device__ __forceinline__ void solve_diag(const float4* li, const double (*)[BE
   }
 }
 
-// Step k of y = L^-1 src (CTA (SOLVE_SPLIT (i - k - 1) + quarter, p)) or, HERM, of
-// out = L^-H src (CTA (SOLVE_SPLIT i + quarter, p), problems join when k < their
-// nt).  src: the right-hand side; the running one is vec_t.
-template <typename WS, typename DV, bool HERM, int PART>
-__global__ void __launch_bounds__(SOLVE_THREADS, PART == PART_UPDATE ? 2 : 1)
+// Step k's block of y = L^-1 src or, HERM, of out = L^-H src; BOTH: and its update,
+// by CTA (SOLVE_SPLIT (i - k - 1) + quarter, p) or, HERM, (SOLVE_SPLIT i + quarter,
+// p), where problems join when k < their nt.  src: the right-hand side; the running
+// one is vec_t.
+template <typename WS, typename DV, bool HERM, bool BOTH>
+__global__ void __launch_bounds__(SOLVE_THREADS, 1)
     solve_step_kernel(BatchView v, int kg, const double2* src, double2* out) {
   using V = typename std::conditional<std::is_same<WS, float4>::value, dfl, double>::type;
   extern __shared__ __align__(16) unsigned char ss_raw[];
   double2* const s_li = reinterpret_cast<double2*>(ss_raw);
-  double2* const s_tile = s_li + solve_li(PART);
-  SolveVecs<V>& sm = *reinterpret_cast<SolveVecs<V>*>(s_tile + solve_tile(PART));
+  double2* const s_tile = s_li + DG_PACK;
+  SolveVecs<V>& sm = *reinterpret_cast<SolveVecs<V>*>(s_tile + (BOTH ? BEOR_TB * SOLVE_ROWS : 0));
   dfl* const dpart = reinterpret_cast<dfl*>(sm.yv);   // HERM, DV float4: halves of yk (yv is filled after)
   const int tid = threadIdx.x, p = blockIdx.y;
   const Prob pr = v.prob[p];
   const int k = HERM ? kg : kg - pr.k_off;   // this problem's step
   const int i = (HERM ? 0 : k + 1) + blockIdx.x / SOLVE_SPLIT, c0 = blockIdx.x % SOLVE_SPLIT * SOLVE_ROWS;
-  const bool upd = PART != PART_BLOCK && (HERM ? i < k : i < pr.nt);   // has a block to update
+  const bool upd = BOTH && (HERM ? i < k : i < pr.nt);   // has a block to update
   const int ti = HERM ? k : i, tj = HERM ? i : k;
-  bool on = k >= 0 && k < pr.nt && (upd || (PART != PART_UPDATE && blockIdx.x == 0)) && !prob_skipped(v.status[p]);
+  bool on = k >= 0 && k < pr.nt && (upd || blockIdx.x == 0) && !prob_skipped(v.status[p]);
   on = on && BEOR_INBOUNDS(v.flags, pr.row_off + (int64_t)pr.nt * BEOR_TB <= v.rows, BC_SOLVE_VEC) &&
        BEOR_INBOUNDS(v.flags, !upd || pr.ws_off + (tri_index(ti, tj) + 1) * BEOR_TILE_ELEMS <= v.ws_elems, BC_SOLVE_VEC) &&
        BEOR_INBOUNDS(v.flags, pr.dinv_off + (int64_t)(k + 1) * DG_PACK <= v.dinv_elems, BC_DIAG_DINV);
   if (on) {
-    if (PART != PART_UPDATE) {
-      const double2* li = reinterpret_cast<const double2*>(v.dinv) + pr.dinv_off + (int64_t)k * DG_PACK;
-      for (int e = tid; e < DG_PACK; e += SOLVE_THREADS) cp_async16(&s_li[e], li + e);
-    }
+    const double2* li = reinterpret_cast<const double2*>(v.dinv) + pr.dinv_off + (int64_t)k * DG_PACK;
+    for (int e = tid; e < DG_PACK; e += SOLVE_THREADS) cp_async16(&s_li[e], li + e);
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (upd) {
       const double2* t = reinterpret_cast<const double2*>(v.ws) + pr.ws_off + tri_index(ti, tj) * BEOR_TILE_ELEMS;
@@ -175,32 +172,29 @@ __global__ void __launch_bounds__(SOLVE_THREADS, PART == PART_UPDATE ? 2 : 1)
   if (!on) return;
   const bool first = k == (HERM ? pr.nt - 1 : 0);
   const double2* r = (first ? src : v.vec_t) + pr.row_off;
-  double2* const yk = out + pr.row_off + k * BEOR_TB;
   const int comp = HERM ? tid >> 8 : (tid >> 6) & 1;               // update: component,
   const int own = HERM ? (tid >> 3) & 31 : tid & 31;               // row (column),
   const int ms = HERM ? tid & 7 : (tid >> 5) & 1;                  // part of the sum
   const bool last = upd && (HERM ? ms == 0 : ms == 0 && tid < 128);   // takes the sum
   double cur = 0.0;
   if (last) cur = reinterpret_cast<const double*>(r + i * BEOR_TB + c0 + own)[comp];
-  if (PART != PART_UPDATE) {
-    if (tid < BEOR_TB) {
-      const double2 q = r[k * BEOR_TB + tid];
-      if constexpr (std::is_same<DV, double2>::value) {
-        sm.rd[0][tid] = q.x;
-        sm.rd[1][tid] = q.y;
-      } else {
-        sm.rf[0][tid] = df_from_double(q.x);
-        sm.rf[1][tid] = df_from_double(q.y);
-      }
-    }
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();
-    solve_diag<HERM>(reinterpret_cast<const DV*>(s_li), sm.rd, sm.rf, dpart, sm.yk);
-    __syncthreads();
-  }
   if (tid < BEOR_TB) {
-    const double2 q = PART == PART_UPDATE ? yk[tid] : sm.yk[tid];
-    if (PART != PART_UPDATE && blockIdx.x == 0) yk[tid] = q;
+    const double2 q = r[k * BEOR_TB + tid];
+    if constexpr (std::is_same<DV, double2>::value) {
+      sm.rd[0][tid] = q.x;
+      sm.rd[1][tid] = q.y;
+    } else {
+      sm.rf[0][tid] = df_from_double(q.x);
+      sm.rf[1][tid] = df_from_double(q.y);
+    }
+  }
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
+  __syncthreads();
+  solve_diag<HERM>(reinterpret_cast<const DV*>(s_li), sm.rd, sm.rf, dpart, sm.yk);
+  __syncthreads();
+  if (tid < BEOR_TB) {
+    const double2 q = sm.yk[tid];
+    if (blockIdx.x == 0) out[pr.row_off + k * BEOR_TB + tid] = q;
     to_real(sm.yv[0][tid], q.x);
     to_real(sm.yv[1][tid], q.y);
   }
@@ -231,28 +225,115 @@ __global__ void __launch_bounds__(SOLVE_THREADS, PART == PART_UPDATE ? 2 : 1)
   if (last) reinterpret_cast<double*>(v.vec_t + pr.row_off + i * BEOR_TB + c0 + own)[comp] = cur - get_part(a);
 }
 
+// The update of step k alone, a CTA per tile: the tile streams through registers,
+// 16 elements in flight per thread (held in shared memory, a tile's quarters wait
+// for their last element and then for the chains: 117 us for 25 tiles of each of
+// 64 points; __UPD__ here, 62 at the copy rate).  y: vec_y or, HERM, the solution.
+template <typename WS, bool HERM>
+__global__ void __launch_bounds__(256, 2)
+    solve_update_kernel(BatchView v, int kg, const double2* src, const double2* y) {
+  using V = typename std::conditional<std::is_same<WS, float4>::value, dfl, double>::type;
+  __shared__ V yv[2][BEOR_TB], part[2][BEOR_TB];
+  const int tid = threadIdx.x, p = blockIdx.y;
+  const Prob pr = v.prob[p];
+  const int k = HERM ? kg : kg - pr.k_off;   // this problem's step
+  const int i = (HERM ? 0 : k + 1) + blockIdx.x, ti = HERM ? k : i, tj = HERM ? i : k;
+  const bool on = k >= 0 && k < pr.nt && (HERM ? i < k : i < pr.nt) && !prob_skipped(v.status[p]) &&
+                  BEOR_INBOUNDS(v.flags, pr.row_off + (int64_t)pr.nt * BEOR_TB <= v.rows, BC_SOLVE_VEC) &&
+                  BEOR_INBOUNDS(v.flags, pr.ws_off + (tri_index(ti, tj) + 1) * BEOR_TILE_ELEMS <= v.ws_elems, BC_SOLVE_VEC);
+  // forward: row and half of the columns; backward: eight lanes per column,
+  // interleaved rows, four columns per warp in turn
+  const int row = tid & 127, half = tid >> 7;
+  const int col = (tid >> 5) * 16 + ((tid >> 3) & 3), mo = tid & 7;
+  const WS* __restrict__ t = reinterpret_cast<const WS*>(v.ws) + pr.ws_off + (on ? tri_index(ti, tj) : 0) * BEOR_TILE_ELEMS +
+                             (HERM ? col * BEOR_TB + mo : half * 64 * BEOR_TB + row);
+  WS a[8], b[8];
+  auto load = [&](WS* o, int c) {   // chunk c of eight elements
+#pragma unroll
+    for (int q = 0; q < 8; ++q) o[q] = __ldcs(t + (HERM ? (c >> 1) * 4 * BEOR_TB + 8 * ((c & 1) * 8 + q) : (8 * c + q) * BEOR_TB));
+  };
+  if (on) load(a, 0);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!on) return;
+  const double2* r = (k == (HERM ? pr.nt - 1 : 0) ? src : v.vec_t) + pr.row_off + i * BEOR_TB;
+  double2* const out = v.vec_t + pr.row_off + i * BEOR_TB;
+  if (tid < BEOR_TB) {
+    const double2 q = y[pr.row_off + k * BEOR_TB + tid];
+    to_real(yv[0][tid], q.x);
+    to_real(yv[1][tid], q.y);
+  }
+  __syncthreads();
+  V acc[2] = {};
+  auto mac = [&](const WS* l, int c) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int m = HERM ? mo + 8 * ((c & 1) * 8 + q) : half * 64 + 8 * c + q;
+#pragma unroll
+      for (int comp = 0; comp < 2; ++comp) mac_part(acc[comp], l + q, HERM, comp, yv[comp][m], yv[1 - comp][m]);
+    }
+  };
+#pragma unroll 1
+  for (int c = 0; c < 8; c += 2) {
+    load(b, c + 1);
+    mac(a, c);
+    if (c + 2 < 8) load(a, c + 2);
+    mac(b, c + 1);
+    if (HERM) {
+#pragma unroll
+      for (int comp = 0; comp < 2; ++comp)
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) add_part(acc[comp], shfl_part(acc[comp], o));
+      if (mo == 0) {
+        const int cc = col + 2 * c;
+        const double2 cur = r[cc];
+        out[cc] = make_double2(cur.x - get_part(acc[0]), cur.y - get_part(acc[1]));
+      }
+      acc[0] = acc[1] = V{};
+    }
+  }
+  if (!HERM) {
+    if (half) {
+      part[0][row] = acc[0];
+      part[1][row] = acc[1];
+    }
+    __syncthreads();
+    if (!half) {
+      const double2 cur = r[row];
+      add_part(acc[0], part[0][row]);
+      add_part(acc[1], part[1][row]);
+      out[row] = make_double2(cur.x - get_part(acc[0]), cur.y - get_part(acc[1]));
+    }
+  }
+}
+
 // after: the launch before on the stream is the step before (its results, not the
 // factor, are what is waited for)
-template <typename WS, typename DV, bool HERM, int PART>
-static cudaError_t launch_part(const BatchView& v, int k, const double2* src, double2* out, cudaStream_t s, bool after) {
-  using V = typename std::conditional<std::is_same<WS, float4>::value, dfl, double>::type;
-  auto kern = solve_step_kernel<WS, DV, HERM, PART>;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_smem<V>(PART));
-  if (attr != cudaSuccess) return attr;
-  const int blocks = PART == PART_BLOCK ? 0 : HERM ? k : v.max_nt - 1 - k;   // to update
-  if (PART == PART_UPDATE && blocks == 0) return cudaSuccess;
+template <typename... Exp, typename... Act>
+static cudaError_t launch_after(void (*kern)(Exp...), dim3 grid, int threads, size_t smem, cudaStream_t s, bool after,
+                                Act&&... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(std::max(1, SOLVE_SPLIT * blocks), v.P);
-  cfg.blockDim = dim3(SOLVE_THREADS);
-  cfg.dynamicSmemBytes = solve_smem<V>(PART);
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = after ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, v, k, src, out);
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<Act>(args)...);
+}
+template <typename WS, typename DV, bool HERM, bool BOTH>
+static cudaError_t launch_block(const BatchView& v, int k, int blocks, const double2* src, double2* out, cudaStream_t s,
+                                bool after) {
+  using V = typename std::conditional<std::is_same<WS, float4>::value, dfl, double>::type;
+  auto kern = solve_step_kernel<WS, DV, HERM, BOTH>;
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_smem<V>(BOTH));
+  if (attr != cudaSuccess) return attr;
+  return launch_after(kern, dim3(BOTH ? std::max(1, SOLVE_SPLIT * blocks) : 1, v.P), SOLVE_THREADS, solve_smem<V>(BOTH), s,
+                      after, v, k, src, out);
 }
 // The products with the inverse block in every CTA pay while the first step's CTAs
 // fit the SMs once.  Solves of one evaluation in ms (one launch per step / two):
@@ -263,9 +344,11 @@ static bool solve_is_small(const BatchView& v) { return (int64_t)SOLVE_SPLIT * v
 // Step k of one pass.
 template <bool HERM, typename WS, typename DV>
 static cudaError_t step_as(const BatchView& v, bool both, int k, const double2* src, double2* out, cudaStream_t s, bool after) {
-  if (both) return launch_part<WS, DV, HERM, PART_BOTH>(v, k, src, out, s, after);
-  const cudaError_t e = launch_part<WS, DV, HERM, PART_BLOCK>(v, k, src, out, s, after);
-  return e == cudaSuccess ? launch_part<WS, DV, HERM, PART_UPDATE>(v, k, src, out, s, true) : e;
+  const int blocks = HERM ? k : v.max_nt - 1 - k;   // to update
+  if (both) return launch_block<WS, DV, HERM, true>(v, k, blocks, src, out, s, after);
+  const cudaError_t e = launch_block<WS, DV, HERM, false>(v, k, blocks, src, out, s, after);
+  if (e != cudaSuccess || blocks == 0) return e;
+  return launch_after(solve_update_kernel<WS, HERM>, dim3(blocks, v.P), 256, 0, s, true, v, k, src, (const double2*)out);
 }
 template <bool HERM>
 static cudaError_t solve_step(const BatchView& v, bool mixed, bool both, int k, const double2* src, double2* out,
