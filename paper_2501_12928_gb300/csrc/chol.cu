@@ -238,51 +238,58 @@ cudaError_t launch_panel_f64(const BatchView& v, int k, cudaStream_t s) {
 }
 
 // --------------------------------------------------------------------------
-// float64 trailing update: A_ij -= L_ik L_jk^H, k < j <= i, 64 x 64 sub-tiles
+// float64 trailing update: A_ij -= L_ik L_jk^H, k < j <= i, 32 x 32 sub-tiles
+//
+// Bound by the float64 pipe: a sub-tile takes 0.13 ms of one SM.  With 64 x 64
+// sub-tiles (0.5 ms) the late steps of a small batch, of fewer sub-tiles than a
+// few per SM, left SMs idle for up to that long: one point of 3280 modes 45.2 ms,
+// now 39.9, with the pipe busy throughout.
 // --------------------------------------------------------------------------
+constexpr int TF_S = 32, TF_N = BEOR_TB / TF_S, TF_K = 32, TF_Q = TF_S / 16;   // sub-tile, per side, terms at once, per thread
 __global__ void __launch_bounds__(256) trail_f64_kernel(BatchView v, int kg) {
-  __shared__ double2 xs[16][64];
-  __shared__ double2 ys[16][64];
+  __shared__ double2 xs[TF_K][TF_S];
+  __shared__ double2 ys[TF_K][TF_S];
   const int p = blockIdx.y;
   const Prob pr = v.prob[p];
   const int k = kg - pr.k_off;
   const int T = k < 0 ? 0 : pr.nt - k - 1;
-  const int64_t t = blockIdx.x >> 2;
+  const int64_t t = blockIdx.x / (TF_N * TF_N);
   if (T <= 0 || t >= tri_count(T) || v.status[p] != 0) return;
-  const int si = (blockIdx.x >> 1) & 1, sj = blockIdx.x & 1;
+  const int si = blockIdx.x / TF_N % TF_N, sj = blockIdx.x % TF_N;
   int a, b;
   tile_of(t, a, b);
   const int i = k + 1 + a, j = k + 1 + b;
   if (i == j && si < sj) return;   // upper part of a diagonal tile is never read
   double2* ws = reinterpret_cast<double2*>(v.ws) + pr.ws_off;
-  const double2* X = ws + tri_index(i, k) * BEOR_TILE_ELEMS + si * 64;
-  const double2* Y = ws + tri_index(j, k) * BEOR_TILE_ELEMS + sj * 64;
+  const double2* X = ws + tri_index(i, k) * BEOR_TILE_ELEMS + si * TF_S;
+  const double2* Y = ws + tri_index(j, k) * BEOR_TILE_ELEMS + sj * TF_S;
   double2* C = ws + tri_index(i, j) * BEOR_TILE_ELEMS;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double ar[4][4], ai[4][4];
+  double ar[TF_Q][TF_Q], ai[TF_Q][TF_Q];
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < TF_Q; ++q)
 #pragma unroll
-    for (int w = 0; w < 4; ++w) ar[q][w] = ai[q][w] = 0.0;
-  for (int m0 = 0; m0 < BEOR_TB; m0 += 16) {
-    for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-      int mm = e / 64, r = e % 64;
+    for (int w = 0; w < TF_Q; ++w) ar[q][w] = ai[q][w] = 0.0;
+  for (int m0 = 0; m0 < BEOR_TB; m0 += TF_K) {
+#pragma unroll
+    for (int e = threadIdx.x; e < TF_K * TF_S; e += 256) {
+      const int mm = e / TF_S, r = e % TF_S;
       xs[mm][r] = X[(m0 + mm) * BEOR_TB + r];
       ys[mm][r] = Y[(m0 + mm) * BEOR_TB + r];
     }
     __syncthreads();
 #pragma unroll 4
-    for (int mm = 0; mm < 16; ++mm) {
-      double2 x[4], y[4];
+    for (int mm = 0; mm < TF_K; ++mm) {
+      double2 x[TF_Q], y[TF_Q];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        x[q] = xs[mm][ty * 4 + q];
-        y[q] = ys[mm][tx * 4 + q];
+      for (int q = 0; q < TF_Q; ++q) {
+        x[q] = xs[mm][ty * TF_Q + q];
+        y[q] = ys[mm][tx * TF_Q + q];
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+      for (int q = 0; q < TF_Q; ++q)
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
+        for (int w = 0; w < TF_Q; ++w) {
           ar[q][w] = fma(x[q].x, y[w].x, fma(x[q].y, y[w].y, ar[q][w]));
           ai[q][w] = fma(x[q].y, y[w].x, fma(-x[q].x, y[w].y, ai[q][w]));
         }
@@ -290,10 +297,10 @@ __global__ void __launch_bounds__(256) trail_f64_kernel(BatchView v, int kg) {
     __syncthreads();
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < TF_Q; ++q)
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      int r = si * 64 + ty * 4 + q, c = sj * 64 + tx * 4 + w;
+    for (int w = 0; w < TF_Q; ++w) {
+      const int r = si * TF_S + ty * TF_Q + q, c = sj * TF_S + tx * TF_Q + w;
       double2 cv = C[c * BEOR_TB + r];
       cv.x -= ar[q][w];
       cv.y -= ai[q][w];
@@ -304,7 +311,7 @@ __global__ void __launch_bounds__(256) trail_f64_kernel(BatchView v, int kg) {
 cudaError_t launch_trail_f64(const BatchView& v, int k, cudaStream_t s) {
   int T = v.max_nt - k - 1;
   if (T <= 0) return cudaSuccess;
-  int64_t nblk = tri_count(T) * 4;
+  int64_t nblk = tri_count(T) * TF_N * TF_N;
   trail_f64_kernel<<<dim3((unsigned)nblk, v.P), 256, 0, s>>>(v, k);
   return cudaGetLastError();
 }

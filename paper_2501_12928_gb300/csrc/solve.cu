@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1)
 // The update of step k alone, a CTA per tile: the tile streams through registers,
 // 16 elements in flight per thread (held in shared memory, a tile's quarters wait
 // for their last element and then for the chains: 117 us for 25 tiles of each of
-// 64 points; __UPD__ here, 62 at the copy rate).  y: vec_y or, HERM, the solution.
+// 64 points; 85 here, 62 at the copy rate).  y: vec_y or, HERM, the solution.
 template <typename WS, bool HERM>
 __global__ void __launch_bounds__(256, 2)
     solve_update_kernel(BatchView v, int kg, const double2* src, const double2* y) {
