@@ -207,6 +207,73 @@ __global__ void __launch_bounds__(256) xh_w_d_kernel(const double2* __restrict__
   atomicAdd(&u[j].y, si);
 }
 
+// The same, same bits, where that has few CTAs.
+// A chunk's sum is one chain of dependent float64 products per component (134
+// cycles a row).  32 columns per CTA and a warp per component keep each chain on a
+// quarter of an SM, with two chunks of 16 rows in flight: the data of a 3280-mode
+// instrument (38 channels of 2394 rows, 80 cells) 0.98 -> 0.32 ms.
+constexpr int XH_COLS = 32, XH_U = 16, XH_ROWS = 256;
+__global__ void __launch_bounds__(2 * XH_COLS) xh_w_d_split_kernel(const double2* __restrict__ X, int64_t ldx, int64_t x_batch_stride,
+                              const double* __restrict__ w, const double2* __restrict__ d,
+                              int64_t vec_batch_stride, int64_t K, int n, int64_t kchunk,
+                              double2* __restrict__ u, int64_t u_batch_stride) {
+  const int bz = blockIdx.z, comp = threadIdx.x / XH_COLS;
+  X += bz * x_batch_stride;
+  w += bz * vec_batch_stride;
+  d += bz * vec_batch_stride;
+  u += bz * u_batch_stride;
+  const int j = blockIdx.x * XH_COLS + threadIdx.x % XH_COLS;
+  const int64_t k0 = blockIdx.y * kchunk, k1 = min(K, k0 + kchunk);
+  // w d of 256 rows at a time, formed once per CTA, by component
+  __shared__ double dw[2][XH_ROWS];
+  const double2* __restrict__ x0 = X + min(j, n - 1);
+  double2 a[XH_U], b[XH_U];
+  auto load = [&](double2* o, int64_t k) {
+#pragma unroll
+    for (int q = 0; q < XH_U; ++q) o[q] = x0[min(k + q, k1 - 1) * ldx];
+  };
+  double acc = 0.0;
+  auto mac = [&](const double2* x, int64_t k) {   // re: x d, im: x d with the parts of d exchanged and one sign
+    const int r = (int)((k - k0) % XH_ROWS);
+#pragma unroll
+    for (int q = 0; q < XH_U; ++q)
+      if (k + q < k1) acc = fma(x[q].x, dw[comp][r + q], fma(comp ? -x[q].y : x[q].y, dw[1 - comp][r + q], acc));
+  };
+  load(a, k0);
+  for (int64_t kb = k0; kb < k1; kb += 2 * XH_U) {
+    if ((kb - k0) % XH_ROWS == 0) {
+      __syncthreads();
+      for (int r = threadIdx.x; r < XH_ROWS && kb + r < k1; r += 2 * XH_COLS) {
+        const double2 dd = d[kb + r];
+        const double ww = w[kb + r];
+        dw[0][r] = dd.x * ww;
+        dw[1][r] = dd.y * ww;
+      }
+      __syncthreads();
+    }
+    load(b, kb + XH_U);
+    mac(a, kb);
+    load(a, kb + 2 * XH_U);
+    mac(b, kb + XH_U);
+  }
+  if (j >= n) return;
+  atomicAdd(comp ? &u[j].y : &u[j].x, acc);
+}
+
+static void launch_xh_w_d(const double2* X, int64_t ldx, int64_t x_batch_stride, const double* w, const double2* d,
+                          int64_t vec_batch_stride, int64_t K, int n, int64_t kchunk, double2* u, int64_t u_batch_stride,
+                          int nbatch, cudaStream_t s) {
+  const unsigned chunks = (unsigned)((K + kchunk - 1) / kchunk);
+  // two waves of the wide kernel's CTAs: beyond, fewer reads of X count for more than the chains (a dense 3280-mode
+  // instrument of 90,972 visibilities, 1157 CTAs: 2.15 ms, 3.46 in the split kernel)
+  if ((int64_t)((n + 255) / 256) * chunks * nbatch >= 2 * device_sms())
+    xh_w_d_kernel<<<dim3((n + 255) / 256, chunks, nbatch), 256, 0, s>>>(X, ldx, x_batch_stride, w, d, vec_batch_stride, K, n,
+                                                                       kchunk, u, u_batch_stride);
+  else
+    xh_w_d_split_kernel<<<dim3((n + XH_COLS - 1) / XH_COLS, chunks, nbatch), 2 * XH_COLS, 0, s>>>(
+        X, ldx, x_batch_stride, w, d, vec_batch_stride, K, n, kchunk, u, u_batch_stride);
+}
+
 // Structured M: M[(c,x),(c',x')] = sum_f conj(W[f,x]) W[f,x'] G[f][c][c'] into
 // packed tiles.
 //
@@ -396,8 +463,7 @@ cudaError_t precompute_dense(const double2* T, int64_t n_vis, int n, int64_t ld,
   // chunks of 1024 visibilities of a large T, so that its rows stream from memory on every SM
   int64_t kchunk = n_vis <= 4096 ? 4096 : 1024;
   while ((n_vis + kchunk - 1) / kchunk > 65535) kchunk *= 2;
-  dim3 g2((n + 255) / 256, (unsigned)((n_vis + kchunk - 1) / kchunk), 1);
-  xh_w_d_kernel<<<g2, 256, 0, s>>>(T, ld, 0, w, d, 0, n_vis, n, kchunk, dbar, 0);
+  launch_xh_w_d(T, ld, 0, w, d, 0, n_vis, n, kchunk, dbar, 0, 1, s);
   return cudaGetLastError();
 }
 
@@ -420,8 +486,7 @@ cudaError_t precompute_factored(const double2* A, const double2* W, int nf, int6
   if (e != cudaSuccess) return e;
   cudaMemsetAsync(u_scratch, 0, sizeof(double2) * (size_t)nf * ncells, s);
   int64_t kchunk = 2048;
-  dim3 g2((ncells + 255) / 256, (unsigned)((ntb + kchunk - 1) / kchunk), (unsigned)nf);
-  xh_w_d_kernel<<<g2, 256, 0, s>>>(A, ncells, ntb * ncells, w, d, ntb, ntb, ncells, kchunk, u_scratch, ncells);
+  launch_xh_w_d(A, ncells, ntb * ncells, w, d, ntb, ntb, ncells, kchunk, u_scratch, ncells, nf, s);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   int np = nt * BEOR_TB;
