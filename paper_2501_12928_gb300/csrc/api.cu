@@ -1217,9 +1217,14 @@ int beor_get_M(beor_ctx* c, beor_c128* M_out) {
     CKC(c, cudaDeviceSynchronize());
     return BEOR_OK;
   }
-  const int64_t band = std::max<int64_t>(1, std::min<int64_t>(n, ((int64_t)1 << 24) / n));
+  int64_t band = std::max<int64_t>(1, std::min<int64_t>(n, ((int64_t)1 << 24) / n));
   DevBuf buf;
-  CKC(c, buf.alloc(sizeof(double2) * (size_t)(band * n)));
+  cudaError_t e = buf.alloc(sizeof(double2) * (size_t)(band * n));
+  for (; e == cudaErrorMemoryAllocation && band > 1; e = buf.alloc(sizeof(double2) * (size_t)(band * n))) {
+    cudaGetLastError();
+    band = (band + 1) / 2;   // on a full device
+  }
+  CKC(c, e);
   for (int64_t r0 = 0; r0 < n; r0 += band) {
     const int64_t rows = std::min(band, n - r0);
     CKC(c, unpack_hermitian(c->M.as<double2>(), c->n, r0, rows, buf.as<double2>(), 0));
