@@ -262,12 +262,12 @@ int beor_set_lookahead(int on);
 /* Schedule of the batched mixed-precision factorisation (the blocked
  * right-looking Cholesky of every problem of a batch, run as a sequence of
  * batched launches per block step, captured in one CUDA graph).  None of
- * these settings changes an operation on any tile: factors and
- * log-determinants are identical under every schedule (the float64
- * residual of the quadratic form sums with atomics, so lnL may differ in
- * its last bits).
+ * these settings changes an operation on any tile: factors,
+ * log-determinants and the residual's sums are identical under every
+ * schedule.
  *   lookahead:  1 = block step k's trailing update is split into the next
- *               block column (high priority, main stream) and the rest
+ *               diagonal block (high priority, main stream), the tiles
+ *               below it (high priority, second stream) and the rest
  *               (low priority, second stream), so that the diagonal block,
  *               slicing and panel of step k + 1 overlap the rest of step k;
  *               0 = one stream, steps in order.
@@ -280,8 +280,9 @@ int beor_set_lookahead(int on);
  *               steps overlap); 0 = all start on step 0.
  *   reserve_diag: 1 = each launch for columns j >= k + 2 also leaves free as
  *               many SMs as step k + 1's diagonal blocks take (one, two or
- *               four CTAs per problem, running beside it at high priority), so
- *               that they start at once; 0 = no such reserve. */
+ *               four CTAs per problem, eight for a posterior mean, running
+ *               beside it at high priority), so that they start at once;
+ *               0 = no such reserve. */
 typedef struct {
   int lookahead;
   int rest_ctas;
