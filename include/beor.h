@@ -278,10 +278,10 @@ int beor_set_lookahead(int on);
  *   align_ends: 1 = in a batch of uneven sizes, smaller problems start late
  *               so that all end on the last block step (their light final
  *               steps overlap); 0 = all start on step 0.
- *   reserve_diag: 1 = each launch for columns j >= k + 2 also leaves free as
- *               many SMs as step k + 1's diagonal blocks take (one, two or
- *               four CTAs per problem, eight for a posterior mean, running
- *               beside it at high priority), so that they start at once;
+ *   reserve_diag: 1 = each launch for columns j >= k + 2 also leaves SMs free
+ *               for step k + 1's diagonal blocks, which run beside it at high
+ *               priority: as many as their clusters have CTAs, but no more
+ *               than 32 or one per problem, whichever is larger;
  *               0 = no such reserve. */
 typedef struct {
   int lookahead;

@@ -304,11 +304,15 @@ cudaError_t run_sequence(Plan& pl, cudaStream_t s, int64_t* nlaunch, bool mark) 
       RUN_ON(KC_SOLVE, pl.side2, launch_fwd_step(v, true, v.vec_b, k, pl.side2));
       L += fwd_step_launches(v, k);
       if (mixed_tiles(pl.maps, 1, k) > 0) {
-        // reserve_diag: leave free the SMs that step k + 1's diagonal blocks
-        // (running beside this launch) need
+        // reserve_diag: leave SMs free for step k + 1's diagonal blocks, which
+        // run beside this launch: as many as their clusters have CTAs in a small
+        // batch, one per problem in a large one (with its 128 CTAs' SMs left
+        // free, 64 points of 3280 modes took 139 instead of 45 ms)
         int cap = 0;
-        if (pl.sch.reserve_diag)
-          cap = std::max(8, device_sms() - (v.mean ? DIAG_MEAN_CTAS : diag_tc_ctas(active(k + 1))));
+        if (pl.sch.reserve_diag) {
+          const int n = active(k + 1), ctas = v.mean ? DIAG_MEAN_CTAS : diag_tc_ctas(n);
+          cap = std::max(8, device_sms() - std::min(ctas, std::max(n, 32)));
+        }
         RUN_ON(KC_TRAIL, pl.side, launch_trail_mixed(v, pl.maps, k, TRAIL_REST, pl.side, 0, cap));
         L += trail_launch_count(pl.maps, k, TRAIL_REST);
       }

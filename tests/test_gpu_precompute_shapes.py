@@ -89,3 +89,19 @@ def test_factored_weights(P, ncells, nx):
     lk.set_data(d, var)
     lk.precompute()
     _close(lk.get_M(), O.herm_structured(A, W, var))
+
+
+def test_dense_dbar_of_many_chunks(P):
+    """Enough chunks of visibilities for the wide kernel.  Bound: chains of 1024
+    rows, the product with the weight and 320 chunk sums, each step within 2^-53 of
+    the sum of magnitudes."""
+    nvis, n = 327680, 3
+    p = random_problem(nvis, n, 2, seed=5)
+    lk = P.Likelihood("fp64")
+    lk.set_T(p["T"], p["kbin"], 2, 2.0)
+    lk.set_data(p["d"], p["noise_var"])
+    lk.precompute()
+    wd = p["d"] / p["noise_var"]
+    ref = np.array([np.sum((np.conj(p["T"][:, j]) * wd).astype(np.clongdouble)) for j in range(n)])
+    mag = np.abs(p["T"]).T @ np.abs(wd)
+    assert np.all(np.abs(lk.get_dbar() - ref) <= 2 * (1024 + 320 + 8) * 2.0 ** -53 * mag)
