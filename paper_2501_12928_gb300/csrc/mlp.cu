@@ -106,9 +106,9 @@ constexpr int rows_smem(int depth) {
 // layers is latency), MT = 4 with two CTAs per SM, one's GELUs beside the
 // other's products, where every SM has rows enough: each CTA reads all the
 // weights (0.5 MB) from L2.  64 rows through 256 x 4: 15 us (five layers'
-// launches of 14 us before), 20,000 rows: 71 us (219 us), of which the products
-// take 35 at the rate of mma.sync and the rest is GELU and a second wave of 9
-// of the 313 CTAs.
+// launches of 14 us before), 20,000 rows: 66 us (219 us), of which the products
+// take 35 at the rate of mma.sync and the rest is GELU and the rows beyond a
+// whole wave.  (Sixteen warps of 16 columns: the same times.)
 template <int MT, int ST, bool TRAIN>
 __global__ void __launch_bounds__(kThreads) rows_kernel(const __grid_constant__ Net g) {
   extern __shared__ __align__(16) __nv_bfloat16 sm_rows[];
@@ -602,7 +602,18 @@ cudaError_t predict(beor_mlp* m, const float* x, int n, float* y, cudaStream_t s
   Net g = net_of(m, x, n);
   g.y = y;
   if (n <= 16 * 2 * sm_count()) return launch_rows<1, 5, false>(g, s);
-  return launch_rows<4, 2, false>(g, s);
+  // whole waves of 64 rows and two CTAs per SM (50 us); a short rest goes 16 rows
+  // to a CTA, 16 us on idle SMs, where the start of another wave takes 21: 20,000
+  // rows 66 us, 71 in one launch
+  const int wave = 64 * 2 * sm_count(), rest = n % wave;
+  if (rest == 0 || rest > 16 * sm_count() || n < wave) return launch_rows<4, 2, false>(g, s);
+  g.n = n - rest;
+  const cudaError_t e = launch_rows<4, 2, false>(g, s);
+  if (e != cudaSuccess) return e;
+  g.x += (int64_t)g.n * g.n_in;
+  g.y += g.n;
+  g.n = rest;
+  return launch_rows<1, 5, false>(g, s);
 }
 
 // loss, and gradients of every parameter or one Adam step (device x and t)

@@ -78,3 +78,13 @@ def test_gradients_and_adam_step(n_in, width, depth):
             # 12 roundings of the step, and 1 - b2 in float32 (2^-24 / 0.001 of v, half of it in the step)
             tol = lr * (12 * 2.0 ** -24 + 2.0 ** -24 / 0.001) + 2.0 ** -24 * np.abs(p).max()
             assert np.abs(q - want).max() <= tol
+
+
+@pytest.mark.parametrize("n_in,width,depth", [(9, 48, 2), (9, 256, 4)])
+def test_forward_of_many_rows(n_in, width, depth):
+    """Whole waves of rows and a rest (on 152 SMs 19,456 rows and up to 2,432)."""
+    em, _, _ = _emulator(n_in, width, depth)
+    x, _ = _data(41500, n_in)
+    y = np.concatenate([em.infer(x[i:i + 4000]) for i in range(0, len(x), 4000)])
+    for n in (19455, 19456, 19457, 21888, 21889, 38912, 38913, 41500):
+        np.testing.assert_array_equal(em.infer(x[:n]), y[:n])
