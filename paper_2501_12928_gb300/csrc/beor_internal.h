@@ -143,8 +143,12 @@ int diag_tc_ctas(int active);   // CTAs of its launch
 constexpr int DIAG_MEAN_CTAS = 8;   // and of the posterior mean's
 // diag_cluster.cu: diagonal blocks of the float64 path and of the posterior mean
 cudaError_t launch_diag_cluster(const BatchView& v, int k, bool mixed, int active, cudaStream_t s, int prio);
+// chol.cu
 cudaError_t launch_panel_f64(const BatchView& v, int k, cudaStream_t s);
 cudaError_t launch_trail_f64(const BatchView& v, int k, cudaStream_t s);
+cudaError_t launch_lnl(const BatchView& v, cudaStream_t s, int corr);   // corr: residual-corrected q
+cudaError_t launch_copy_dbar(const BatchView& v, cudaStream_t s);
+// solve.cu (both precisions)
 cudaError_t launch_solve(const BatchView& v, bool mixed, const double2* rhs, double2* out, cudaStream_t s);
 // The solve's two halves: forward step k (0 .. max_nt - 1) of vec_y = L^-1 rhs, the
 // whole forward pass, and the whole backward pass out = L^-H vec_y.
@@ -152,9 +156,7 @@ cudaError_t launch_fwd_step(const BatchView& v, bool mixed, const double2* rhs, 
 int fwd_step_launches(const BatchView& v, int k);
 cudaError_t launch_bwd(const BatchView& v, bool mixed, double2* out, cudaStream_t s);
 int solve_pass_launches(const BatchView& v);   // of a whole pass
-cudaError_t launch_lnl(const BatchView& v, cudaStream_t s, int corr);   // corr: residual-corrected q
 cudaError_t launch_solve_fwd(const BatchView& v, bool mixed, const double2* rhs, cudaStream_t s);   // vec_y = L^-1 rhs
-cudaError_t launch_copy_dbar(const BatchView& v, cudaStream_t s);
 
 // mixed.cu
 struct MixedMaps;  // opaque TMA descriptors of one batch

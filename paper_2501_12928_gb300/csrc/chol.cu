@@ -1,15 +1,12 @@
 // Blocked right-looking complex Cholesky of Sigma = M + Phi^-1 for a batch of
-// problems, the triangular solves for abar = Sigma^-1 dbar, and the lnL
-// assembly (lnL = -1/2 log|Phi| - 1/2 log|Sigma| + 1/2 dbar^H abar).
+// problems, and the lnL assembly (lnL = -1/2 log|Phi| - 1/2 log|Sigma| + 1/2
+// dbar^H abar).
 //
-// Kernels here serve both precisions:
 //  * prior / init:  Phi^-1 from phi (one amplitude per k bin, Eq. for P(k_i)),
 //                   log|Phi|, and the working matrix W = M + diag(Phi^-1);
-//  * diag:          float64 factorisation of the 128 x 128 diagonal block,
-//                   log|Sigma| accumulation, status, and its inverse (float64;
-//                   on the fp32 pipe, with bf16 slices, on the mixed path);
+//  * diag:          choice of the diagonal blocks' kernel (diag_tc.cu,
+//                   diag_cluster.cu);
 //  * panel/trail:   float64 tile GEMMs (the float64 comparator path);
-//  * solve:         blocked forward / backward substitution;
 //  * lnl:           q = Re(dbar^H abar), or its residual-corrected form, and lnL.
 #include <algorithm>
 #include <cmath>
