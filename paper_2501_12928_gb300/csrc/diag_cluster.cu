@@ -17,7 +17,8 @@
 // The inverse goes by columns, which do not depend on each other, from the copy
 // of L that every CTA then has.  One point of 3280 modes, one CTA with barriers
 // per column -> eight: float64 1.16 ms -> 0.39 per block, posterior mean 0.79 ->
-// 0.33; with the pivots' square roots and reciprocals from integers 0.35 and 0.30.
+// 0.33; with the pivots' square roots and reciprocals from integers 0.35 and
+// 0.30; with the posterior mean's 32 x 32 inverses dealt by columns 0.28.
 #include <cooperative_groups.h>
 
 #include <cmath>
@@ -92,34 +93,31 @@ __device__ __forceinline__ dfl df_add_quick(dfl x, dfl y) {
   const dfl t = df_two_sum(x.hi, y.hi);
   return dfl{t.hi, t.lo + (x.lo + y.lo)};
 }
-// Barrier of the 128 threads (four warps) of group id - 1.
-__device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
 
-// Inverse of one 32 x 32 diagonal block g of L (packed, double-float Af with
-// third terms Lt), in place, row by row, by the 128 threads of barrier 1 + g.
-// invs: reciprocals of L's diagonal.
-__device__ __forceinline__ void invert_diag32(float4* Af, const float2* Lt, const dfl* invs, int g, int lt) {
-  const int jl = lt >> 2, part = lt & 3, jj = 32 * g + jl;
-  for (int il = 0; il < 32; ++il) {
-    const int i = 32 * g + il;
+// Columns c0 .. c0 + 7 (c0 a multiple of 8) of the inverse of their 32 x 32
+// diagonal block of L (packed, double-float Af with third terms Lt), in place,
+// row by row, by one warp, four lanes per column.  invs: reciprocals of L's
+// diagonal.
+__device__ __forceinline__ void invert_diag_columns(float4* Af, const float2* Lt, const dfl* invs, int c0, int lane) {
+  const int jj = c0 + (lane >> 2), part = lane & 3;
+#pragma unroll 1
+  for (int i = c0; i < (c0 | 31) + 1; ++i) {
     dfl c[4] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
-    if (jl < il)
-      for (int m = jj + part; m < i; m += 4) cmac_l(c, Af[pk(i, m)], Lt[pk(i, m)], Af[pk(m, jj)]);
+    for (int m = jj + part; m < i; m += 4) cmac_l(c, Af[pk(i, m)], Lt[pk(i, m)], Af[pk(m, jj)]);
     dfl sr = df_add_quick(c[0], c[1]), si = df_add_quick(c[2], c[3]);
 #pragma unroll
     for (int o = 1; o <= 2; o <<= 1) {
       sr = df_add_quick(sr, dfl{__shfl_xor_sync(0xffffffffu, sr.hi, o), __shfl_xor_sync(0xffffffffu, sr.lo, o)});
       si = df_add_quick(si, dfl{__shfl_xor_sync(0xffffffffu, si.hi, o), __shfl_xor_sync(0xffffffffu, si.lo, o)});
     }
-    group_sync(1 + g);   // every read of row i (as L) is done
-    if (jl < il && part == 0) {
+    __syncwarp();   // every read of row i (as L) is done
+    if (jj <= i && part == 0) {
       const dfl inv = invs[i];
       const dfl qr = df_mul(df_fast_two_sum(sr.hi, sr.lo), inv);
       const dfl qi = df_mul(df_fast_two_sum(si.hi, si.lo), inv);
-      Af[pk(i, jj)] = make_float4(-qr.hi, -qr.lo, -qi.hi, -qi.lo);
+      Af[pk(i, jj)] = jj < i ? make_float4(-qr.hi, -qr.lo, -qi.hi, -qi.lo) : make_float4(inv.hi, inv.lo, 0.0f, 0.0f);
     }
-    if (lt == 0) Af[pk(i, i)] = make_float4(invs[i].hi, invs[i].lo, 0.0f, 0.0f);
-    group_sync(1 + g);   // row i of Linv is complete
+    __syncwarp();   // row i of these columns is complete
   }
 }
 
@@ -374,7 +372,8 @@ __global__ void __launch_bounds__(DC_THREADS, 1) diag_cluster_kernel(BatchView v
     // 40-bit panel slices and the solves only.  Exact float triples of L (each
     // CTA splits its share for all), so that each product keeps its terms down
     // to 2^-48 of the leading part (Dot2 accumulation); Linv is held as
-    // double-float.  Blocked by 32: the diagonal blocks row by row in every CTA,
+    // double-float.  Blocked by 32: the own columns of the diagonal blocks row by
+    // row, sent to every CTA (all columns in every CTA: 83,000 of 590,000 cycles),
     // then X_IJ = sum_{M=J}^{I-1} L_IM Linv_MJ and Linv_IJ = -Linv_II X_IJ for
     // the own columns (blocks of eight, dealt like the rows).
     float4* Af = reinterpret_cast<float4*>(A);
@@ -398,8 +397,17 @@ __global__ void __launch_bounds__(DC_THREADS, 1) diag_cluster_kernel(BatchView v
       sm.invs[tid] = df_from_double(1.0 / ((double)d.x + (double)d.y + (double)Lt[pk(tid, tid)].x));
     }
     __syncthreads();
-    invert_diag32(Af, Lt, sm.invs, tid >> 7, tid & 127);
-    __syncthreads();
+    if (warp < NBLK) invert_diag_columns(Af, Lt, sm.invs, 8 * dc_block<C>(rank, warp), lane);
+    cg::this_cluster().sync();   // L's diagonal blocks are read everywhere
+    for (int e = tid; e < NBLK * 256; e += DC_THREADS) {
+      const int c0 = 8 * dc_block<C>(rank, e >> 8), i = (c0 & ~31) + ((e >> 3) & 31), jj = c0 + (e & 7);
+      if (i < jj) continue;
+      const float4 f = Af[pk(i, jj)];
+#pragma unroll
+      for (int c = 0; c < C; ++c)
+        if (c != rank) dc_peer(Af, c)[pk(i, jj)] = f;
+    }
+    cg::this_cluster().sync();
     // block row I: X_IJ = sum_{m=jj}^{32 I - 1} L[i][m] Linv[m][jj], then Linv_IJ = -Linv_II X_IJ
     constexpr int NQ = NBLK / 2;   // outputs per thread: two blocks of eight columns x 32 rows at a time
     const int cr = (tid >> 3) & 31, cc = tid & 7;
