@@ -452,14 +452,20 @@ __global__ void to_bf16_kernel(const float* __restrict__ W, int rows, int cols, 
   Wb[(int64_t)r * ldb + c] = __float2bfloat16_rn(W[e]);
 }
 
-bool on_device(const void* p) {
+// Where a caller's array lies: host memory, device memory, or device memory that
+// the kernels of `device` may address as it stands (that device's own, on a float
+// boundary; anything else a copy reaches, and only a copy).
+enum Where { HOST, DEVICE, HERE };
+Where where_is(const void* p, int device) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return HOST;
   }
-  return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+  if (a.type == cudaMemoryTypeDevice && a.device == device && reinterpret_cast<uintptr_t>(p) % alignof(float) == 0) return HERE;
+  return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged ? DEVICE : HOST;
 }
+bool on_device(const void* p) { return where_is(p, -1) != HOST; }
 
 int pad16(int x) { return (x + 15) / 16 * 16; }
 
@@ -740,19 +746,26 @@ int beor_mlp_infer(beor_mlp* m, const float* x, int n, float* y_out, void* strea
   cudaSetDevice(m->device);
   cudaStream_t s = (cudaStream_t)stream;
   const int chunk = 65536;
-  const bool dev_in = on_device(x), dev_out = on_device(y_out);
-  if ((!dev_in || !dev_out) && ensure_io(m, std::min(n, chunk)) != cudaSuccess) return BEOR_ENOMEM;
+  // In place where the kernel may address the caller's memory; predictions that
+  // would go over inputs which other CTAs have yet to read are copied out after
+  // the chunk's kernel, as those to other memory are.
+  const uintptr_t x0 = reinterpret_cast<uintptr_t>(x), y0 = reinterpret_cast<uintptr_t>(y_out);
+  const bool apart = y0 + sizeof(float) * (size_t)n <= x0 || x0 + sizeof(float) * (size_t)n * m->n_in <= y0;
+  const Where xw = where_is(x, m->device), yw = where_is(y_out, m->device);
+  const bool x_here = xw == HERE, y_here = yw == HERE && (apart || !x_here), dev_out = yw != HOST;
+  if ((!x_here || !y_here) && ensure_io(m, std::min(n, chunk)) != cudaSuccess) return BEOR_ENOMEM;
   for (int off = 0; off < n; off += chunk) {
     const int c = std::min(chunk, n - off);
     const float* xc = x + (int64_t)off * m->n_in;
-    if (!dev_in) {
-      if (cudaMemcpyAsync(m->xin, xc, sizeof(float) * (size_t)c * m->n_in, cudaMemcpyHostToDevice, s) != cudaSuccess)
+    if (!x_here) {
+      if (cudaMemcpyAsync(m->xin, xc, sizeof(float) * (size_t)c * m->n_in,
+                          xw == HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return BEOR_ECUDA;
       xc = m->xin;
     }
-    if (predict(m, xc, c, dev_out ? y_out + off : m->yout, s) != cudaSuccess) return BEOR_ECUDA;
-    if (!dev_out &&
-        cudaMemcpyAsync(y_out + off, m->yout, sizeof(float) * c, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    if (predict(m, xc, c, y_here ? y_out + off : m->yout, s) != cudaSuccess) return BEOR_ECUDA;
+    if (!y_here && cudaMemcpyAsync(y_out + off, m->yout, sizeof(float) * c,
+                                   dev_out ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s) != cudaSuccess)
       return BEOR_ECUDA;
   }
   if (!dev_out && cudaStreamSynchronize(s) != cudaSuccess) return BEOR_ECUDA;

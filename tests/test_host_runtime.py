@@ -1,0 +1,82 @@
+"""Host code of the library on a CUDA runtime without a GPU (fake_cudart.cpp): the
+paths of a call that its kernels' results do not depend on."""
+
+import ctypes
+import glob
+import os
+import re
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2501_12928_gb300 import _build, beor
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+STREAM = 0x1000   # any stream but the null one
+
+
+@pytest.fixture(scope="module")
+def fake_library(tmp_path_factory):
+    if shutil.which("g++") is None or (shutil.which("nvcc") is None and not os.path.exists(_build._nvcc())):
+        pytest.skip("no compiler")
+    objs = [os.path.join(_build.OUT_DIR, s.replace(".cu", ".o")) for s in _build.SOURCES]
+    newest = max(map(os.path.getmtime, glob.glob(os.path.join(_build.CSRC, "*")) + [_build.__file__]))
+    if not all(os.path.exists(o) and os.path.getmtime(o) > newest for o in objs):
+        _build.build()
+    lib = str(tmp_path_factory.mktemp("fake") / "libbeor_fake.so")
+    include = os.path.join(os.path.dirname(os.path.dirname(_build._nvcc())) or "/usr/local/cuda", "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I", include, "-o", lib,
+                    os.path.join(HERE, "fake_cudart.cpp"), *objs], check=True)
+    return lib
+
+
+@pytest.fixture
+def fake(fake_library, tmp_path, monkeypatch):
+    """The package on a copy of its own, so that nothing is left from another test."""
+    monkeypatch.setattr(beor, "LIB_PATH", shutil.copy(fake_library, tmp_path))
+    lib = beor._load()
+    lib.fake_log.restype = ctypes.c_char_p
+    lib.fake_used.restype = ctypes.c_size_t
+    lib.fake_set_total.argtypes = [ctypes.c_int, ctypes.c_size_t]
+    monkeypatch.setattr(beor, "lib", lib)
+    return lib
+
+
+class Array:
+    """Device memory with what the package asks of a tensor."""
+
+    def __init__(self, lib, device, nbytes, offset=0):
+        p = ctypes.c_void_p()
+        lib.cudaSetDevice(device)
+        assert lib.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(nbytes)) == 0
+        self.address = p.value + offset
+
+
+def _copies(lib, key, address):
+    """Copies from (key 2) or to (key 1) an address: their sizes."""
+    rows = [r.split() for r in lib.fake_log().decode().splitlines() if r.startswith("copy")]
+    return [int(r[3]) for r in rows if int(r[key]) == address]
+
+
+N_IN, N = 3, 5000
+
+
+@pytest.mark.parametrize("where_x, where_y, copies", [
+    ("own", "own", (0, 0)), ("other", "own", (1, 0)), ("own", "other", (0, 1)), ("host", "own", (1, 0)),
+    ("own", "head of x", (0, 1)), ("own", "last of x", (0, 1)), ("own", "behind x", (0, 0)), ("odd", "odd", (1, 1))])
+def test_predictions_in_place_only_where_the_kernel_may(fake, where_x, where_y, copies):
+    """The kernel addresses the caller's arrays only if they are its own device's,
+    aligned and apart; otherwise inputs and predictions are copied."""
+    em = beor.Emulator(N_IN, 16, 1, device=0)
+    x_bytes, host = 4 * N_IN * N, np.zeros((N, N_IN), np.float32)
+    base = Array(fake, 1 if where_x == "other" else 0, x_bytes + 4 * N + 4, 1 if where_x == "odd" else 0)
+    x = host.ctypes.data if where_x == "host" else base.address
+    y = {"head of x": x, "last of x": x + x_bytes - 4, "behind x": x + x_bytes}.get(where_y) or Array(
+        fake, 1 if where_y == "other" else 0, 4 * N + 4, 1 if where_y == "odd" else 0).address
+    fake.fake_clear_log()
+    assert fake.beor_mlp_infer(em._h, x, N, y, STREAM) == 0
+    assert _copies(fake, 2, x) == [x_bytes] * copies[0]
+    assert _copies(fake, 1, y) == [4 * N] * copies[1]
+    assert re.search("launch 0 .*rows_kernel", fake.fake_log().decode())
