@@ -40,6 +40,17 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// memory of that very device, aligned: a kernel may address it as it stands
+// (other device memory a copy reaches, and only a copy)
+bool kernel_may_address(const void* p, int device, size_t align) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == device && reinterpret_cast<uintptr_t>(p) % align == 0;
+}
+
 // copy n bytes from a host-or-device source to device memory
 cudaError_t to_device(void* dst, const void* src, size_t n, cudaStream_t s) {
   return cudaMemcpyAsync(dst, src, n, is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
@@ -1213,11 +1224,11 @@ int beor_get_M(beor_ctx* c, beor_c128* M_out) {
   if (r) return r;
   if (!c->have_pre || !M_out) return c->have_pre ? BEOR_EINVAL : BEOR_ESTATE;
   cudaSetDevice(c->device);
-  // unpacked on the device, by bands of rows of up to 256 MB for a host output
+  // unpacked on the device, by bands of rows of up to 256 MB unless the kernel may
+  // store to the output itself (16 bytes at a time; beor_c128 is aligned to 8)
   const int64_t n = c->n;
-  double2* out = reinterpret_cast<double2*>(M_out);
-  if (is_device_ptr(M_out)) {
-    CKC(c, unpack_hermitian(c->M.as<double2>(), c->n, 0, n, out, 0));
+  if (kernel_may_address(M_out, c->device, sizeof(double2))) {
+    CKC(c, unpack_hermitian(c->M.as<double2>(), c->n, 0, n, reinterpret_cast<double2*>(M_out), 0));
     CKC(c, cudaDeviceSynchronize());
     return BEOR_OK;
   }
@@ -1232,8 +1243,9 @@ int beor_get_M(beor_ctx* c, beor_c128* M_out) {
   for (int64_t r0 = 0; r0 < n; r0 += band) {
     const int64_t rows = std::min(band, n - r0);
     CKC(c, unpack_hermitian(c->M.as<double2>(), c->n, r0, rows, buf.as<double2>(), 0));
-    CKC(c, cudaMemcpy(out + r0 * n, buf.p, sizeof(double2) * (size_t)(rows * n), cudaMemcpyDeviceToHost));
+    CKC(c, from_device(M_out + r0 * n, buf.p, sizeof(double2) * (size_t)(rows * n), 0));
   }
+  CKC(c, cudaDeviceSynchronize());
   return BEOR_OK;
 }
 

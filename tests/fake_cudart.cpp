@@ -94,7 +94,10 @@ API cudaError_t cudaSetDevice(int d) {
   return cudaSuccess;
 }
 API cudaError_t cudaGetDevice(int* d) { return *d = g_device, cudaSuccess; }
-API cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
+API cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
+  *v = a == cudaDevAttrComputeCapabilityMajor ? 10 : a == cudaDevAttrComputeCapabilityMinor ? 3 : 152;
+  return cudaSuccess;
+}
 API cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int) {
   std::memset(p, 0, sizeof(*p));
   p->major = 10;

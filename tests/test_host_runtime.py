@@ -80,3 +80,27 @@ def test_predictions_in_place_only_where_the_kernel_may(fake, where_x, where_y, 
     assert _copies(fake, 2, x) == [x_bytes] * copies[0]
     assert _copies(fake, 1, y) == [4 * N] * copies[1]
     assert re.search("launch 0 .*rows_kernel", fake.fake_log().decode())
+
+
+def _like(lib, n=140, n_vis=200, precision="mixed", device=0):
+    from synth.instrument import random_problem
+    p = random_problem(n_vis, n, 3, seed=n)
+    lk = beor.Likelihood(precision, device)
+    lk.set_T(p["T"], p["kbin"], 3, 2.0)
+    lk.set_data(p["d"], p["noise_var"])
+    lk.precompute(STREAM)
+    return lk, p
+
+
+@pytest.mark.parametrize("where, copied", [("own", False), ("own, 8 bytes on", True), ("other", True), ("host", True)])
+def test_normal_matrix_stored_by_the_kernel_only_where_it_may(fake, where, copied):
+    """16-byte stores go to 16-byte aligned memory of the context's own device; a
+    beor_c128 is aligned to 8 bytes, and other memory takes a copy."""
+    lk, p = _like(fake)
+    n = p["T"].shape[1]
+    host = np.zeros((n, n), np.complex128)
+    out = host.ctypes.data if where == "host" else Array(fake, where == "other", 16 * n * n + 8, 8 * ("8" in where)).address
+    fake.fake_clear_log()
+    assert fake.beor_get_M(lk._h, out) == 0
+    assert _copies(fake, 1, out) == [16 * n * n] * copied
+    assert "unpack_hermitian" in fake.fake_log().decode()
