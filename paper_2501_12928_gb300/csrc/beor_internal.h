@@ -7,6 +7,7 @@
 #include <utility>
 
 #include "beor_common.cuh"
+#include "per_device.h"
 
 namespace beor {
 
@@ -177,7 +178,6 @@ cudaError_t launch_panel_mixed(const BatchView& v, const MixedMaps* m, int k, cu
 cudaError_t launch_trail_mixed(const BatchView& v, const MixedMaps* m, int k, int part, cudaStream_t s,
                                int prio = 0, int max_ctas = 0);
 int trail_launch_count(const MixedMaps* m, int k, int part);   // kernels launch_trail_mixed launches
-int device_sms();   // SMs of the current device
 cudaError_t launch_residual(const BatchView& v, cudaStream_t s);      // vec_r = dbar - Sigma x (float64)
 cudaError_t launch_refine_update(const BatchView& v, cudaStream_t s); // x += vec_d; residual norm
 int mixed_supported(int device);

@@ -636,11 +636,11 @@ __global__ void __launch_bounds__(512) diag_f64_kernel(BatchView v, int kg) {
 template <typename WS, int C>
 static int dc_fit() {   // blocks that are factored at once
   constexpr size_t smem = dc_smem<std::is_same<WS, float4>::value>();
-  static const int n = [] {   // once: the kernel's attribute, and the device's answer
-    cudaFuncSetAttribute(diag_cluster_kernel<WS, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static PerDevice<int> fit;
+  return fit.get([] {   // once: the kernel's attribute, and the device's answer
+    allow_smem<diag_cluster_kernel<WS, C>>((int)smem);
     return max_clusters(diag_cluster_kernel<WS, C>, DC_THREADS, smem, C);
-  }();
-  return n;
+  });
 }
 template <typename WS, int C>
 static cudaError_t launch_dc(const BatchView& v, int k, cudaStream_t s, int prio) {
@@ -659,8 +659,7 @@ cudaError_t launch_diag_cluster(const BatchView& v, int k, bool mixed, int activ
   if (active <= dc_fit<double2, 4>()) return launch_dc<double2, 4>(v, k, s, prio);
   if (active <= dc_fit<double2, 2>()) return launch_dc<double2, 2>(v, k, s, prio);
   constexpr size_t smem = sizeof(double2) * (DG_PACK + 2 * BEOR_TB);   // packed block and two columns
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(diag_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t attr = allow_smem<diag_f64_kernel>((int)smem);
   if (attr != cudaSuccess) return attr;
   return launch_prio(diag_f64_kernel, dim3(v.P), dim3(512), smem, s, prio, v, k);
 }

@@ -683,11 +683,11 @@ __global__ void __launch_bounds__(DT_THREADS, 1) diag_tc_kernel(BatchView v, int
 
 template <int C>
 static int dt_fit() {   // blocks that are factored at once
-  static const int n = [] {   // once: the kernel's attribute, and the device's answer
-    cudaFuncSetAttribute(diag_tc_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DtSmem));
+  static PerDevice<int> fit;
+  return fit.get([] {   // once: the kernel's attribute, and the device's answer
+    allow_smem<diag_tc_kernel<C>>((int)sizeof(DtSmem));
     return C == 1 ? device_sms() : max_clusters(diag_tc_kernel<C>, DT_THREADS, sizeof(DtSmem), C);
-  }();
-  return n;
+  });
 }
 template <int C>
 static cudaError_t launch_dt(const BatchView& v, int k, cudaStream_t s, int prio) {

@@ -483,16 +483,9 @@ cudaError_t herk_dense_tc(const double2* T, int64_t n_vis, int n, int64_t ld, co
   CUtensorMap ma, mb;
   if (e == cudaSuccess) e = hk_map(&ma, planes, rows, nkb_buf, HK_M, 1);
   if (e == cudaSuccess) e = hk_map(&mb, planes, rows, nkb_buf, HK_N, 2);
-  static bool attr = false;
-  if (e == cudaSuccess && !attr) {
-    e = cudaFuncSetAttribute(herk_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, HK_SMEM);
-    attr = e == cudaSuccess;
-  }
-  int nsm = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = allow_smem<herk_tc_kernel>(HK_SMEM);
   const int64_t ntiles = tri_count(nt) * 2;
-  const int grid = (int)std::min<int64_t>(ntiles, std::max(1, nsm));
+  const int grid = (int)std::min<int64_t>(ntiles, device_sms());
   int* d_ctr = static_cast<int*>(ctr);
   if (e == cudaSuccess) e = cudaMemsetAsync(d_ctr + 1, 0, sizeof(int), s);
   for (int64_t kb0 = 0; kb0 < nkb_total && e == cudaSuccess; kb0 += nkb_buf) {

@@ -615,7 +615,6 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-static int num_sms();
 static __nv_bfloat16* slice_buf(const BatchView& v, int k) {
   return v.panel_sl + (size_t)(k & 1) * BEOR_NPLANE * v.rows * BEOR_TB;
 }
@@ -624,8 +623,7 @@ static int32_t* exp_buf(const BatchView& v, int k) { return v.panel_exp + (size_
 template <int SL_GROUPS>
 static cudaError_t launch_slice(const BatchView& v, int k, cudaStream_t s, int prio) {
   constexpr int smem = (SL_GROUPS > 1 ? 2 : 1) * SL_BUF * (int)sizeof(float4);   // one group, or two in turn
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(slice_panel_kernel<SL_GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t attr = allow_smem<slice_panel_kernel<SL_GROUPS>>(smem);
   if (attr != cudaSuccess) return attr;
   const int nblk = BEOR_TB / (SL_R * SL_GROUPS) * (v.max_nt - 1 - k);   // CTAs of the block rows below block column k
   return launch_prio(slice_panel_kernel<SL_GROUPS>, dim3(nblk, v.P), dim3(256), (size_t)smem, s, prio, v, k,
@@ -640,7 +638,7 @@ cudaError_t launch_slice_panel(const BatchView& v, int k, cudaStream_t s, int pr
   // lnL of 3280 modes in ms (one / four): 1 point 7.06 / 7.55, 8 points 11.05 /
   // 11.26, 12 points 14.28 / 14.28, 32 points 27.9 / 27.2; 700 modes, 32 points
   // 2.30 / 2.33.
-  return (int64_t)(BEOR_TB / SL_R) * (v.max_nt - 1 - k) * v.P <= 12 * num_sms() ? launch_slice<1>(v, k, s, prio)
+  return (int64_t)(BEOR_TB / SL_R) * (v.max_nt - 1 - k) * v.P <= 12 * device_sms() ? launch_slice<1>(v, k, s, prio)
                                                                                   : launch_slice<4>(v, k, s, prio);
 }
 
@@ -737,15 +735,12 @@ cudaError_t mixed_maps_create(const BatchView& v, MixedMaps** out) {
     mixed_maps_destroy(m);
     return e;
   }
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(slice_gemm_kernel<MODE_TRAIL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         Ring<MODE_TRAIL>::smem);
-    cudaFuncSetAttribute(slice_gemm_kernel<MODE_TRAIL_DIAG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         Ring<MODE_TRAIL_DIAG>::smem);
-    cudaFuncSetAttribute(slice_gemm_kernel<MODE_PANEL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         Ring<MODE_PANEL>::smem);
-    attr = true;
+  e = allow_smem<slice_gemm_kernel<MODE_TRAIL>>(Ring<MODE_TRAIL>::smem);
+  if (e == cudaSuccess) e = allow_smem<slice_gemm_kernel<MODE_TRAIL_DIAG>>(Ring<MODE_TRAIL_DIAG>::smem);
+  if (e == cudaSuccess) e = allow_smem<slice_gemm_kernel<MODE_PANEL>>(Ring<MODE_PANEL>::smem);
+  if (e != cudaSuccess) {
+    mixed_maps_destroy(m);
+    return e;
   }
   *out = m;
   return cudaSuccess;
@@ -772,24 +767,13 @@ int64_t mixed_tiles(const MixedMaps* m, int kind, int k) {
   return m->h_total[kind][k] + (diag >= 0 ? m->h_total[diag][k] : 0);
 }
 
-static int num_sms() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
-  }
-  return n;
-}
-
 static cudaError_t launch_gemm(const BatchView& v, const MixedMaps* m, int k, int kind, cudaStream_t s, int prio,
                                int max_ctas = 0) {
   const int64_t nt = m->h_total[kind][k];
   if (nt <= 0) return cudaSuccess;
   int cap = (kind == KIND_REST || kind == KIND_DREST) ? v.grid_rest
             : (kind == KIND_COL || kind == KIND_DCOL || kind == KIND_PANEL) ? v.grid_col : 0;
-  if (cap <= 0) cap = num_sms();
+  if (cap <= 0) cap = device_sms();
   if (max_ctas > 0) cap = std::min(cap, max_ctas);
   const int grid = (int)std::min<int64_t>(nt, cap);
   const int64_t* pre = m->d_prefix + ((size_t)kind * m->max_nt + k) * (m->P + 1);
@@ -831,8 +815,6 @@ int trail_launch_count(const MixedMaps* m, int k, int part) {
   const int kind = part_kind(part), diag = part_diag(part);
   return (kind >= 0 && mixed_tiles_kind(m, kind, k) > 0) + (diag >= 0 && mixed_tiles_kind(m, diag, k) > 0);
 }
-
-int device_sms() { return num_sms(); }
 
 // ---------------------------------------------------------------------------
 // float64 residual: vec_r = dbar - (M + diag Phi^-1) x; refinement: x += vec_d
@@ -1004,12 +986,8 @@ __global__ void resid_sum_kernel(BatchView v) {
 }
 
 cudaError_t launch_residual(const BatchView& v, cudaStream_t s) {
-  static bool attr = false;
-  constexpr int smem = (int)(sizeof(float) * 16 * BEOR_TB * 6);
-  if (!attr) {
-    cudaFuncSetAttribute(resid_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
+  const cudaError_t attr = allow_smem<resid_df_kernel>((int)(sizeof(float) * 16 * BEOR_TB * 6));
+  if (attr != cudaSuccess) return attr;
   xsplit_kernel<<<dim3(8, v.P), 256, 0, s>>>(v);
   resid_df_kernel<<<v.n_rwork, 256, v.rgroup * sizeof(float) * BEOR_TB * 6, s>>>(v);
   resid_sum_kernel<<<dim3((v.max_nt * BEOR_TB + 255) / 256, v.P), 256, 0, s>>>(v);

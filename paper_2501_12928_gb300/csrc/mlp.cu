@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "../../include/beor.h"
+#include "per_device.h"
 
 namespace {
 
@@ -587,32 +588,22 @@ Net net_of(const beor_mlp* m, const float* x, int n) {
 template <int MT, int ST, bool TRAIN>
 cudaError_t launch_rows(const Net& g, cudaStream_t s) {
   constexpr int deepest = TRAIN && ST > 2 ? 4 : kMaxLayers - 1;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      rows_kernel<MT, ST, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem<MT, ST, TRAIN>(deepest));
+  const cudaError_t attr = beor::allow_smem<rows_kernel<MT, ST, TRAIN>>(rows_smem<MT, ST, TRAIN>(deepest));
   if (attr != cudaSuccess) return attr;
   rows_kernel<MT, ST, TRAIN><<<(g.n + 16 * MT - 1) / (16 * MT), kThreads, rows_smem<MT, ST, TRAIN>(g.L - 1), s>>>(g);
   return cudaGetLastError();
-}
-
-int sm_count() {
-  static const int n = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 1;
-  }();
-  return n;
 }
 
 // predictions of n rows (device x and y)
 cudaError_t predict(beor_mlp* m, const float* x, int n, float* y, cudaStream_t s) {
   Net g = net_of(m, x, n);
   g.y = y;
-  if (n <= 16 * 2 * sm_count()) return launch_rows<1, 5, false>(g, s);
+  if (n <= 16 * 2 * beor::device_sms()) return launch_rows<1, 5, false>(g, s);
   // whole waves of 64 rows and two CTAs per SM (50 us); a short rest goes 16 rows
   // to a CTA, 16 us on idle SMs, where the start of another wave takes 21: 20,000
   // rows 66 us, 71 in one launch
-  const int wave = 64 * 2 * sm_count(), rest = n % wave;
-  if (rest == 0 || rest > 16 * sm_count() || n < wave) return launch_rows<4, 2, false>(g, s);
+  const int wave = 64 * 2 * beor::device_sms(), rest = n % wave;
+  if (rest == 0 || rest > 16 * beor::device_sms() || n < wave) return launch_rows<4, 2, false>(g, s);
   g.n = n - rest;
   const cudaError_t e = launch_rows<4, 2, false>(g, s);
   if (e != cudaSuccess) return e;

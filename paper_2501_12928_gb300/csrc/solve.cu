@@ -328,11 +328,9 @@ template <typename WS, typename DV, bool HERM, bool BOTH>
 static cudaError_t launch_block(const BatchView& v, int k, int blocks, const double2* src, double2* out, cudaStream_t s,
                                 bool after) {
   using V = typename std::conditional<std::is_same<WS, float4>::value, dfl, double>::type;
-  auto kern = solve_step_kernel<WS, DV, HERM, BOTH>;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_smem<V>(BOTH));
+  const cudaError_t attr = allow_smem<solve_step_kernel<WS, DV, HERM, BOTH>>((int)solve_smem<V>(BOTH));
   if (attr != cudaSuccess) return attr;
-  return launch_after(kern, dim3(BOTH ? std::max(1, SOLVE_SPLIT * blocks) : 1, v.P), SOLVE_THREADS, solve_smem<V>(BOTH), s,
+  return launch_after(solve_step_kernel<WS, DV, HERM, BOTH>, dim3(BOTH ? std::max(1, SOLVE_SPLIT * blocks) : 1, v.P), SOLVE_THREADS, solve_smem<V>(BOTH), s,
                       after, v, k, src, out);
 }
 // The products with the inverse block in every CTA pay while the first step's CTAs

@@ -94,8 +94,8 @@ API cudaError_t cudaSetDevice(int d) {
   return cudaSuccess;
 }
 API cudaError_t cudaGetDevice(int* d) { return *d = g_device, cudaSuccess; }
-API cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
-  *v = a == cudaDevAttrComputeCapabilityMajor ? 10 : a == cudaDevAttrComputeCapabilityMinor ? 3 : 152;
+API cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int device) {
+  *v = a == cudaDevAttrComputeCapabilityMajor ? 10 : a == cudaDevAttrComputeCapabilityMinor ? 3 : device ? 76 : 152;
   return cudaSuccess;
 }
 API cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int) {

@@ -104,3 +104,38 @@ def test_normal_matrix_stored_by_the_kernel_only_where_it_may(fake, where, copie
     assert fake.beor_get_M(lk._h, out) == 0
     assert _copies(fake, 1, out) == [16 * n * n] * copied
     assert "unpack_hermitian" in fake.fake_log().decode()
+
+
+def _kernels(lib, device):
+    return re.findall(rf"launch {device} (\S+)", lib.fake_log().decode())
+
+
+@pytest.mark.parametrize("first", [0, 1])
+def test_emulators_on_two_devices(fake, first):
+    """A second device allows the kernels their shared memory too, and the split of
+    the rows follows its own number of SMs."""
+    rows = np.zeros((4000, N_IN), np.float32)
+    for device in (first, 1 - first):
+        fake.fake_clear_log()
+        for depth in (1, 8):
+            em = beor.Emulator(N_IN, 32, depth, device=device)
+            for n in (16, 4000):
+                em.train_step(rows[:n], np.zeros(n, np.float32), 1e-3, stream=STREAM)
+                em.infer(rows[:n], stream=STREAM)
+        wide = "rows_kernelILi4ELi2ELb0E"   # 64 rows a CTA: beyond 16 rows on each half of 76 SMs, not of 152
+        assert any(wide in k for k in _kernels(fake, device)) == (device == 1)
+        assert not _kernels(fake, 1 - device)
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("first", [0, 1])
+def test_likelihoods_on_two_devices(fake, first, precision):
+    """The same for the likelihood's kernels, in batches of each size class."""
+    for device in (first, 1 - first):
+        lk, p = _like(fake, 300, 400, precision, device)
+        for B in (1, 20, 70, 200):
+            phi = np.zeros((B, 3))
+            lk.lnl(phi, stream=STREAM)
+            lk.lnl(phi, stream=STREAM)
+        lk.posterior_mean(np.zeros(3), stream=STREAM)
+        assert _kernels(fake, device)
