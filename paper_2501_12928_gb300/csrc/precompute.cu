@@ -312,12 +312,12 @@ __global__ void __launch_bounds__(AM_THREADS)
 #pragma unroll
     for (int q = 0; q < AM_Q; ++q) {
       const int c = J * BEOR_TB + c0 + q * (AM_THREADS / BEOR_TB);
-      on[q] = r < n && c < n;
+      on[q] = r < n && c <= r;   // G's lower triangle; the diagonal tiles' upper halves are zero
       cc[q] = on[q] ? c / nx : 0;
       xc[q] = on[q] ? c % nx : 0;
       vr[q] = vi[q] = 0.0;
     }
-    if (r < n) {
+    if (on[0]) {   // else all four lie above the diagonal or beyond n
 #pragma unroll 2
       for (int f = 0; f < nf; ++f) {
         const double2* __restrict__ g0 = G + ((int64_t)f * ncells + cr) * ncells;
