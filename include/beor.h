@@ -166,8 +166,9 @@ int beor_precompute(beor_ctx *ctx, void *stream);
  * callers with varying B should use a few sizes (e.g. pad to powers of two).
  * New data (beor_set_data, beor_precompute) only end the results' validity:
  * the next call of the shape takes the batch up again.  Such idle batches
- * hold at most a sixteenth of the device's memory in all, and give it back
- * when an allocation of the library does not fit otherwise.
+ * hold at most a sixteenth of the device's memory in all, and no more than is
+ * free beside them at the time of the new data (else they are released then),
+ * and give it back when an allocation of the library does not fit otherwise.
  * Mixed precision: the quadratic form q = dbar^H Sigma^-1 dbar is evaluated
  * from the first solution x~ of the approximate factor L~ and one float64
  * residual r = dbar - Sigma x~ as q = dbar^H x~ + x~^H r + |L~^-1 r|^2

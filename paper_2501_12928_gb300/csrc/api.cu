@@ -61,6 +61,21 @@ cudaError_t from_device(void* dst, const void* src, size_t n, cudaStream_t s) {
 
 bool release_retired_plans();   // frees their memory; false: there was none
 
+}  // namespace
+
+namespace beor {
+cudaError_t device_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && release_retired_plans()) {
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+}  // namespace beor
+
+namespace {
+
 struct DevBuf {
   void* p = nullptr;
   size_t n = 0;
@@ -73,11 +88,7 @@ struct DevBuf {
   cudaError_t alloc(size_t bytes) {
     release();
     if (bytes == 0) return cudaSuccess;
-    cudaError_t e = cudaMalloc(&p, bytes);
-    if (e == cudaErrorMemoryAllocation && release_retired_plans()) {
-      cudaGetLastError();
-      e = cudaMalloc(&p, bytes);
-    }
+    const cudaError_t e = device_malloc(&p, bytes);
     if (e != cudaSuccess) {
       p = nullptr;
       return e;
@@ -650,18 +661,10 @@ void drop_plans_of(beor_ctx* c) {
 // Plans of a context whose data set is about to change: nothing may read their
 // results any more, but buffers and graph stay for the next call of the shape
 // (building them again took 4 of the 28 ms of a data set of 3280 modes with 16
-// points).  They hold a sixteenth of the device's memory at most; an allocation
-// that fails releases them.
+// points).  An allocation of the library that fails releases them; they hold a
+// sixteenth of the device's memory at most, and no more than is left for others.
 void retire_plans_of(beor_ctx* c) {
   std::lock_guard<std::recursive_mutex> lk(g_mu);
-  static const size_t limit = [] {
-    size_t avail = 0, total = 0;
-    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
-      cudaGetLastError();
-      total = 0;
-    }
-    return total / 16;
-  }();
   auto bytes = [](const Plan* p) {
     size_t n = 0;
     for (const DevBuf* b : {&p->d_prob, &p->d_sets, &p->ws, &p->dinv, &p->phi_inv, &p->vecs, &p->scal, &p->phis, &p->panel_sl,
@@ -669,9 +672,9 @@ void retire_plans_of(beor_ctx* c) {
       n += b->n;
     return n;
   };
-  size_t held = 0;
+  size_t held = 0, limit = 0;
   for (const Plan* p : g_plans)
-    if (p->retired) held += bytes(p);
+    if (p->retired && p->device == c->device) held += bytes(p);
   bool synced = false;
   std::vector<Plan*> keep;
   for (Plan* p : g_plans) {
@@ -682,6 +685,11 @@ void retire_plans_of(beor_ctx* c) {
     if (!synced) {   // no evaluation of the plan may still be running
       cudaDeviceSynchronize();
       synced = true;
+      size_t avail = 0, total = 0;
+      if (cudaMemGetInfo(&avail, &total) == cudaSuccess)
+        limit = std::min(total / 16, avail);
+      else
+        cudaGetLastError();
     }
     for (beor_ctx* o : p->ctxs)
       if (o->last_plan == p) o->last_plan = nullptr;

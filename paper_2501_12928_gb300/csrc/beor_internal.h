@@ -11,6 +11,11 @@
 
 namespace beor {
 
+// api.cu: cudaMalloc, for every allocation of the library.  Where the memory does
+// not suffice, the idle batches give theirs back first.
+cudaError_t device_malloc(void** p, size_t bytes);
+template <typename T>
+cudaError_t device_malloc(T** p, size_t bytes) { return device_malloc(reinterpret_cast<void**>(p), bytes); }
 // precompute.cu
 cudaError_t split_double_float(const double2* M, int64_t n, float4* out, cudaStream_t s);
 // Full nt x nt tile square of the packed lower M (n x n, padding zero), each

@@ -477,9 +477,9 @@ cudaError_t herk_dense_tc(const double2* T, int64_t n_vis, int n, int64_t ld, co
   const int nkb_buf = (int)std::min<int64_t>(HK_KB_PASS, nkb_total);
   const size_t plane_bytes = (size_t)rows * BEOR_TB * nkb_buf * 2;
   void *planes = nullptr, *exps = nullptr, *ctr = nullptr;
-  cudaError_t e = cudaMalloc(&planes, plane_bytes * HK_NPLANE);
-  if (e == cudaSuccess) e = cudaMalloc(&exps, sizeof(int32_t) * (size_t)rows * nkb_buf);
-  if (e == cudaSuccess) e = cudaMalloc(&ctr, sizeof(int) * 2);   // tile counter, error word
+  cudaError_t e = device_malloc(&planes, plane_bytes * HK_NPLANE);
+  if (e == cudaSuccess) e = device_malloc(&exps, sizeof(int32_t) * (size_t)rows * nkb_buf);
+  if (e == cudaSuccess) e = device_malloc(&ctr, sizeof(int) * 2);   // tile counter, error word
   CUtensorMap ma, mb;
   if (e == cudaSuccess) e = hk_map(&ma, planes, rows, nkb_buf, HK_M, 1);
   if (e == cudaSuccess) e = hk_map(&mb, planes, rows, nkb_buf, HK_N, 2);

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "../../include/beor.h"
+#include "beor_internal.h"
 
 namespace {
 
@@ -178,11 +179,11 @@ extern "C" int beor_set_instrument_desc(beor_ctx* ctx, const beor_instrument_des
   DevArr dcells, dBF, duv, dfreq, dA;
   cudaError_t e;
   const size_t nbf = (size_t)npx * npx * ncells;
-  if ((e = cudaMalloc(&dcells.p, sizeof(int) * cells.size())) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc(&dBF.p, sizeof(double2) * nbf)) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc(&duv.p, sizeof(double) * uv.size())) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc(&dfreq.p, sizeof(double) * nf)) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc(&dA.p, sizeof(double2) * (size_t)nf * ntb * ncells)) != cudaSuccess) return fail(e);
+  if ((e = beor::device_malloc(&dcells.p, sizeof(int) * cells.size())) != cudaSuccess) return fail(e);
+  if ((e = beor::device_malloc(&dBF.p, sizeof(double2) * nbf)) != cudaSuccess) return fail(e);
+  if ((e = beor::device_malloc(&duv.p, sizeof(double) * uv.size())) != cudaSuccess) return fail(e);
+  if ((e = beor::device_malloc(&dfreq.p, sizeof(double) * nf)) != cudaSuccess) return fail(e);
+  if ((e = beor::device_malloc(&dA.p, sizeof(double2) * (size_t)nf * ntb * ncells)) != cudaSuccess) return fail(e);
   if ((e = cudaMemcpy(dcells.p, cells.data(), sizeof(int) * cells.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(duv.p, uv.data(), sizeof(double) * uv.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(dfreq.p, freqs.data(), sizeof(double) * nf, cudaMemcpyHostToDevice)) != cudaSuccess)

@@ -728,9 +728,9 @@ cudaError_t mixed_maps_create(const BatchView& v, MixedMaps** out) {
       }
       m->h_total[kind][k] = pk[v.P];
     }
-  e = cudaMalloc(&m->d_prefix, sizeof(int64_t) * pre.size());
+  e = device_malloc(&m->d_prefix, sizeof(int64_t) * pre.size());
   if (e == cudaSuccess) e = cudaMemcpy(m->d_prefix, pre.data(), sizeof(int64_t) * pre.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d_counter, sizeof(int) * KIND_COUNT * (size_t)v.max_nt);
+  if (e == cudaSuccess) e = device_malloc(&m->d_counter, sizeof(int) * KIND_COUNT * (size_t)v.max_nt);
   if (e != cudaSuccess) {
     mixed_maps_destroy(m);
     return e;

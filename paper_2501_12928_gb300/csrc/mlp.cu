@@ -29,7 +29,7 @@
 #include <vector>
 
 #include "../../include/beor.h"
-#include "per_device.h"
+#include "beor_internal.h"
 
 namespace {
 
@@ -497,7 +497,7 @@ struct beor_mlp {
 namespace {
 
 cudaError_t dalloc(beor_mlp* m, void** p, size_t bytes) {
-  cudaError_t e = cudaMalloc(p, bytes);
+  cudaError_t e = beor::device_malloc(p, bytes);
   if (e == cudaSuccess) {
     m->owned.push_back(*p);
     cudaMemset(*p, 0, bytes);

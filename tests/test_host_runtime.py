@@ -139,3 +139,59 @@ def test_likelihoods_on_two_devices(fake, first, precision):
             lk.lnl(phi, stream=STREAM)
         lk.posterior_mean(np.zeros(3), stream=STREAM)
         assert _kernels(fake, device)
+
+
+def _idle_batch(lib):
+    """A context with new data and the idle batch of an earlier evaluation; its bytes."""
+    lk, p = _like(lib)
+    before = lib.fake_used(0)
+    lk.lnl(np.zeros((8, 3)), stream=STREAM)
+    batch = lib.fake_used(0) - before
+    lk.set_data(p["d"], p["noise_var"])
+    return lk, p, batch
+
+
+def _set_instrument(lk, p):
+    geometry = dict(nu=7, nf=12, nf_grid=0, n_pix=64, n_k=3, f0_hz=1.5e8, df_hz=1e6, beam_fwhm_rad=0.2, latitude_rad=-0.5,
+                    lssm_prior_var=2.0, bl_enu_m=np.random.default_rng(0).uniform(-30, 30, (200, 3)),
+                    hour_angle_rad=np.linspace(-0.1, 0.1, 4))
+    beor.Likelihood("fp64").set_instrument_desc(geometry)
+
+
+@pytest.mark.parametrize("call", [
+    lambda lk, p: lk.precompute(STREAM),                       # digit planes of the dense precompute
+    lambda lk, p: beor.Emulator(9, 256, 8),
+    _set_instrument,
+    lambda lk, p: beor.Likelihood("mixed").set_T(np.ones((1000, 300)), np.zeros(300, np.int32), 1, 2.0)])
+def test_allocations_get_the_idle_batches_memory(fake, call):
+    """On a full device, whatever the library allocates."""
+    lk, p, batch = _idle_batch(fake)
+    used = fake.fake_used(0)
+    fake.fake_set_total(0, used + (1 << 20))
+    call(lk, p)
+    assert fake.fake_used(0) < used + (1 << 20) and batch > 4 << 20
+
+
+def test_idle_batches_leave_memory_to_others(fake):
+    """They are kept on a device with room, and not beyond a sixteenth of it or
+    beyond what is free beside them."""
+    lk, p, batch = _idle_batch(fake)
+
+    def kept(free, total=None):
+        lk.precompute(STREAM)
+        lk.lnl(np.zeros((8, 3)), stream=STREAM)
+        used = fake.fake_used(0)
+        ballast = Array(fake, 0, total - free - used) if total else None
+        fake.fake_set_total(0, total or used + free)
+        before = fake.fake_used(0)
+        lk.set_data(p["d"], p["noise_var"])
+        idle = before - fake.fake_used(0) < batch // 2
+        fake.fake_set_total(0, 1 << 38)
+        if ballast:
+            fake.cudaFree(ctypes.c_void_p(ballast.address))
+        return idle
+
+    assert kept(20 * batch)
+    assert not kept(4 * batch)                       # more than a sixteenth
+    assert kept(2 * batch, total=64 * batch)
+    assert not kept(batch // 2, total=64 * batch)    # more than what is free
