@@ -974,6 +974,10 @@ static int lnl_multi_impl(beor_ctx* const* ctxs, int nsets, const double* const*
     if (ctxs[s]->device != ctxs[0]->device || ctxs[s]->precision != ctxs[0]->precision) return BEOR_EINVAL;
     if (B[s] <= 0 || B[s] > 4096 || !phi[s]) return BEOR_EINVAL;
   }
+  // validate phi values (finite) on the host when possible, before anything changes
+  for (int s = 0; s < nsets; ++s)
+    for (size_t i = 0, cnt = is_device_ptr(phi[s]) ? 0 : (size_t)B[s] * ctxs[s]->n_k; i < cnt; ++i)
+      if (!std::isfinite(phi[s][i])) return BEOR_EINVAL;
   beor_ctx* c0 = ctxs[0];
   cudaSetDevice(c0->device);
   cudaStream_t st = (cudaStream_t)stream;
@@ -986,10 +990,7 @@ static int lnl_multi_impl(beor_ctx* const* ctxs, int nsets, const double* const*
     g_plans.push_back(pl);
   }
   const bool first_use = !pl->exec || pl->retired;
-  if (pl->retired) {
-    CKC(c0, refresh_sets(*pl));
-    pl->retired = false;
-  }
+  if (pl->retired) CKC(c0, refresh_sets(*pl));
   size_t on_host = 0, phi_end = 0;   // sets, values
   for (int s = 0; s < nsets; ++s) {
     const size_t off = (size_t)pl->phi_off[s], cnt = (size_t)B[s] * ctxs[s]->n_k;
@@ -998,9 +999,6 @@ static int lnl_multi_impl(beor_ctx* const* ctxs, int nsets, const double* const*
       CKC(c0, cudaMemcpyAsync(pl->phis.as<double>() + off, phi[s], sizeof(double) * cnt, cudaMemcpyDeviceToDevice, st));
       continue;
     }
-    // validate phi values (finite) on the host when possible
-    for (size_t i = 0; i < cnt; ++i)
-      if (!std::isfinite(phi[s][i])) return BEOR_EINVAL;
     std::memcpy(pl->h_phi.as<double>() + off, phi[s], sizeof(double) * cnt);
     ++on_host;
   }
@@ -1045,6 +1043,7 @@ static int lnl_multi_impl(beor_ctx* const* ctxs, int nsets, const double* const*
     CKC(c0, cudaGraphLaunch(pl->exec, st));
     CKC(c0, cudaEventRecord(pl->ev1, st));
   }
+  pl->retired = false;
   auto lnl_at = [&](int s) { return lnl_out ? lnl_out[s] : nullptr; };
   auto status_at = [&](int s) { return status_out ? status_out[s] : nullptr; };
   for (int s = 0; s < nsets; ++s) {   // results to device memory

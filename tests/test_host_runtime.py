@@ -14,6 +14,7 @@ import pytest
 from paper_2501_12928_gb300 import _build, beor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
+HEADER = os.path.join(os.path.dirname(HERE), "include", "beor.h")
 STREAM = 0x1000   # any stream but the null one
 
 
@@ -22,7 +23,7 @@ def fake_library(tmp_path_factory):
     if shutil.which("g++") is None or (shutil.which("nvcc") is None and not os.path.exists(_build._nvcc())):
         pytest.skip("no compiler")
     objs = [os.path.join(_build.OUT_DIR, s.replace(".cu", ".o")) for s in _build.SOURCES]
-    newest = max(map(os.path.getmtime, glob.glob(os.path.join(_build.CSRC, "*")) + [_build.__file__]))
+    newest = max(map(os.path.getmtime, glob.glob(os.path.join(_build.CSRC, "*")) + [_build.__file__, HEADER]))
     if not all(os.path.exists(o) and os.path.getmtime(o) > newest for o in objs):
         _build.build()
     lib = str(tmp_path_factory.mktemp("fake") / "libbeor_fake.so")
@@ -195,3 +196,24 @@ def test_idle_batches_leave_memory_to_others(fake):
     assert not kept(4 * batch)                       # more than a sixteenth
     assert kept(2 * batch, total=64 * batch)
     assert not kept(batch // 2, total=64 * batch)    # more than what is free
+
+
+def test_rejected_points_leave_an_idle_batch_idle(fake):
+    """Points that are refused are no evaluation of the new data: the wait for one
+    still reports that there is none, and the batch's memory is still given back."""
+    lk, p, batch = _idle_batch(fake)
+    lk.precompute(STREAM)
+    for B in (8, 5):   # an idle batch, and a shape that has none
+        phi = np.zeros((B, 3))
+        phi[-1, 1] = np.nan
+        with pytest.raises(beor.BeorError, match="invalid argument"):
+            lk.lnl(phi, stream=STREAM)
+        with pytest.raises(beor.BeorError, match="out of order"):
+            beor.lnl_multi_wait([lk], [B], 0, STREAM)
+    used = fake.fake_used(0)
+    fake.fake_set_total(0, used)
+    beor.Emulator(9, 256, 8)
+    assert fake.fake_used(0) < used
+    fake.fake_set_total(0, 1 << 38)
+    lk.lnl(np.zeros((8, 3)), stream=STREAM)
+    beor.lnl_multi_wait([lk], [8], 0, STREAM)
