@@ -43,8 +43,7 @@ struct BatchView {
   int max_nt;
   // workspaces
   void* ws;                  // packed tiles of every problem (double2 or float4)
-  double2* dinv;             // inverse diagonal blocks, packed lower 128x128 per block (lnL on the mixed
-                             // path: float4 double-float elements in the same place)
+  double2* dinv;             // inverse diagonal blocks, packed lower 128x128 per block
   double* phi_inv;           // [rows] prior inverse per problem row (padded rows = 1)
   double2* vec_b;            // [rows] right-hand side / residual
   double2* vec_y;            // [rows] forward-solve result

@@ -645,9 +645,9 @@ __global__ void __launch_bounds__(DT_THREADS, 1) diag_tc_kernel(BatchView v, int
     for (int o = 16; o > 0; o >>= 1) ld += __shfl_xor_sync(0xffffffffu, ld, o);
     if (lane == 0) sm.red[warp] = ld;
   }
-  // Linv = Linv~ diag(2^-e_j) (double-float) for the solves, and its rows'
+  // Linv = Linv~ diag(2^-e_j) (float64) for the solves, and its rows'
   // exponents for the slices
-  float4* dinv = reinterpret_cast<float4*>(v.dinv) + pr.dinv_off + (int64_t)k * DG_PACK;
+  double2* dinv = v.dinv + pr.dinv_off + (int64_t)k * DG_PACK;
   float4* Af = reinterpret_cast<float4*>(sm.s);
   for (int w = warp; w < BEOR_TB / C; w += DT_WARPS) {
     const int r = ((w >> 4) * C + rank) * 16 + (w & 15);
@@ -658,7 +658,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) diag_tc_kernel(BatchView v, int
       const pow2 ps = make_pow2(-sm.es[c]);
       const float4 g = make_float4(scale2f(f.x, ps), scale2f(f.y, ps), scale2f(f.z, ps), scale2f(f.w, ps));
       Af[e] = g;
-      dinv[e] = g;
+      dinv[e] = make_double2((double)g.x + (double)g.y, (double)g.z + (double)g.w);
       mx = fmaxf(mx, fmaxf(fabsf(g.x), fabsf(g.z)));
     }
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));

@@ -1,4 +1,6 @@
 // Triangular solves with the factor (both precisions).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -8,26 +10,34 @@
 
 namespace beor {
 
+namespace cg = cooperative_groups;
+
 // --------------------------------------------------------------------------
 // Triangular solves with the factor: out = L^-H L^-1 rhs, blocked by 128.  Step k
 // has two parts: its block of the solution, y_k = Linv_k r_k, and the update of
 // the other blocks, r_i -= L_ik y_k (backward: with L_ki^H).
-//   - Large batches launch one after the other: a CTA per problem, then a CTA per
-//     tile.  Small ones do both in one launch, a CTA per quarter tile, every one
-//     forming y_k for itself (33,000 products, cheaper than a launch that waits
-//     for one CTA).
+//   - Large batches launch one after the other: the block, then the update with a CTA
+//     per tile. Small ones do both in one launch, a CTA per quarter tile, every four
+//     forming y_k for themselves (cheaper than a launch that waits for one CTA).
+//   - lnL: four CTAs of a cluster form y_k together, eight lanes per row, and exchange
+//     it through distributed shared memory.  Its 33,000 float64 products take 8 us on
+//     one SM (and 9 as chains of 128 pairs): with all of it in every CTA one point of
+//     3280 modes took 7.57 ms and 64 points 46.1, now 6.63 and 45.7.  (In double-float,
+//     which loses the last bits of r_k, 6.68 and 45.2.)  The float64 path and the
+//     posterior mean keep one chain per sum: any other order moves the mean's
+//     amplitudes by as much as the rounding of its factor does.
 //   - Inverse block and quarter tile are copied to shared memory by cp.async, all
 //     in flight at once, before the step waits for the one before (programmatic
 //     dependent launch): the factor is final by then.
-//   - Real and imaginary part of a sum go to two threads.
+//   - Real and imaginary part of an update's sum go to two threads.
 // Off-diagonal products: float64 for the float64 path, double-float (fp32 pairs,
-// error-free sums) for the mixed path's double-float factor; the inverse blocks
-// are float64 for the float64 path and the posterior mean.  The order of each sum
-// is fixed, so the results do not depend on the batch.
+// error-free sums) for the mixed path's double-float factor; the inverse blocks are
+// applied in float64.  The order of each sum is fixed, so the results do not depend
+// on the batch.
 // Bound by memory in large batches, by the launch and by the chains of dependent
 // products in small ones.  A step with one CTA per tile and 16 rounds of loads,
 // the inverse block in one CTA at its end, took 35 us with one point of 3280
-// modes and 71 with 64; now 5 and 60.  Float64, one point of 2000 modes: 38
+// modes and 71 with 64; now 7 and 70.  Float64, one point of 2000 modes: 38
 // -> 30 us, whose chains of 128 dependent pairs of products alone are 9 us.
 // --------------------------------------------------------------------------
 constexpr int SOLVE_SPLIT = 4;                       // CTAs per tile
@@ -37,15 +47,25 @@ template <typename V>   // V: the factor's real type, double or dfl
 struct SolveVecs {
   double2 yk[BEOR_TB];
   double rd[2][BEOR_TB];               // r_k by component
-  dfl rf[2][BEOR_TB];
   V yv[2][BEOR_TB];                    // y_k by component
   V part[2][SOLVE_ROWS];
 };
-// shared memory: Linv_k, packed (double2 or float4 elements); the quarter tile,
+// Who forms y_k = Linv_k r_k: a CTA alone, one chain per sum (the order of the
+// float64 path and of the posterior mean), or SHARE CTAs, a quarter of the rows or
+// all of them each, eight chains per sum (lnL).
+constexpr int SOLVE_CHAIN = 0;
+// A quarter's rows: four rows in turn give one to each quarter.  Row s of quarter c
+// (backward: column, counted from the last); it has solve_row + 1 terms, stored from
+// solve_row_off on.
+constexpr int SOLVE_QUARTER = 2 * SOLVE_ROWS * (SOLVE_ROWS + 1);   // elements
+__device__ __forceinline__ int solve_row(int c, int s) { return 4 * s + (s & 1 ? 3 - c : c); }
+__device__ __forceinline__ int solve_row_off(int s) { return 2 * s * (s + 1); }
+// shared memory: Linv_k, packed or by quarters; the quarter tile,
 // forward [column][own row], backward [own column][row]; the vectors
+constexpr size_t solve_li(int share) { return share == SOLVE_CHAIN ? DG_PACK : SOLVE_SPLIT / share * SOLVE_QUARTER; }
 template <typename V>
-constexpr size_t solve_smem(bool both) {
-  return sizeof(double2) * (size_t)(DG_PACK + (both ? BEOR_TB * SOLVE_ROWS : 0)) + sizeof(SolveVecs<V>);
+constexpr size_t solve_smem(int share, bool both) {
+  return sizeof(double2) * (solve_li(share) + (both ? BEOR_TB * SOLVE_ROWS : 0)) + sizeof(SolveVecs<V>);
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -78,11 +98,10 @@ __device__ __forceinline__ dfl shfl_part(dfl a, int o) {
 __device__ __forceinline__ double get_part(double a) { return a; }
 __device__ __forceinline__ double get_part(dfl a) { return (double)a.hi + (double)a.lo; }
 
-// yk = Linv rk or (HERM) Linv^H rk.  Float64: 256 threads, one per row and
-// component; the two warps of an SM quarter get rows of 160 terms together.
+// yk = Linv rk or (HERM) Linv^H rk, by 256 threads, one per row and component; the
+// two warps of an SM quarter get rows of 160 terms together.
 template <bool HERM>
-__device__ __forceinline__ void solve_diag(const double2* li, const double (*rd)[BEOR_TB], const dfl (*)[BEOR_TB], dfl*,
-                                           double2* yk) {
+__device__ __forceinline__ void solve_diag(const double2* li, const double (*rd)[BEOR_TB], double2* yk) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp >= 8) return;
   const int comp = warp & 1, gl = warp < 4 ? 3 - (warp >> 1) : (warp - 4) >> 1;   // group by length, 3 the longest
@@ -93,38 +112,31 @@ __device__ __forceinline__ void solve_diag(const double2* li, const double (*rd)
     mac_part(acc, li + (HERM ? pk(m, t) : pk(t, m)), HERM, comp, rd[comp][m], rd[1 - comp][m]);
   (comp ? yk[t].y : yk[t].x) = acc;
 }
-// Double-float: forward eight lanes per row, backward two threads per column
-// and component; warps of an SM quarter get columns of all lengths.
-template <bool HERM>
-__device__ __forceinline__ void solve_diag(const float4* li, const double (*)[BEOR_TB], const dfl (*rf)[BEOR_TB], dfl* part,
-                                           double2* yk) {
-  const int tid = threadIdx.x;
-  if (!HERM) {
-    const int lane8 = tid & 7;
-    for (int t = tid >> 3; t < BEOR_TB; t += SOLVE_THREADS / 8) {
-      dfl a[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
+
+// The same by SHARE CTAs, eight lanes per row, both components.  The warps of an SM
+// quarter get rows of about the same number of terms together.  Row results go to
+// every CTA of the cluster (SHARE 1: no cluster).
+template <bool HERM, int SHARE>
+__device__ __forceinline__ void solve_diag_shared(const double2* s_li, int rank, const double (*rd)[BEOR_TB], double2* yk) {
+  constexpr int NQ = SOLVE_SPLIT / SHARE, NG = 8 * NQ;   // quarters of this CTA, groups of four rows by length
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lane8 = lane & 7;
+  for (int w = warp; w < NG; w += SOLVE_THREADS / 32) {
+    const int gl = w < NG / 2 ? NG - 1 - w : w - NG / 2, q = gl % NQ, c = SHARE == 1 ? q : rank;
+    const int s = 4 * (gl / NQ) + (lane >> 3), n = solve_row(c, s), t = HERM ? BEOR_TB - 1 - n : n;
+    const double2* li = s_li + q * SOLVE_QUARTER + solve_row_off(s);
+    double a[2] = {0.0, 0.0};
 #pragma unroll 2
-      for (int m = lane8; m <= t; m += 8)
+    for (int m = lane8; m <= n; m += 8) {
+      const int u = HERM ? t + m : m;
 #pragma unroll
-        for (int comp = 0; comp < 2; ++comp) mac_part(a[comp], li + pk(t, m), false, comp, rf[comp][m], rf[1 - comp][m]);
-#pragma unroll
-      for (int comp = 0; comp < 2; ++comp)
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) add_part(a[comp], shfl_part(a[comp], o));
-      if (lane8 == 0) yk[t] = make_double2(get_part(a[0]), get_part(a[1]));
+      for (int comp = 0; comp < 2; ++comp) mac_part(a[comp], li + m, HERM, comp, rd[comp][u], rd[1 - comp][u]);
     }
-  } else {
-    const int warp = tid >> 5, comp = warp >> 3, half = (warp >> 2) & 1;
-    const int t = 32 * ((warp + (warp >> 2)) & 3) + (tid & 31);
-    dfl a{0.0f, 0.0f};
-#pragma unroll 2
-    for (int m = t + half; m < BEOR_TB; m += 2) mac_part(a, li + pk(m, t), true, comp, rf[comp][m], rf[1 - comp][m]);
-    if (half) part[comp * BEOR_TB + t] = a;
-    __syncthreads();
-    if (!half) {
-      add_part(a, part[comp * BEOR_TB + t]);
-      (comp ? yk[t].y : yk[t].x) = get_part(a);
-    }
+    __syncwarp();
+#pragma unroll
+    for (int comp = 0; comp < 2; ++comp)
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) add_part(a[comp], shfl_part(a[comp], o));   // the same bits in every lane
+    if (lane8 < SHARE) (SHARE == 1 ? yk : cg::this_cluster().map_shared_rank(yk, lane8))[t] = make_double2(a[0], a[1]);
   }
 }
 
@@ -132,28 +144,38 @@ __device__ __forceinline__ void solve_diag(const float4* li, const double (*)[BE
 // by CTA (SOLVE_SPLIT (i - k - 1) + quarter, p) or, HERM, (SOLVE_SPLIT i + quarter,
 // p), where problems join when k < their nt.  src: the right-hand side; the running
 // one is vec_t.
-template <typename WS, typename DV, bool HERM, bool BOTH>
+template <typename WS, bool HERM, bool BOTH, int SHARE>
 __global__ void __launch_bounds__(SOLVE_THREADS, 1)
     solve_step_kernel(BatchView v, int kg, const double2* src, double2* out) {
   using V = typename std::conditional<std::is_same<WS, float4>::value, dfl, double>::type;
   extern __shared__ __align__(16) unsigned char ss_raw[];
   double2* const s_li = reinterpret_cast<double2*>(ss_raw);
-  double2* const s_tile = s_li + DG_PACK;
+  double2* const s_tile = s_li + solve_li(SHARE);
   SolveVecs<V>& sm = *reinterpret_cast<SolveVecs<V>*>(s_tile + (BOTH ? BEOR_TB * SOLVE_ROWS : 0));
-  dfl* const dpart = reinterpret_cast<dfl*>(sm.yv);   // HERM, DV float4: halves of yk (yv is filled after)
   const int tid = threadIdx.x, p = blockIdx.y;
   const Prob pr = v.prob[p];
   const int k = HERM ? kg : kg - pr.k_off;   // this problem's step
   const int i = (HERM ? 0 : k + 1) + blockIdx.x / SOLVE_SPLIT, c0 = blockIdx.x % SOLVE_SPLIT * SOLVE_ROWS;
   const bool upd = BOTH && (HERM ? i < k : i < pr.nt);   // has a block to update
   const int ti = HERM ? k : i, tj = HERM ? i : k;
-  bool on = k >= 0 && k < pr.nt && (upd || blockIdx.x == 0) && !prob_skipped(v.status[p]);
+  // CTAs that share are on together, whatever becomes of the status meanwhile
+  const bool skipped = prob_skipped(v.status[p]);
+  bool on = k >= 0 && k < pr.nt && (upd || blockIdx.x < (SHARE > 1 ? SHARE : 1)) && (SHARE > 1 || !skipped);
   on = on && BEOR_INBOUNDS(v.flags, pr.row_off + (int64_t)pr.nt * BEOR_TB <= v.rows, BC_SOLVE_VEC) &&
        BEOR_INBOUNDS(v.flags, !upd || pr.ws_off + (tri_index(ti, tj) + 1) * BEOR_TILE_ELEMS <= v.ws_elems, BC_SOLVE_VEC) &&
        BEOR_INBOUNDS(v.flags, pr.dinv_off + (int64_t)(k + 1) * DG_PACK <= v.dinv_elems, BC_DIAG_DINV);
   if (on) {
-    const double2* li = reinterpret_cast<const double2*>(v.dinv) + pr.dinv_off + (int64_t)k * DG_PACK;
-    for (int e = tid; e < DG_PACK; e += SOLVE_THREADS) cp_async16(&s_li[e], li + e);
+    const double2* li = v.dinv + pr.dinv_off + (int64_t)k * DG_PACK;
+    if constexpr (SHARE == SOLVE_CHAIN) {
+      for (int e = tid; e < DG_PACK; e += SOLVE_THREADS) cp_async16(&s_li[e], li + e);
+    } else {
+      for (int w = tid >> 5; w < SOLVE_ROWS * SOLVE_SPLIT / SHARE; w += SOLVE_THREADS / 32) {
+        const int s = w % SOLVE_ROWS, q = w / SOLVE_ROWS, n = solve_row(SHARE == 1 ? q : blockIdx.x % SHARE, s);
+        for (int m = tid & 31; m <= n; m += 32)
+          cp_async16(&s_li[q * SOLVE_QUARTER + solve_row_off(s) + m],
+                     li + (HERM ? pk(BEOR_TB - 1 - n + m, BEOR_TB - 1 - n) : pk(n, m)));
+      }
+    }
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (upd) {
       const double2* t = reinterpret_cast<const double2*>(v.ws) + pr.ws_off + tri_index(ti, tj) * BEOR_TILE_ELEMS;
@@ -164,6 +186,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1)
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+    if (SHARE > 1) cg::cluster_group::barrier_arrive();
   }
   // every CTA waits, those without work too: the grid after this one must not
   // run past the one before
@@ -180,18 +203,22 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1)
   if (last) cur = reinterpret_cast<const double*>(r + i * BEOR_TB + c0 + own)[comp];
   if (tid < BEOR_TB) {
     const double2 q = r[k * BEOR_TB + tid];
-    if constexpr (std::is_same<DV, double2>::value) {
-      sm.rd[0][tid] = q.x;
-      sm.rd[1][tid] = q.y;
-    } else {
-      sm.rf[0][tid] = df_from_double(q.x);
-      sm.rf[1][tid] = df_from_double(q.y);
-    }
+    sm.rd[0][tid] = q.x;
+    sm.rd[1][tid] = q.y;
   }
   asm volatile("cp.async.wait_group 1;" ::: "memory");
   __syncthreads();
-  solve_diag<HERM>(reinterpret_cast<const DV*>(s_li), sm.rd, sm.rf, dpart, sm.yk);
-  __syncthreads();
+  if constexpr (SHARE == SOLVE_CHAIN) {
+    solve_diag<HERM>(s_li, sm.rd, sm.yk);
+  } else {
+    if (SHARE > 1) cg::cluster_group::barrier_wait();   // every CTA of the cluster has started
+    solve_diag_shared<HERM, SHARE>(s_li, blockIdx.x % SHARE, sm.rd, sm.yk);
+  }
+  if (SHARE > 1)
+    cg::this_cluster().sync();   // the last access to another CTA's memory is behind
+  else
+    __syncthreads();
+  if (SHARE > 1 && skipped) return;
   if (tid < BEOR_TB) {
     const double2 q = sm.yk[tid];
     if (blockIdx.x == 0) out[pr.row_off + k * BEOR_TB + tid] = q;
@@ -311,54 +338,68 @@ __global__ void __launch_bounds__(256, 2)
 // factor, are what is waited for)
 template <typename... Exp, typename... Act>
 static cudaError_t launch_after(void (*kern)(Exp...), dim3 grid, int threads, size_t smem, cudaStream_t s, bool after,
-                                Act&&... args) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
+                                int cluster, Act&&... args) {
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (after) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = cluster;
+    at[n].val.clusterDim.y = 1;
+    at[n++].val.clusterDim.z = 1;
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cfg.attrs = &at;
-  cfg.numAttrs = after ? 1 : 0;
+  cfg.attrs = at;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Act>(args)...);
 }
-template <typename WS, typename DV, bool HERM, bool BOTH>
+template <typename WS, bool HERM, bool BOTH, int SHARE>
 static cudaError_t launch_block(const BatchView& v, int k, int blocks, const double2* src, double2* out, cudaStream_t s,
                                 bool after) {
   using V = typename std::conditional<std::is_same<WS, float4>::value, dfl, double>::type;
-  const cudaError_t attr = allow_smem<solve_step_kernel<WS, DV, HERM, BOTH>>((int)solve_smem<V>(BOTH));
+  static_assert(SHARE <= 1 || SHARE == SOLVE_SPLIT, "a cluster is the CTAs of one tile");
+  constexpr int ctas = SHARE > 1 ? SHARE : 1;
+  constexpr size_t smem = solve_smem<V>(SHARE, BOTH);
+  const cudaError_t attr = allow_smem<solve_step_kernel<WS, HERM, BOTH, SHARE>>((int)smem);
   if (attr != cudaSuccess) return attr;
-  return launch_after(solve_step_kernel<WS, DV, HERM, BOTH>, dim3(BOTH ? std::max(1, SOLVE_SPLIT * blocks) : 1, v.P), SOLVE_THREADS, solve_smem<V>(BOTH), s,
-                      after, v, k, src, out);
+  return launch_after(solve_step_kernel<WS, HERM, BOTH, SHARE>, dim3(BOTH ? std::max(ctas, SOLVE_SPLIT * blocks) : ctas, v.P),
+                      SOLVE_THREADS, smem, s, after, ctas, v, k, src, out);
 }
-// The products with the inverse block in every CTA pay while the first step's CTAs
-// fit the SMs once.  Solves of one evaluation in ms (one launch per step / two):
+// The products with the inverse block beside every tile pay while the first step's
+// CTAs fit the SMs once.  Solves of one evaluation in ms (one launch per step / two):
 // mixed, 3280 modes (26 blocks) one point 0.89 / 0.96, two 1.06 / 1.02; 1000 modes
 // (8 blocks) four points 0.28 / 0.30, eight 0.35 / 0.32.  Float64, 2000 modes (16
 // blocks) two points 0.95 / 0.96, four 1.33 / 1.04.
 static bool solve_is_small(const BatchView& v) { return (int64_t)SOLVE_SPLIT * v.P * v.max_nt <= device_sms(); }
 // Step k of one pass.
-template <bool HERM, typename WS, typename DV>
+template <bool HERM, typename WS, int SHARE>
 static cudaError_t step_as(const BatchView& v, bool both, int k, const double2* src, double2* out, cudaStream_t s, bool after) {
   const int blocks = HERM ? k : v.max_nt - 1 - k;   // to update
-  if (both) return launch_block<WS, DV, HERM, true>(v, k, blocks, src, out, s, after);
-  const cudaError_t e = launch_block<WS, DV, HERM, false>(v, k, blocks, src, out, s, after);
+  if (both) return launch_block<WS, HERM, true, SHARE>(v, k, blocks, src, out, s, after);
+  const cudaError_t e = launch_block<WS, HERM, false, SHARE>(v, k, blocks, src, out, s, after);
   if (e != cudaSuccess || blocks == 0) return e;
-  return launch_after(solve_update_kernel<WS, HERM>, dim3(blocks, v.P), 256, 0, s, true, v, k, src, (const double2*)out);
+  return launch_after(solve_update_kernel<WS, HERM>, dim3(blocks, v.P), 256, 0, s, true, 1, v, k, src, (const double2*)out);
 }
 template <bool HERM>
 static cudaError_t solve_step(const BatchView& v, bool mixed, bool both, int k, const double2* src, double2* out,
                               cudaStream_t s, bool after) {
-  return !mixed   ? step_as<HERM, double2, double2>(v, both, k, src, out, s, after)
-         : v.mean ? step_as<HERM, float4, double2>(v, both, k, src, out, s, after)
-                  : step_as<HERM, float4, float4>(v, both, k, src, out, s, after);
+  return !mixed   ? step_as<HERM, double2, SOLVE_CHAIN>(v, both, k, src, out, s, after)
+         : v.mean ? step_as<HERM, float4, SOLVE_CHAIN>(v, both, k, src, out, s, after)
+                  : step_as<HERM, float4, SOLVE_SPLIT>(v, both, k, src, out, s, after);
 }
 
 // Step k (0 .. max_nt - 1) of vec_y = L^-1 rhs, beside other work: the parts one
-// after the other, which take less of an SM than both in one.
+// after the other, which take less of an SM than both in one, and no clusters but in
+// the last two steps, which nothing else runs beside (16 -> 9 us each).
 cudaError_t launch_fwd_step(const BatchView& v, bool mixed, const double2* rhs, int k, cudaStream_t s) {
+  if (mixed && !v.mean && k + 2 < v.max_nt) return step_as<false, float4, 1>(v, false, k, rhs, v.vec_y, s, false);
   return solve_step<false>(v, mixed, false, k, rhs, v.vec_y, s, false);
 }
 int fwd_step_launches(const BatchView& v, int k) { return k + 1 < v.max_nt ? 2 : 1; }
