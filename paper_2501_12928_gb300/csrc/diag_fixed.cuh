@@ -60,6 +60,21 @@ __host__ __device__ __forceinline__ long long fx_mulhi(long long a, long long b)
   return (long long)(((__int128)a * b) >> 64);
 #endif
 }
+// v 2^-61 as three floats, |v| <= 2^61: exact, and each at most half an ulp of the
+// one before.
+__host__ __device__ __forceinline__ void fx_split3(long long v, float& hi, float& lo, float& t) {
+  const float a = (float)(int)(v >> 38) * 0x1p-23f, b = (float)(int)((v >> 14) & 0xffffff) * 0x1p-47f;
+  const float c = (float)(int)(v & 0x3fff) * 0x1p-61f;
+  const float h = a + b;                     // a = 0 or |a| > |b|
+  const float r = b - (h - a);
+  const float l = r + c;
+  const float rr = l - r;
+  const float e = (r - (l - rr)) + (c - rr);
+  hi = h + l;
+  const float m = l - (hi - h);              // may have lost a binade against e
+  lo = m + e;
+  t = e - (lo - m);
+}
 // A positive number d <= 1 as D 2^(-2g), D in [1/4, 1) (g >= -1).
 __host__ __device__ __forceinline__ long long fx_normalise(long long d, int& g) {
   g = (fx_clz((unsigned long long)d) - 3) >> 1;

@@ -32,7 +32,10 @@
 //    pipe), the rows below take B -= L~ Y by the same products (digits of Y
 //    scaled per column, the 21 pairs s + t <= 5: 2^-51) into double-float
 //    elements; column j of Linv~ takes the storage that column j of the block
-//    no longer needs.
+//    no longer needs.  The three floats of an element of L are each at most half
+//    an ulp of the one before, since the products of the lower ones are rounded
+//    (cut at fixed bits instead, small elements brought errors of 2^-47 of the
+//    row's largest into the inverse).
 //  * Eight warps update and factor the next panel's diagonal while the others
 //    do the rest of the rank-16 update.  The panel loops are kept rolled: a
 //    warp alone runs straight-line code at the rate of instruction fetches
@@ -47,6 +50,12 @@
 // (clusters of two) and 0.295 ms with 100 (single CTAs).  Most of it is the
 // chain of 128 columns in the panel factors and, between them, the
 // substitutions; loading and output take 13 us.
+//
+// Accuracy against 113-bit arithmetic over 78 blocks (dense random ones of 5 to 128
+// rows, condition 7 to 200, and blocks of drift scans, up to 3e6), as a fraction of
+// the float64 factor's and its fp32 inverse's: largest backward error 0.13 to 0.21
+// (at most 3e-16 of sqrt(a_ii a_ll)), rms error of L 0.23 to 0.79, of the inverse
+// 0.12 to 0.63, of the log-determinant 0.09 to 0.79.
 //
 // tcgen05 is not used: its smallest tile (M = 64 or 128 of one CTA, operands
 // by descriptor, accumulators in tensor memory) does not fit a triangle of
@@ -348,11 +357,10 @@ __device__ __forceinline__ void dt_factor(DtSmem& sm, float4* __restrict__ ws, i
     const longlong2 l = make_longlong2(fx_mul<1>(x.x, y), fx_mul<1>(x.y, y));
     // L~ y, 60 fractional bits: the multipliers of the rows below
     const fxs re = fx_split(fx_mul<0>(l.x, y)), im = fx_split(fx_mul<0>(l.y, y));
-    // -L~ as three floats per component, exactly (24, 24 and 14 bits)
-    const long long a = -l.x, b = -l.y;
-    const float4 f = make_float4((float)(int)(a >> 38) * 0x1p-23f, (float)(int)((a >> 14) & 0xffffff) * 0x1p-47f,
-                                 (float)(int)(b >> 38) * 0x1p-23f, (float)(int)((b >> 14) & 0xffffff) * 0x1p-47f);
-    const float2 t = make_float2((float)(int)(a & 0x3fff) * 0x1p-61f, (float)(int)(b & 0x3fff) * 0x1p-61f);
+    float4 f;   // -L~
+    float2 t;
+    fx_split3(-l.x, f.x, f.y, t.x);
+    fx_split3(-l.y, f.z, f.w, t.y);
 #pragma unroll
     for (int q = 0; q < C; ++q) {
       DtSmem* o = dt_peer<C>(sm, q);
