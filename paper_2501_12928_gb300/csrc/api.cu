@@ -599,6 +599,8 @@ int build_plan(beor_ctx* const* ctxs, int nsets, const int* Bs, bool need_x, int
   }
   chk(cudaEventCreate(&pl->ev0));
   chk(cudaEventCreate(&pl->ev1));
+  // the copies and fills above are the null stream's, which the caller's need not wait for
+  chk(cudaStreamSynchronize(nullptr));
   if (e != cudaSuccess) {
     delete pl;
     return BEOR_ECUDA;
@@ -720,8 +722,8 @@ bool release_retired_plans() {
 }
 
 // The set descriptors follow the contexts' buffers when a retired plan is
-// taken up again (the graph reads them from device memory).
-cudaError_t refresh_sets(Plan& pl) {
+// taken up again (the graph, next on the stream, reads them from device memory).
+cudaError_t refresh_sets(Plan& pl, cudaStream_t s) {
   bool changed = false;
   for (size_t s = 0; s < pl.ctxs.size(); ++s) {
     const beor_ctx* c = pl.ctxs[s];
@@ -734,7 +736,7 @@ cudaError_t refresh_sets(Plan& pl) {
     changed = changed || std::memcmp(&sd, &pl.h_sets[s], sizeof(sd)) != 0;
     pl.h_sets[s] = sd;
   }
-  return changed ? cudaMemcpy(pl.d_sets.p, pl.h_sets.data(), sizeof(SetDesc) * pl.h_sets.size(), cudaMemcpyHostToDevice)
+  return changed ? cudaMemcpyAsync(pl.d_sets.p, pl.h_sets.data(), sizeof(SetDesc) * pl.h_sets.size(), cudaMemcpyHostToDevice, s)
                  : cudaSuccess;
 }
 
@@ -990,7 +992,7 @@ static int lnl_multi_impl(beor_ctx* const* ctxs, int nsets, const double* const*
     g_plans.push_back(pl);
   }
   const bool first_use = !pl->exec || pl->retired;
-  if (pl->retired) CKC(c0, refresh_sets(*pl));
+  if (pl->retired) CKC(c0, refresh_sets(*pl, st));
   size_t on_host = 0, phi_end = 0;   // sets, values
   for (int s = 0; s < nsets; ++s) {
     const size_t off = (size_t)pl->phi_off[s], cnt = (size_t)B[s] * ctxs[s]->n_k;

@@ -525,6 +525,7 @@ cudaError_t ensure_io(beor_mlp* m, int n) {
   cudaError_t e = dalloc(m, (void**)&m->xin, sizeof(float) * (size_t)cap * m->n_in);
   if (e == cudaSuccess) e = dalloc(m, (void**)&m->tin, sizeof(float) * (size_t)cap);
   if (e == cudaSuccess) e = dalloc(m, (void**)&m->yout, sizeof(float) * (size_t)cap);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);   // the fills, before another stream's work
   if (e == cudaSuccess) m->iocap = cap;
   return e;
 }
@@ -551,6 +552,7 @@ cudaError_t ensure_cap(beor_mlp* m, int n) {
     if (e == cudaSuccess) e = dalloc(m, (void**)&m->dZb[l], sizeof(__nv_bfloat16) * (size_t)cap * m->kout[l]);
   }
   if (e == cudaSuccess) e = dalloc(m, (void**)&m->loss_part, sizeof(float) * (size_t)(cap / 16));
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
   if (e == cudaSuccess) m->cap = cap;
   return e;
 }

@@ -217,3 +217,21 @@ def test_rejected_points_leave_an_idle_batch_idle(fake):
     fake.fake_set_total(0, 1 << 38)
     lk.lnl(np.zeros((8, 3)), stream=STREAM)
     beor.lnl_multi_wait([lk], [8], 0, STREAM)
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_work_waits_for_the_null_streams(fake, precision):
+    """Buffers that the library fills on the null stream are filled before it works
+    with them on the caller's, which need not wait for the null stream: first calls of
+    a shape, batches taken up again, growing emulator batches."""
+    lk, p = _like(fake, 140, 200, precision)
+    lk.lnl(np.zeros((8, 3)), stream=STREAM)
+    lk.posterior_mean(np.zeros(3), stream=STREAM)
+    lk.set_data(p["d"], p["noise_var"])
+    lk.precompute(STREAM)
+    lk.lnl(np.zeros((8, 3)), stream=STREAM)
+    em = beor.Emulator(N_IN, 32, 2)
+    for n in (100, 3000, 9000):
+        em.infer(np.zeros((n, N_IN), np.float32), stream=STREAM)
+        em.train_step(np.zeros((n, N_IN), np.float32), np.zeros(n, np.float32), 1e-3, stream=STREAM)
+    assert fake.fake_unordered() == 0
