@@ -928,6 +928,7 @@ int beor_precompute(beor_ctx* c, void* stream) {
   cudaSetDevice(c->device);
   cudaStream_t s = (cudaStream_t)stream;
   retire_plans_of(c);
+  c->have_pre = false;   // what follows overwrites the last one's matrices
   CKC(c, c->M.ensure(sizeof(double2) * (size_t)tri_count(c->nt) * BEOR_TILE_ELEMS));
   CKC(c, c->dbar.ensure(sizeof(double2) * (size_t)c->nt * BEOR_TB));
   if (c->model_kind == 1) {

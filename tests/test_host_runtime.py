@@ -235,3 +235,19 @@ def test_work_waits_for_the_null_streams(fake, precision):
         em.infer(np.zeros((n, N_IN), np.float32), stream=STREAM)
         em.train_step(np.zeros((n, N_IN), np.float32), np.zeros(n, np.float32), 1e-3, stream=STREAM)
     assert fake.fake_unordered() == 0
+
+
+def test_no_evaluation_after_a_failed_precompute(fake):
+    """A precompute that runs out of memory leaves matrices of which some are the new
+    data's: there is nothing to evaluate until one succeeds."""
+    lk, p = _like(fake)
+    fake.fake_set_total(0, fake.fake_used(0) + (1 << 20))
+    with pytest.raises(beor.BeorError, match="out of memory"):
+        lk.precompute(STREAM)
+    fake.fake_set_total(0, 1 << 38)
+    for call in (lambda: lk.lnl(np.zeros((1, 3)), stream=STREAM), lambda: lk.posterior_mean(np.zeros(3), stream=STREAM),
+                 lk.get_M, lk.get_dbar):
+        with pytest.raises(beor.BeorError, match="out of order"):
+            call()
+    lk.precompute(STREAM)
+    lk.lnl(np.zeros((1, 3)), stream=STREAM)
