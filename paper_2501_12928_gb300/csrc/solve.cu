@@ -22,10 +22,11 @@ namespace cg = cooperative_groups;
 //   - lnL: four CTAs of a cluster form y_k together, eight lanes per row, and exchange
 //     it through distributed shared memory.  Its 33,000 float64 products take 8 us on
 //     one SM (and 9 as chains of 128 pairs): with all of it in every CTA one point of
-//     3280 modes took 7.57 ms and 64 points 46.1, now 6.63 and 45.7.  (In double-float,
-//     which loses the last bits of r_k, 6.68 and 45.2.)  The float64 path and the
-//     posterior mean keep one chain per sum: any other order moves the mean's
-//     amplitudes by as much as the rounding of its factor does.
+//     3280 modes took 7.57 ms and 64 points 46.1, now 6.63 and 45.3.  (In double-float,
+//     which loses the last bits of r_k, 6.66 and 45.1.)  With more problems than SMs
+//     float64's pipe bounds the blocks: 200 points of 240 modes 1.80 ms (1.69 in
+//     double-float).  The float64 path and the posterior mean keep one chain per sum:
+//     any other order changes the bits of the mean's amplitudes.
 //   - Inverse block and quarter tile are copied to shared memory by cp.async, all
 //     in flight at once, before the step waits for the one before (programmatic
 //     dependent launch): the factor is final by then.
@@ -132,11 +133,16 @@ __device__ __forceinline__ void solve_diag_shared(const double2* s_li, int rank,
       for (int comp = 0; comp < 2; ++comp) mac_part(a[comp], li + m, HERM, comp, rd[comp][u], rd[1 - comp][u]);
     }
     __syncwarp();
-#pragma unroll
-    for (int comp = 0; comp < 2; ++comp)
-#pragma unroll
-      for (int o = 1; o < 8; o <<= 1) add_part(a[comp], shfl_part(a[comp], o));   // the same bits in every lane
-    if (lane8 < SHARE) (SHARE == 1 ? yk : cg::this_cluster().map_shared_rank(yk, lane8))[t] = make_double2(a[0], a[1]);
+    // the even lanes add up the real parts, the odd ones the imaginary
+    const int comp = lane8 & 1;
+    double sum = a[comp ? 1 : 0] + shfl_part(a[comp ? 0 : 1], 1);
+    sum += shfl_part(sum, 2);
+    sum += shfl_part(sum, 4);
+    const int peer = lane8 >> 1;
+    if (peer < SHARE) {
+      double2* o = SHARE == 1 ? yk : cg::this_cluster().map_shared_rank(yk, peer);
+      (comp ? o[t].y : o[t].x) = sum;
+    }
   }
 }
 
@@ -366,8 +372,14 @@ static cudaError_t launch_block(const BatchView& v, int k, int blocks, const dou
   using V = typename std::conditional<std::is_same<WS, float4>::value, dfl, double>::type;
   static_assert(SHARE <= 1 || SHARE == SOLVE_SPLIT, "a cluster is the CTAs of one tile");
   constexpr int ctas = SHARE > 1 ? SHARE : 1;
-  constexpr size_t smem = solve_smem<V>(SHARE, BOTH);
-  const cudaError_t attr = allow_smem<solve_step_kernel<WS, HERM, BOTH, SHARE>>((int)smem);
+  constexpr size_t need = solve_smem<V>(SHARE, BOTH), most = 120 * 1024;
+  // Float64's pipe bounds the block alone: its CTAs, which start beside the update
+  // before them, must not gather on the SMs that are free first.  Where n of them
+  // belong on an SM, each takes more than 1 / (n + 1) of its 227 KB: 11.5 -> 5 us a
+  // step after the update's end with 16 points of 3280 modes, 15 -> 8 with 64.
+  const int64_t n = ((int64_t)ctas * v.P + device_sms() - 1) / device_sms();
+  const size_t smem = SHARE <= 1 || BOTH ? need : std::max(need, 2 * most / (size_t)(n + 1));
+  const cudaError_t attr = allow_smem<solve_step_kernel<WS, HERM, BOTH, SHARE>>((int)(SHARE <= 1 || BOTH ? need : most));
   if (attr != cudaSuccess) return attr;
   return launch_after(solve_step_kernel<WS, HERM, BOTH, SHARE>, dim3(BOTH ? std::max(ctas, SOLVE_SPLIT * blocks) : ctas, v.P),
                       SOLVE_THREADS, smem, s, after, ctas, v, k, src, out);
