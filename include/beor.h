@@ -252,10 +252,12 @@ int beor_set_profiling(int on);
 
 /* Process-wide switch of the mixed-precision factorisation schedule (default
  * on).  On: look-ahead -- block step k's trailing update is split into the
- * next block column and the rest; the rest runs on a second, low-priority
- * stream while the diagonal block, slicing and panel of step k + 1 run at high
- * priority (the same blocked right-looking Cholesky, reordered as a task
- * graph: every tile sees the same operations, so the results are identical).
+ * next diagonal block, the tiles below it and the rest.  The tiles below it
+ * and then, at low priority, the rest run on a second stream beside the
+ * diagonal block of step k + 1, which starts as soon as its own tile is
+ * updated; that step's slicing and panel follow at high priority beside the
+ * rest (the same blocked right-looking Cholesky, reordered as a task graph:
+ * every tile sees the same operations, so the results are identical).
  * Off: one stream, steps in order.
  * Float64 contexts always use the in-order schedule. */
 int beor_set_lookahead(int on);

@@ -954,7 +954,9 @@ __global__ void __launch_bounds__(256, 2) resid_df_kernel(BatchView v) {
 
 // vec_r = dbar - Phi^-1 x - sum of the partial sums: groups of 16 block columns
 // added up from the left, the last group first if it is a shorter one, then
-// the others in order (the order in which concurrent groups would finish).
+// the others in order.  Any fixed order would do; this one is the order in which
+// the groups' atomic additions used to arrive, chosen so that the posterior
+// mean's bits stayed the same.
 __global__ void resid_sum_kernel(BatchView v) {
   const int p = blockIdx.y;
   const Prob pr = v.prob[p];
