@@ -603,7 +603,8 @@ int build_plan(beor_ctx* const* ctxs, int nsets, const int* Bs, bool need_x, int
   chk(cudaStreamSynchronize(nullptr));
   if (e != cudaSuccess) {
     delete pl;
-    return BEOR_ECUDA;
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? BEOR_ENOMEM : BEOR_ECUDA;
   }
   *out = pl;
   return BEOR_OK;

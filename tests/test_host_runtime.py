@@ -251,3 +251,19 @@ def test_no_evaluation_after_a_failed_precompute(fake):
             call()
     lk.precompute(STREAM)
     lk.lnl(np.zeros((1, 3)), stream=STREAM)
+
+
+@pytest.mark.parametrize("short", [1, 300, 1000, 3000, 100000, 1 << 22])
+def test_a_batch_that_does_not_fit_is_out_of_memory(fake, short):
+    """Whichever of its allocations fails, the tile lists' at the end among them; the
+    shape works once there is room."""
+    lk, p = _like(fake)
+    before = fake.fake_used(0)
+    lk.lnl(np.zeros((8, 3)), stream=STREAM)
+    batch = fake.fake_used(0) - before
+    lk, p = _like(fake)
+    fake.fake_set_total(0, fake.fake_used(0) + batch - short)
+    with pytest.raises(beor.BeorError, match="out of memory"):
+        lk.lnl(np.zeros((8, 3)), stream=STREAM)
+    fake.fake_set_total(0, 1 << 38)
+    lk.lnl(np.zeros((8, 3)), stream=STREAM)
